@@ -2,8 +2,10 @@
 
 Argument marshalling only: every function takes torch tensors (device memory and streams are
 PyTorch's job here), checks dtype / device / contiguity, and passes raw pointers and sizes to
-the function of the same name in ``libomni_mla.so``.  There is no Python or CPU fallback: if
-the library is missing or a call fails, an exception is raised.
+the function of the same name in ``libomni_mla.so``.  The calls of a decode step do this in native
+code (the CPython module ``_marshal``, csrc/marshal.cpp: about 1 us of host time instead of
+8-10), the others through ctypes.  There is no Python or CPU fallback: if the library is missing
+or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
@@ -62,6 +64,7 @@ class OmniError(RuntimeError):
 
 
 _lib = None
+_native = None
 
 
 def load() -> ctypes.CDLL:
@@ -124,6 +127,15 @@ def load() -> ctypes.CDLL:
     lib.omni_sparse_mla_set_profile_events.argtypes = [vp, vp]
     _lib = lib
     return lib
+
+
+def _load_native():
+    """The CPython module that marshals the per-step calls (built beside the library)."""
+    global _native
+    load()
+    from . import _marshal
+    _native = _marshal
+    return _native
 
 
 def omni_version() -> int:
@@ -196,42 +208,28 @@ def omni_sparse_mla_set_profile_events(before=None, after=None) -> None:
 
 def omni_sparse_mla_decode(desc, q, kv_cache, page_table, sel_idx, sel_len, out, lse,
                            workspace=None, device_status=None, stream=None) -> None:
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    code = load().omni_sparse_mla_decode(
-        ctypes.byref(desc), _ptr(q, torch.bfloat16, "cuda", "q"),
-        _ptr(kv_cache, torch.bfloat16, "cuda", "kv_cache"),
-        _ptr(page_table, torch.int32, "cuda", "page_table"),
-        _ptr(sel_idx, torch.int32, "cuda", "sel_idx"), _ptr(sel_len, torch.int32, "cuda", "sel_len"),
-        _ptr(out, torch.bfloat16, "cuda", "out"), _ptr(lse, torch.float32, "cuda", "lse"),
-        None if workspace is None else ctypes.c_void_p(workspace.data_ptr()), ws_bytes,
-        _ptr(device_status, torch.int32, "cuda", "device_status"), _stream(stream))
-    _check(code, "omni_sparse_mla_decode")
+    code = (_native or _load_native()).decode(desc, q, kv_cache, page_table, sel_idx, sel_len, out, lse, workspace,
+                                              device_status, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_sparse_mla_decode")
 
 
 def omni_sparse_mla_decode_sink_recent(desc, q, kv_cache, page_table, ctx_len, n_sink, n_recent, out, lse,
                                        workspace=None, device_status=None, stream=None) -> None:
     """Decode with Eq. 2's selection (attention sink + recent tokens) given as N_sink, N_recent and
     the context length of every request instead of an index list."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    code = load().omni_sparse_mla_decode_sink_recent(
-        ctypes.byref(desc), _ptr(q, torch.bfloat16, "cuda", "q"),
-        _ptr(kv_cache, torch.bfloat16, "cuda", "kv_cache"),
-        _ptr(page_table, torch.int32, "cuda", "page_table"),
-        _ptr(ctx_len, torch.int32, "cuda", "ctx_len"), int(n_sink), int(n_recent),
-        _ptr(out, torch.bfloat16, "cuda", "out"), _ptr(lse, torch.float32, "cuda", "lse"),
-        None if workspace is None else ctypes.c_void_p(workspace.data_ptr()), ws_bytes,
-        _ptr(device_status, torch.int32, "cuda", "device_status"), _stream(stream))
-    _check(code, "omni_sparse_mla_decode_sink_recent")
+    code = (_native or _load_native()).decode_sink_recent(desc, q, kv_cache, page_table, ctx_len, n_sink, n_recent, out,
+                                                          lse, workspace, device_status, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_sparse_mla_decode_sink_recent")
 
 
 def omni_topk_select(scores, ctx_len, k, sel_idx, sel_len, stream=None) -> None:
     """Positions of the k largest scores of every request, as sel_idx / sel_len for the decode call."""
     batch, stride = scores.shape
-    code = load().omni_topk_select(
-        _ptr(scores, torch.float32, "cuda", "scores"), _ptr(ctx_len, torch.int32, "cuda", "ctx_len"),
-        int(batch), int(stride), int(k), _ptr(sel_idx, torch.int32, "cuda", "sel_idx"),
-        _ptr(sel_len, torch.int32, "cuda", "sel_len"), _stream(stream))
-    _check(code, "omni_topk_select")
+    code = (_native or _load_native()).topk_select(scores, ctx_len, batch, stride, k, sel_idx, sel_len, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_topk_select")
 
 
 def omni_rolling_pages_per_request(n_sink: int, n_recent: int) -> int:
@@ -241,27 +239,19 @@ def omni_rolling_pages_per_request(n_sink: int, n_recent: int) -> int:
 def omni_kv_append_rolling(desc, kv_cache, page_table, ctx_len, new_rows, n_sink, n_recent,
                            device_status=None, stream=None) -> None:
     """Append one latent row per request to the rolling cache of a compressed layer."""
-    code = load().omni_kv_append_rolling(
-        ctypes.byref(desc), _ptr(kv_cache, torch.bfloat16, "cuda", "kv_cache"),
-        _ptr(page_table, torch.int32, "cuda", "page_table"), _ptr(ctx_len, torch.int32, "cuda", "ctx_len"),
-        _ptr(new_rows, torch.bfloat16, "cuda", "new_rows"), int(n_sink), int(n_recent),
-        _ptr(device_status, torch.int32, "cuda", "device_status"), _stream(stream))
-    _check(code, "omni_kv_append_rolling")
+    code = (_native or _load_native()).append_rolling(desc, kv_cache, page_table, ctx_len, new_rows, n_sink, n_recent,
+                                                      device_status, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_kv_append_rolling")
 
 
 def omni_sparse_mla_decode_rolling(desc, q, kv_cache, page_table, ctx_len, n_sink, n_recent, out, lse,
                                    workspace=None, device_status=None, stream=None) -> None:
     """Decode over the rolling cache of a compressed layer (Eq. 2's index set, any context length)."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    code = load().omni_sparse_mla_decode_rolling(
-        ctypes.byref(desc), _ptr(q, torch.bfloat16, "cuda", "q"),
-        _ptr(kv_cache, torch.bfloat16, "cuda", "kv_cache"),
-        _ptr(page_table, torch.int32, "cuda", "page_table"),
-        _ptr(ctx_len, torch.int32, "cuda", "ctx_len"), int(n_sink), int(n_recent),
-        _ptr(out, torch.bfloat16, "cuda", "out"), _ptr(lse, torch.float32, "cuda", "lse"),
-        None if workspace is None else ctypes.c_void_p(workspace.data_ptr()), ws_bytes,
-        _ptr(device_status, torch.int32, "cuda", "device_status"), _stream(stream))
-    _check(code, "omni_sparse_mla_decode_rolling")
+    code = (_native or _load_native()).decode_rolling(desc, q, kv_cache, page_table, ctx_len, n_sink, n_recent, out, lse,
+                                                      workspace, device_status, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_sparse_mla_decode_rolling")
 
 
 OMNI_Q8_ROW_BYTES = 640
@@ -269,25 +259,18 @@ OMNI_Q8_ROW_BYTES = 640
 
 def omni_kv_quantize_q8(kv_rows, kv_q8, kv_scale, stream=None) -> None:
     """bf16 rows [..., 576] -> 8-bit cache rows [..., 640] (uint8) and one fp32 scale per row."""
-    num_rows = kv_rows.numel() // 576
-    code = load().omni_kv_quantize_q8(
-        _ptr(kv_rows, torch.bfloat16, "cuda", "kv_rows"), int(num_rows), _ptr(kv_q8, torch.uint8, "cuda", "kv_q8"),
-        _ptr(kv_scale, torch.float32, "cuda", "kv_scale"), _stream(stream))
-    _check(code, "omni_kv_quantize_q8")
+    code = (_native or _load_native()).quantize_q8(kv_rows, kv_q8, kv_scale, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_kv_quantize_q8")
 
 
 def omni_sparse_mla_decode_q8(desc, q, kv_q8, kv_scale, page_table, sel_idx, sel_len, out, lse,
                               workspace=None, device_status=None, stream=None) -> None:
     """Decode over the 8-bit latent cache (see ``omni_kv_quantize_q8``)."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    code = load().omni_sparse_mla_decode_q8(
-        ctypes.byref(desc), _ptr(q, torch.bfloat16, "cuda", "q"), _ptr(kv_q8, torch.uint8, "cuda", "kv_q8"),
-        _ptr(kv_scale, torch.float32, "cuda", "kv_scale"), _ptr(page_table, torch.int32, "cuda", "page_table"),
-        _ptr(sel_idx, torch.int32, "cuda", "sel_idx"), _ptr(sel_len, torch.int32, "cuda", "sel_len"),
-        _ptr(out, torch.bfloat16, "cuda", "out"), _ptr(lse, torch.float32, "cuda", "lse"),
-        None if workspace is None else ctypes.c_void_p(workspace.data_ptr()), ws_bytes,
-        _ptr(device_status, torch.int32, "cuda", "device_status"), _stream(stream))
-    _check(code, "omni_sparse_mla_decode_q8")
+    code = (_native or _load_native()).decode_q8(desc, q, kv_q8, kv_scale, page_table, sel_idx, sel_len, out, lse,
+                                                 workspace, device_status, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_sparse_mla_decode_q8")
 
 
 OMNI_PLAN_BYTES = 1024
@@ -315,14 +298,10 @@ def omni_sparse_mla_plan_init(desc, q, kv_cache) -> LaunchPlan:
 
 def omni_sparse_mla_decode_planned(plan, page_table, sel_idx, sel_len, out, lse, workspace=None,
                                    device_status=None, stream=None) -> None:
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    code = load().omni_sparse_mla_decode_planned(
-        plan.ptr, _ptr(page_table, torch.int32, "cuda", "page_table"),
-        _ptr(sel_idx, torch.int32, "cuda", "sel_idx"), _ptr(sel_len, torch.int32, "cuda", "sel_len"),
-        _ptr(out, torch.bfloat16, "cuda", "out"), _ptr(lse, torch.float32, "cuda", "lse"),
-        None if workspace is None else ctypes.c_void_p(workspace.data_ptr()), ws_bytes,
-        _ptr(device_status, torch.int32, "cuda", "device_status"), _stream(stream))
-    _check(code, "omni_sparse_mla_decode_planned")
+    code = (_native or _load_native()).decode_planned(plan.address, page_table, sel_idx, sel_len, out, lse, workspace,
+                                                      device_status, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_sparse_mla_decode_planned")
 
 
 def bind_planned(plan, page_table, sel_idx, sel_len, out, lse, workspace=None, device_status=None, stream=None):
@@ -401,18 +380,10 @@ def omni_sparse_mla_resolve_rows(desc, page_table, sel_idx, sel_len, rows, strea
 def omni_sparse_mla_decode_host(desc, q_host, kv_cache, page_table_host, sel_idx_host,
                                 sel_len_host, out_host, lse_host, staging, workspace=None,
                                 device_status=None, stream=None) -> None:
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    code = load().omni_sparse_mla_decode_host(
-        ctypes.byref(desc), _ptr(q_host, torch.bfloat16, "cpu", "q_host"),
-        _ptr(kv_cache, torch.bfloat16, "cuda", "kv_cache"),
-        _ptr(page_table_host, torch.int32, "cpu", "page_table_host"),
-        _ptr(sel_idx_host, torch.int32, "cpu", "sel_idx_host"),
-        _ptr(sel_len_host, torch.int32, "cpu", "sel_len_host"),
-        _ptr(out_host, torch.bfloat16, "cpu", "out_host"), _ptr(lse_host, torch.float32, "cpu", "lse_host"),
-        ctypes.c_void_p(staging.data_ptr()), staging.numel() * staging.element_size(),
-        None if workspace is None else ctypes.c_void_p(workspace.data_ptr()), ws_bytes,
-        _ptr(device_status, torch.int32, "cuda", "device_status"), _stream(stream))
-    _check(code, "omni_sparse_mla_decode_host")
+    code = (_native or _load_native()).decode_host(desc, q_host, kv_cache, page_table_host, sel_idx_host, sel_len_host,
+                                                   out_host, lse_host, staging, workspace, device_status, stream)
+    if code != OMNI_OK:
+        raise OmniError(code, "omni_sparse_mla_decode_host")
 
 
 # ---------------------------------------------------------------------------------------

@@ -1,0 +1,306 @@
+// CPython side of binding.py: the per-step entry points with their argument marshalling in native
+// code.  One attention call from Python takes a dozen tensors; checking and unpacking them through
+// ctypes costs 8-10 us of host time, as much as the smallest decode step takes on the GPU, so a loop
+// of such steps was bound by it.  Here a tensor is one type check and four field reads, and a call
+// is a single C function behind binding.py's functions, which keep the names, defaults and checks.
+//
+// Every function takes its arguments by position, in the order of the binding.py function of the same
+// name with the last argument the stream (None: PyTorch's current one), and returns the status
+// code of the C function it calls.
+#include <Python.h>
+
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "omni_mla.h"
+
+namespace {
+
+struct Dtype {
+    at::ScalarType type;
+    const char *name;
+};
+constexpr Dtype kBf16 = {at::kBFloat16, "torch.bfloat16"}, kF32 = {at::kFloat, "torch.float32"},
+                kI32 = {at::kInt, "torch.int32"}, kU8 = {at::kByte, "torch.uint8"};
+
+// A call's arguments, taken one after the other.  The first failure sets a Python exception and
+// `bad`; everything taken after it is null.
+class Args {
+public:
+    Args(const char *fn, PyObject *const *args, Py_ssize_t n, Py_ssize_t want) : args_(args)
+    {
+        if (n != want) {
+            PyErr_Format(PyExc_TypeError, "%s takes %zd arguments, got %zd", fn, want, n);
+            bad = true;
+        }
+    }
+    ~Args()
+    {
+        if (has_view_) PyBuffer_Release(&view_);
+    }
+
+    const omni_mla_desc_t *desc()
+    {
+        PyObject *o = next();
+        if (bad) return nullptr;
+        if (PyObject_GetBuffer(o, &view_, PyBUF_SIMPLE) != 0) {
+            bad = true;
+            return nullptr;
+        }
+        has_view_ = true;
+        if (view_.len != (Py_ssize_t)sizeof(omni_mla_desc_t)) {
+            PyErr_SetString(PyExc_TypeError, "desc must be an OmniDesc");
+            bad = true;
+            return nullptr;
+        }
+        return static_cast<const omni_mla_desc_t *>(view_.buf);
+    }
+
+    // Tensor of one dtype, device kind and contiguity, or None (a null pointer).
+    template <class T>
+    T *tensor(const Dtype &dtype, const char *name, bool cuda = true)
+    {
+        PyObject *o = next();
+        if (bad || o == Py_None) return nullptr;
+        if (!THPVariable_Check(o)) {
+            PyErr_Format(PyExc_TypeError, "%s must be a tensor", name);
+            bad = true;
+            return nullptr;
+        }
+        const at::Tensor &t = THPVariable_Unpack(o);
+        if (t.scalar_type() != dtype.type) {
+            PyObject *got = PyObject_GetAttrString(o, "dtype");
+            PyErr_Format(PyExc_TypeError, "%s must be %s, got %S", name, dtype.name, got ? got : Py_None);
+            Py_XDECREF(got);
+            bad = true;
+        } else if (cuda ? !t.is_cuda() : !t.is_cpu()) {
+            PyErr_Format(PyExc_ValueError, "%s must live on %s", name, cuda ? "cuda" : "cpu");
+            bad = true;
+        } else if (!t.is_contiguous()) {
+            PyErr_Format(PyExc_ValueError, "%s must be contiguous", name);
+            bad = true;
+        }
+        return bad ? nullptr : static_cast<T *>(t.data_ptr());
+    }
+
+    // Raw storage of any dtype (workspace, staging), or None.
+    void *buffer(const char *name, size_t *bytes)
+    {
+        *bytes = 0;
+        PyObject *o = next();
+        if (bad || o == Py_None) return nullptr;
+        if (!THPVariable_Check(o)) {
+            PyErr_Format(PyExc_TypeError, "%s must be a tensor", name);
+            bad = true;
+            return nullptr;
+        }
+        const at::Tensor &t = THPVariable_Unpack(o);
+        *bytes = (size_t)t.numel() * t.element_size();
+        return t.data_ptr();
+    }
+
+    int64_t elements()                                    // of the argument taken next (it is not consumed)
+    {
+        PyObject *o = args_[at_];
+        return !bad && THPVariable_Check(o) ? THPVariable_Unpack(o).numel() : 0;
+    }
+
+    int64_t integer()
+    {
+        PyObject *o = next();
+        if (bad) return 0;
+        PyObject *whole = PyNumber_Long(o);                // as int() does
+        const long long v = whole ? PyLong_AsLongLong(whole) : -1;
+        Py_XDECREF(whole);
+        if (v == -1 && PyErr_Occurred()) bad = true;
+        return v;
+    }
+
+    int32_t int32()
+    {
+        return (int32_t)integer();
+    }
+
+    void *stream()
+    {
+        PyObject *o = next();
+        if (bad) return nullptr;
+        if (o == Py_None) {
+            try {
+                return c10::cuda::getCurrentCUDAStream().stream();
+            } catch (const std::exception &e) {
+                PyErr_SetString(PyExc_RuntimeError, e.what());
+                bad = true;
+                return nullptr;
+            }
+        }
+        PyObject *handle = PyObject_GetAttrString(o, "cuda_stream");
+        void *s = handle ? PyLong_AsVoidPtr(handle) : nullptr;
+        Py_XDECREF(handle);
+        if (PyErr_Occurred()) bad = true;
+        return s;
+    }
+
+    bool bad = false;
+
+private:
+    PyObject *next() { return bad ? nullptr : args_[at_++]; }
+
+    PyObject *const *args_;
+    Py_ssize_t at_ = 0;
+    Py_buffer view_;
+    bool has_view_ = false;
+};
+
+// A launch can block for as long as the stream's queue is full: other Python threads run meanwhile.
+template <class Call>
+PyObject *finish(const Args &a, Call &&call)
+{
+    if (a.bad) return nullptr;
+    omni_status_t st;
+    Py_BEGIN_ALLOW_THREADS;
+    st = call();
+    Py_END_ALLOW_THREADS;
+    return PyLong_FromLong((long)st);
+}
+
+}  // namespace
+
+static PyObject *decode(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    Args a("decode", args, n, 11);
+    const omni_mla_desc_t *desc = a.desc();
+    const void *q = a.tensor<void>(kBf16, "q"), *kv = a.tensor<void>(kBf16, "kv_cache");
+    const int32_t *table = a.tensor<int32_t>(kI32, "page_table"), *idx = a.tensor<int32_t>(kI32, "sel_idx"),
+                  *len = a.tensor<int32_t>(kI32, "sel_len");
+    void *out = a.tensor<void>(kBf16, "out");
+    float *lse = a.tensor<float>(kF32, "lse");
+    size_t ws_bytes;
+    void *ws = a.buffer("workspace", &ws_bytes);
+    int32_t *status = a.tensor<int32_t>(kI32, "device_status");
+    void *stream = a.stream();
+    return finish(a, [&] { return omni_sparse_mla_decode(desc, q, kv, table, idx, len, out, lse, ws, ws_bytes, status, stream); });
+}
+
+static PyObject *decode_planned(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    Args a("decode_planned", args, n, 9);
+    const omni_mla_plan_t *plan = reinterpret_cast<const omni_mla_plan_t *>(a.integer());
+    const int32_t *table = a.tensor<int32_t>(kI32, "page_table"), *idx = a.tensor<int32_t>(kI32, "sel_idx"),
+                  *len = a.tensor<int32_t>(kI32, "sel_len");
+    void *out = a.tensor<void>(kBf16, "out");
+    float *lse = a.tensor<float>(kF32, "lse");
+    size_t ws_bytes;
+    void *ws = a.buffer("workspace", &ws_bytes);
+    int32_t *status = a.tensor<int32_t>(kI32, "device_status");
+    void *stream = a.stream();
+    return finish(a, [&] { return omni_sparse_mla_decode_planned(plan, table, idx, len, out, lse, ws, ws_bytes, status, stream); });
+}
+
+// decode_sink_recent and decode_rolling: the same arguments
+template <class Fn>
+static PyObject *decode_ranges(Fn fn, const char *name, PyObject *const *args, Py_ssize_t n)
+{
+    Args a(name, args, n, 12);
+    const omni_mla_desc_t *desc = a.desc();
+    const void *q = a.tensor<void>(kBf16, "q"), *kv = a.tensor<void>(kBf16, "kv_cache");
+    const int32_t *table = a.tensor<int32_t>(kI32, "page_table"), *ctx = a.tensor<int32_t>(kI32, "ctx_len");
+    const int32_t n_sink = a.int32(), n_recent = a.int32();
+    void *out = a.tensor<void>(kBf16, "out");
+    float *lse = a.tensor<float>(kF32, "lse");
+    size_t ws_bytes;
+    void *ws = a.buffer("workspace", &ws_bytes);
+    int32_t *status = a.tensor<int32_t>(kI32, "device_status");
+    void *stream = a.stream();
+    return finish(a, [&] { return fn(desc, q, kv, table, ctx, n_sink, n_recent, out, lse, ws, ws_bytes, status, stream); });
+}
+
+static PyObject *decode_sink_recent(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    return decode_ranges(omni_sparse_mla_decode_sink_recent, "decode_sink_recent", args, n);
+}
+
+static PyObject *decode_rolling(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    return decode_ranges(omni_sparse_mla_decode_rolling, "decode_rolling", args, n);
+}
+
+static PyObject *append_rolling(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    Args a("append_rolling", args, n, 9);
+    const omni_mla_desc_t *desc = a.desc();
+    void *kv = a.tensor<void>(kBf16, "kv_cache");
+    const int32_t *table = a.tensor<int32_t>(kI32, "page_table"), *ctx = a.tensor<int32_t>(kI32, "ctx_len");
+    const void *rows = a.tensor<void>(kBf16, "new_rows");
+    const int32_t n_sink = a.int32(), n_recent = a.int32();
+    int32_t *status = a.tensor<int32_t>(kI32, "device_status");
+    void *stream = a.stream();
+    return finish(a, [&] { return omni_kv_append_rolling(desc, kv, table, ctx, rows, n_sink, n_recent, status, stream); });
+}
+
+static PyObject *decode_q8(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    Args a("decode_q8", args, n, 12);
+    const omni_mla_desc_t *desc = a.desc();
+    const void *q = a.tensor<void>(kBf16, "q"), *kv = a.tensor<void>(kU8, "kv_q8");
+    const float *scale = a.tensor<float>(kF32, "kv_scale");
+    const int32_t *table = a.tensor<int32_t>(kI32, "page_table"), *idx = a.tensor<int32_t>(kI32, "sel_idx"),
+                  *len = a.tensor<int32_t>(kI32, "sel_len");
+    void *out = a.tensor<void>(kBf16, "out");
+    float *lse = a.tensor<float>(kF32, "lse");
+    size_t ws_bytes;
+    void *ws = a.buffer("workspace", &ws_bytes);
+    int32_t *status = a.tensor<int32_t>(kI32, "device_status");
+    void *stream = a.stream();
+    return finish(a, [&] { return omni_sparse_mla_decode_q8(desc, q, kv, scale, table, idx, len, out, lse, ws, ws_bytes, status, stream); });
+}
+
+static PyObject *quantize_q8(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    Args a("quantize_q8", args, n, 4);
+    const int64_t rows = a.elements() / 576;
+    const void *kv = a.tensor<void>(kBf16, "kv_rows");
+    void *codes = a.tensor<void>(kU8, "kv_q8");
+    float *scale = a.tensor<float>(kF32, "kv_scale");
+    void *stream = a.stream();
+    return finish(a, [&] { return omni_kv_quantize_q8(kv, rows, codes, scale, stream); });
+}
+
+static PyObject *topk_select(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    Args a("topk_select", args, n, 8);
+    const float *scores = a.tensor<float>(kF32, "scores");
+    const int32_t *ctx = a.tensor<int32_t>(kI32, "ctx_len");
+    const int32_t batch = a.int32(), stride = a.int32(), k = a.int32();
+    int32_t *idx = a.tensor<int32_t>(kI32, "sel_idx"), *len = a.tensor<int32_t>(kI32, "sel_len");
+    void *stream = a.stream();
+    return finish(a, [&] { return omni_topk_select(scores, ctx, batch, stride, k, idx, len, stream); });
+}
+
+static PyObject *decode_host(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    Args a("decode_host", args, n, 12);
+    const omni_mla_desc_t *desc = a.desc();
+    const void *q = a.tensor<void>(kBf16, "q_host", false), *kv = a.tensor<void>(kBf16, "kv_cache");
+    const int32_t *table = a.tensor<int32_t>(kI32, "page_table_host", false),
+                  *idx = a.tensor<int32_t>(kI32, "sel_idx_host", false), *len = a.tensor<int32_t>(kI32, "sel_len_host", false);
+    void *out = a.tensor<void>(kBf16, "out_host", false);
+    float *lse = a.tensor<float>(kF32, "lse_host", false);
+    size_t staging_bytes, ws_bytes;
+    void *staging = a.buffer("staging", &staging_bytes), *ws = a.buffer("workspace", &ws_bytes);
+    int32_t *status = a.tensor<int32_t>(kI32, "device_status");
+    void *stream = a.stream();
+    return finish(a, [&] {
+        return omni_sparse_mla_decode_host(desc, q, kv, table, idx, len, out, lse, staging, staging_bytes, ws, ws_bytes, status, stream);
+    });
+}
+
+#define OMNI_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
+static PyMethodDef methods[] = {
+    OMNI_METHOD(decode),         OMNI_METHOD(decode_planned), OMNI_METHOD(decode_sink_recent), OMNI_METHOD(decode_rolling),
+    OMNI_METHOD(append_rolling), OMNI_METHOD(decode_q8),      OMNI_METHOD(quantize_q8),        OMNI_METHOD(topk_select),
+    OMNI_METHOD(decode_host),    {nullptr, nullptr, 0, nullptr}};
+static PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", "native argument marshalling of binding.py", -1, methods,
+                             nullptr, nullptr, nullptr, nullptr};
+
+PyMODINIT_FUNC PyInit__marshal(void) { return PyModule_Create(&module); }
