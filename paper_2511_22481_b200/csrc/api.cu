@@ -154,6 +154,24 @@ bool merge_in_kernel(const omni_mla_desc_t *d)
     return use_pair_kernel(d) && (d->flags & OMNI_FLAG_FUSED_MERGE);
 }
 
+// Launch whose blocks may become resident while the kernel in front of it in the stream still runs
+// (programmatic dependent launch); the kernel itself waits (griddepcontrol.wait) before it touches
+// global memory, so only the launch gap between the two kernels goes away.
+template <class... KernelArgs, class... CallArgs>
+omni_status_t launch_overlapped(void (*kernel)(KernelArgs...), unsigned blocks, unsigned threads, cudaStream_t stream, CallArgs... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KernelArgs(args)...) == cudaSuccess ? OMNI_OK : OMNI_ERR_CUDA;
+}
+
 omni_status_t launch_combine(int batch, int heads, int max_splits, const float *part_out,
                              const float *part_lse, const int32_t *num_splits, void *out,
                              float *lse, cudaStream_t stream)
@@ -165,22 +183,8 @@ omni_status_t launch_combine(int batch, int heads, int max_splits, const float *
         cudaFuncSetAttribute(combine_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         carveout_set = true;
     }
-    // Programmatic dependent launch: the merge blocks may become resident while the decode kernel
-    // is still running and wait (griddepcontrol.wait) until it has completed and its writes are
-    // visible, which removes most of the launch gap between the two kernels.
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(batch * heads));
-    cfg.blockDim = dim3(128);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, combine_kernel, part_out, part_lse, num_splits, max_splits, heads,
-                              static_cast<__nv_bfloat16 *>(out), lse) == cudaSuccess
-               ? OMNI_OK
-               : OMNI_ERR_CUDA;
+    return launch_overlapped(combine_kernel, (unsigned)(batch * heads), 128, stream, part_out, part_lse, num_splits, max_splits,
+                             heads, static_cast<__nv_bfloat16 *>(out), lse);
 }
 
 omni_status_t launch_resolve(const omni_mla_desc_t *d, const int32_t *page_table,
@@ -494,10 +498,10 @@ omni_status_t omni_kv_quantize_q8(const void *kv_rows, int64_t num_rows, void *k
     if (!kv_rows || !kv_q8 || !kv_scale) return OMNI_ERR_NULL;
     if (num_rows < 1 || num_rows > (int64_t)0x7fffffff * 8) return OMNI_ERR_SHAPE;
     if (!aligned(kv_rows, 16) || !aligned(kv_q8, 128) || !aligned(kv_scale, 4)) return OMNI_ERR_ALIGN;
-    const unsigned blocks = (unsigned)((num_rows + 7) / 8);
-    quantize_q8_kernel<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16 *>(kv_rows), num_rows, static_cast<uint8_t *>(kv_q8), kv_scale);
-    return cudaPeekAtLastError() == cudaSuccess ? OMNI_OK : OMNI_ERR_CUDA;
+    constexpr int kRowsPerBlock = kQ8QuantWarps * kQ8RowsPerWarp;
+    return launch_overlapped(quantize_q8_kernel, (unsigned)((num_rows + kRowsPerBlock - 1) / kRowsPerBlock), kQ8QuantWarps * 32,
+                             static_cast<cudaStream_t>(stream), static_cast<const __nv_bfloat16 *>(kv_rows), num_rows,
+                             static_cast<uint8_t *>(kv_q8), kv_scale);
 }
 
 omni_status_t omni_sparse_mla_plan_init(const omni_mla_desc_t *desc, const void *q, const void *kv_cache,
