@@ -178,13 +178,18 @@ omni_status_t launch_combine(int batch, int heads, int max_splits, const float *
 {
     // Keep the shared-memory / L1 split the decode kernel needs: alternating between two splits
     // makes every launch wait for the SMs to be reconfigured.
-    static bool carveout_set = false;
-    if (!carveout_set) {
-        cudaFuncSetAttribute(combine_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        carveout_set = true;
-    }
-    return launch_overlapped(combine_kernel, (unsigned)(batch * heads), 128, stream, part_out, part_lse, num_splits, max_splits,
-                             heads, static_cast<__nv_bfloat16 *>(out), lse);
+    static const bool carveout_set = [] {
+        cudaFuncSetAttribute(combine_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        cudaFuncSetAttribute(combine_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        return true;
+    }();
+    (void)carveout_set;
+    // Four thread groups per block while all blocks fit the SMs at once (three of 512 threads per SM)
+    // and there are more splits than one thread keeps in flight.
+    const int blocks = batch * heads;
+    const bool wide = max_splits > kCombineAhead && blocks <= 3 * device_info().sm_count;
+    return launch_overlapped(wide ? combine_kernel<4> : combine_kernel<1>, (unsigned)blocks, wide ? 512 : 128, stream, part_out,
+                             part_lse, num_splits, max_splits, heads, static_cast<__nv_bfloat16 *>(out), lse);
 }
 
 omni_status_t launch_resolve(const omni_mla_desc_t *d, const int32_t *page_table,

@@ -5,49 +5,96 @@
 
 namespace omni {
 
-// One block per (request, head); thread t owns value columns 4t..4t+3.
-// lse = ln sum_s exp(lse_s); out = sum_s exp(lse_s - lse) * out_s.
-__global__ void __launch_bounds__(128) combine_kernel(const float *__restrict__ part_out,
-                                                      const float *__restrict__ part_lse,
-                                                      const int32_t *__restrict__ num_splits,
-                                                      int max_splits, int heads,
-                                                      __nv_bfloat16 *__restrict__ out,
-                                                      float *__restrict__ lse)
+// One block per (request, head): lse = ln sum_s exp(lse_s); out = sum_s exp(lse_s - lse) * out_s.
+// 128 * kGroups threads: thread t owns value columns 4 (t % 128) .. + 3 of the splits t / 128,
+// t / 128 + kGroups, ...; the partial sums of a column meet in shared memory.  The kernel is a chain of
+// latencies, not of bytes (the partials sit in L2): first every log-sum-exp at once (a lane per
+// split in every warp), then the partial rows, kCombineAhead loads of a thread in flight.  With one thread
+// per column walking the splits one after the other, 32 splits of one request took 11 us; now about 3.
+// Four groups pay where a launch has few blocks and many splits; with more blocks than the
+// SMs hold at once the larger blocks only make more waves (64 requests of 64 heads, two splits: 80 us
+// per step with four groups, 66 with one), see launch_combine.
+constexpr int kCombineAhead = 4;
+template <int kGroups>
+__global__ void __launch_bounds__(128 * kGroups) combine_kernel(const float *__restrict__ part_out,
+                                                                const float *__restrict__ part_lse,
+                                                                const int32_t *__restrict__ num_splits,
+                                                                int max_splits, int heads,
+                                                                __nv_bfloat16 *__restrict__ out,
+                                                                float *__restrict__ lse)
 {
+    __shared__ float4 sums[kGroups > 1 ? kGroups - 1 : 1][128];
+    const int b = blockIdx.x / heads, h = blockIdx.x % heads;
+    const int lane = threadIdx.x & 31, col = threadIdx.x & 127, group = threadIdx.x >> 7;
+    const float4 *rows = reinterpret_cast<const float4 *>(part_out + ((size_t)b * max_splits * heads + h) * kDv) + col;
+    const size_t row_pitch = (size_t)heads * (kDv / 4);
+    const float *pl = part_lse + (size_t)b * max_splits * heads + h;
     // no-op unless launched as a programmatic dependent: then wait for the producing kernel;
     // the kernel that follows may be scheduled early in turn (it waits before it reads)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int b = blockIdx.x / heads, h = blockIdx.x % heads;
     int ns = num_splits ? __ldg(num_splits + b) : max_splits;
     ns = max(0, min(ns, max_splits));
-    const float *pl = part_lse + (size_t)b * max_splits * heads + h;
-    float mx = -INFINITY;
-    for (int s = 0; s < ns; ++s) mx = fmaxf(mx, __ldg(pl + (size_t)s * heads));
+    // total over all splits, 32 at a time: every warp does it for itself
+    float mx = -INFINITY, z = 0.f, first = -INFINITY;      // z: sum of exp(lse - mx)
+    for (int s0 = 0; s0 < ns; s0 += 32) {
+        const float v = s0 + lane < ns ? __ldg(pl + (size_t)(s0 + lane) * heads) : -INFINITY;
+        if (s0 == 0) first = v;
+        float m = v;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
+        m = fmaxf(m, mx);
+        if (m == -INFINITY) continue;
+        float e = exp2f((v - m) * kLog2e);
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) e += __shfl_xor_sync(0xffffffffu, e, d);
+        z = (mx == -INFINITY ? 0.f : z * exp2f((mx - m) * kLog2e)) + e;
+        mx = m;
+    }
+    const float total = mx > -INFINITY ? mx + logf(z) : -INFINITY;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    float total = -INFINITY;
-    if (mx > -INFINITY) {
-        float z = 0.f;
-        for (int s = 0; s < ns; ++s) z += exp2f((__ldg(pl + (size_t)s * heads) - mx) * kLog2e);
-        total = mx + logf(z);
-        for (int s = 0; s < ns; ++s) {
-            const float ls = __ldg(pl + (size_t)s * heads);
-            if (ls == -INFINITY) continue;
-            const float w = exp2f((ls - total) * kLog2e);
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(
-                                       part_out + (((size_t)b * max_splits + s) * heads + h) * kDv) +
-                                   threadIdx.x);
-            acc.x = fmaf(w, v.x, acc.x);
-            acc.y = fmaf(w, v.y, acc.y);
-            acc.z = fmaf(w, v.z, acc.z);
-            acc.w = fmaf(w, v.w, acc.w);
+    for (int s0 = 0; s0 < ns; s0 += 32) {
+        const float v = s0 == 0 ? first : (s0 + lane < ns ? __ldg(pl + (size_t)(s0 + lane) * heads) : -INFINITY);
+        const float weight = v > -INFINITY ? exp2f((v - total) * kLog2e) : 0.f;      // of split s0 + lane
+        const int here = min(32, ns - s0);
+        for (int i0 = group; i0 < here; i0 += kGroups * kCombineAhead) {
+            float4 x[kCombineAhead];
+            float w[kCombineAhead];
+#pragma unroll
+            for (int k = 0; k < kCombineAhead; ++k) {
+                const int i = i0 + k * kGroups;
+                w[k] = __shfl_sync(0xffffffffu, weight, i & 31);
+                if (i >= here) w[k] = 0.f;
+                // the row of an empty split is not read: it may hold anything
+                x[k] = w[k] != 0.f ? __ldg(rows + (size_t)(s0 + i) * row_pitch) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < kCombineAhead; ++k) {
+                acc.x = fmaf(w[k], x[k].x, acc.x);
+                acc.y = fmaf(w[k], x[k].y, acc.y);
+                acc.z = fmaf(w[k], x[k].z, acc.z);
+                acc.w = fmaf(w[k], x[k].w, acc.w);
+            }
+        }
+    }
+    if (kGroups > 1) {
+        if (group > 0) sums[group - 1][col] = acc;
+        __syncthreads();
+        if (group > 0) return;
+#pragma unroll
+        for (int g = 0; g < kGroups - 1; ++g) {
+            const float4 x = sums[g][col];
+            acc.x += x.x;
+            acc.y += x.y;
+            acc.z += x.z;
+            acc.w += x.w;
         }
     }
     __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
     uint2 packed;
     packed.x = *reinterpret_cast<uint32_t *>(&lo);
     packed.y = *reinterpret_cast<uint32_t *>(&hi);
-    reinterpret_cast<uint2 *>(out + ((size_t)b * heads + h) * kDv)[threadIdx.x] = packed;
+    reinterpret_cast<uint2 *>(out + ((size_t)b * heads + h) * kDv)[col] = packed;
     if (threadIdx.x == 0) lse[(size_t)b * heads + h] = total;
 }
 
