@@ -65,16 +65,31 @@ int64_t rolling_ring_pages(int32_t n_recent) { return ((int64_t)n_recent + kPage
 
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
-// More than 64 heads run on the paired-CTA kernel (one cluster of two CTAs per work unit).
-bool use_pair_kernel(const omni_mla_desc_t *d) { return !(d->flags & OMNI_FLAG_SIMT) && d->num_heads > kTcHeads; }
+// Which tensor-core kernel serves a problem: the paired-CTA one (a cluster of two CTAs per work unit)
+// unless there are few heads and little to read.  Up to 64 heads fill only one CTA of a pair, but the
+// other still carries half of every tile's loads and holds half of its operands, and an M = 128 pair runs the
+// tensor pipe at full rate where the single CTA's M = 64 runs it at half rate, with 2 tiles of
+// buffers to the pair's 4: 64 requests x 33 tiles 42 us against 64 with 64 heads, 41 against 58
+// with 16; one request of 128 tiles 17 against 24 and 15.6 against 18.7.  What the single-CTA kernel has is the
+// shorter start and end and twice as many work units, which shows up to 32 heads while two tiles per
+// unit spread over all SMs in one wave (4 requests x 33 tiles of 16 heads: 13.0 against 15.1 us).
+constexpr int kSingleCtaHeads = 32, kSingleCtaUnits = 148;
+bool use_pair_kernel(const omni_mla_desc_t *d)
+{
+    if (d->flags & OMNI_FLAG_SIMT) return false;
+    const int tiles = (d->max_sel + kTile - 1) / kTile;
+    return d->num_heads > kSingleCtaHeads || (long)d->batch * ((tiles + 1) / 2) > kSingleCtaUnits;
+}
+
+// The 8-bit kernel takes more than 64 heads (both CTAs of its pairs have some).
+bool q8_shape_ok(const omni_mla_desc_t *d) { return !(d->flags & OMNI_FLAG_SIMT) && d->num_heads > kTcHeads; }
 
 // Work units one split of one request occupies in the kernel that will run.
 int units_per_request(const omni_mla_desc_t *d)
 {
     if (d->flags & OMNI_FLAG_SIMT)
         return (d->num_heads + kSimtWarps * kSimtHeadsPerWarp - 1) / (kSimtWarps * kSimtHeadsPerWarp);
-    if (use_pair_kernel(d)) return 1;
-    return (d->num_heads + kTcHeads - 1) / kTcHeads;
+    return 1;
 }
 
 // Two splits of a request can be merged inside a cluster of two CTA pairs as long as all those
@@ -93,7 +108,8 @@ bool merge_in_cluster(const omni_mla_desc_t *d, int splits, int resident_merge_c
 // results to global memory for a later merge costs about 6 more when the grid runs in several
 // waves (256 KiB written and read back against 72 KiB per tile; about 2 within one wave, where
 // they stay in L2), and so does the merge kernel at the end.  Two splits merged inside a
-// cluster of two CTA pairs avoid the partial results and pay about 5 for the exchange.
+// cluster of two CTA pairs avoid the partial results and pay about 5 for the exchange.  A tile of the
+// single-CTA kernel takes twice as long, and the merge of its few heads about 4.
 // Minimise waves * (granules per unit + fixed parts) + merge.
 int choose_splits(const omni_mla_desc_t *d, int sm_count, int resident_merge_clusters = -1)
 {
@@ -103,6 +119,7 @@ int choose_splits(const omni_mla_desc_t *d, int sm_count, int resident_merge_clu
     const int granules = (d->max_sel + granule - 1) / granule;
     const long units = (long)d->batch * units_per_request(d);
     if (use_pair_kernel(d)) sm_count /= 2;               // a work unit occupies two SMs
+    const bool single = !use_pair_kernel(d) && !(d->flags & OMNI_FLAG_SIMT);
     long best_cost = -1;
     int best = 1;
     for (int s = 1; s <= kMaxSplits && s <= granules; ++s) {
@@ -110,9 +127,11 @@ int choose_splits(const omni_mla_desc_t *d, int sm_count, int resident_merge_clu
         const long per = (granules + s - 1) / s;
         long cost;
         if (s == 1)
-            cost = waves * (per + 6);
+            cost = waves * ((single ? 2 * per : per) + 6);
         else if (merge_in_cluster(d, s, resident_merge_clusters))
             cost = waves * (per + 6) + 5;
+        else if (single)
+            cost = waves * (2 * per + 6 + (waves > 1 ? 6 : 2)) + 4;
         else
             cost = waves * (per + 6 + (waves > 1 ? 6 : 2)) + 6;     // partial results stay in L2 within one wave
         if (best_cost < 0 || cost < best_cost) {
@@ -135,10 +154,10 @@ size_t part_lse_bytes(const omni_mla_desc_t *d, int splits)
     return align_up((size_t)d->batch * splits * d->num_heads * sizeof(float), 256);
 }
 
-// Arrival counters of the in-kernel merge: one per (request, head group of 64).
+// Arrival counters of the in-kernel merge: one per (request, CTA of a pair).
 size_t counter_bytes(const omni_mla_desc_t *d)
 {
-    return align_up((size_t)d->batch * ((d->num_heads + kTcHeads - 1) / kTcHeads) * sizeof(int32_t), 256);
+    return align_up((size_t)d->batch * 2 * sizeof(int32_t), 256);
 }
 
 size_t workspace_need(const omni_mla_desc_t *d, int splits)
@@ -317,8 +336,7 @@ static omni_status_t build_plan(const omni_mla_desc_t *desc, const void *q, cons
 {
     if (!desc || !q || !kv_cache || (q8 && !kv_scale)) return OMNI_ERR_NULL;
     if (!desc_ok(desc)) return OMNI_ERR_SHAPE;
-    // the 8-bit path exists for the paired-CTA kernel only (more than 64 heads, tensor cores)
-    if (q8 && !use_pair_kernel(desc)) return OMNI_ERR_SHAPE;
+    if (q8 && !q8_shape_ok(desc)) return OMNI_ERR_SHAPE;
     if (!aligned(q, 16) || !aligned(kv_cache, 128) || !aligned(kv_scale, 4)) return OMNI_ERR_ALIGN;
     const DeviceInfo &dev = device_info();
     if (!dev.ok) return OMNI_ERR_CUDA;
@@ -487,7 +505,7 @@ omni_status_t omni_sparse_mla_decode_q8(const omni_mla_desc_t *desc, const void 
                                         size_t workspace_bytes, int32_t *device_status, void *stream)
 {
     if (!desc || !q || !kv_q8 || !kv_scale || !page_table || !sel_idx || !sel_len || !out || !lse) return OMNI_ERR_NULL;
-    if (!desc_ok(desc) || !use_pair_kernel(desc)) return OMNI_ERR_SHAPE;
+    if (!desc_ok(desc) || !q8_shape_ok(desc)) return OMNI_ERR_SHAPE;
     omni_status_t st = check_step_args(desc, page_table, sel_idx, sel_len, nullptr, 0, 0, false, out, lse);
     if (st == OMNI_OK && (!aligned(q, 16) || !aligned(kv_q8, 128) || !aligned(kv_scale, 4))) st = OMNI_ERR_ALIGN;
     if (st != OMNI_OK) return st;

@@ -1,4 +1,4 @@
-// Paired-CTA tensor-core decode kernel for sm_100a (the fast path for more than 64 heads).
+// Paired-CTA tensor-core decode kernel for sm_100a (every problem but the smallest with few heads).
 //
 // A cluster of two CTAs owns all heads of one (request, split): CTA r serves heads
 // [64r, 64r+64).  The pair issues cta_group::2 MMAs with M = 128 (64 rows per CTA), which run
@@ -706,7 +706,8 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         const uint32_t q_bar = map_to_rank(smem_u32(&ctl->q_full), leader);
         if (lane == 0) {
             if (rank == 0) mbar_expect_tx(&ctl->q_full, 2 * kTileBytes);
-            tma_box3d_pair(smem_base + kC2SmemQ, &q_map, q_bar, b * p.heads + h0, 0);
+            // a CTA without heads (64 or fewer in all) takes zeros: the box starts past the last row
+            tma_box3d_pair(smem_base + kC2SmemQ, &q_map, q_bar, head_rows > 0 ? b * p.heads + h0 : p.batch * p.heads, 0);
         }
         bool any_bad = bad_len;
         TileIdx x1, x2;                      // one and two tiles ahead

@@ -1,7 +1,7 @@
-// Tensor-core decode kernel for sm_100a: TMA row gather through the page table, tcgen05 MMAs
+// Single-CTA tensor-core decode kernel for sm_100a (few heads and little to read): TMA row gather through the page table, tcgen05 MMAs
 // with fp32 accumulators in tensor memory, fp32 online softmax.
 //
-// One CTA owns 64 heads of one (request, split) and walks the split's selected tokens in
+// One CTA owns all heads (up to 64) of one (request, split) and walks the split's selected tokens in
 // 64-token tiles:
 //   warp 0      producer: resolves token positions to pool rows and brings the rows into a
 //               2-stage ring of 128B-swizzled tiles with TMA: one 64x64 box per column panel
@@ -312,12 +312,8 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
     TcControl *ctl = reinterpret_cast<TcControl *>(smem + kSmemCtl);
     const uint32_t smem_base = smem_u32(smem);
 
-    const int head_groups = (p.heads + kTcHeads - 1) / kTcHeads;
-    const int hg = blockIdx.x % head_groups;
-    const int s = (blockIdx.x / head_groups) % p.splits;
-    const int b = blockIdx.x / (head_groups * p.splits);
+    const int s = blockIdx.x % p.splits, b = blockIdx.x / p.splits;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform
-    const int h0 = hg * kTcHeads;
 
     // Programmatic dependent launch, both ways: nothing in global memory is touched until the
     // kernel before this one in the stream has completed, and the kernel after this one (the split
@@ -335,7 +331,7 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
         // empty split: zero output / -inf log-sum-exp, no tensor-core work
         if (threadIdx.x == 0 && bad_len) flag_status(p.status, OMNI_DEV_BAD_INDEX);
         for (int r = warp; r < kTcHeads; r += kTcThreads / 32) {
-            const int h = h0 + r;
+            const int h = r;
             if (h >= p.heads) break;
             if (p.splits == 1) {
                 uint4 *o = reinterpret_cast<uint4 *>(p.out + ((size_t)b * p.heads + h) * kDv);
@@ -384,7 +380,7 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
         const int32_t *pt = p.page_table + (size_t)b * p.max_pages;
         if (lane == 0) {
             mbar_expect_tx(&ctl->q_full, kTileBytes);
-            tma_box3d(smem_base + kSmemQ, &q_map, &ctl->q_full, b * p.heads + h0, 0);
+            tma_box3d(smem_base + kSmemQ, &q_map, &ctl->q_full, b * p.heads, 0);
         }
         bool any_bad = bad_len;
         // Lane l serves tokens l and l+32 of a tile.  Token positions are fetched two tiles
@@ -408,8 +404,15 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
             }
             const uint32_t m0 = __ballot_sync(0xffffffffu, r0 >= 0), m1 = __ballot_sync(0xffffffffu, r1 >= 0);
             mask = (uint64_t)m0 | ((uint64_t)m1 << 32);
-            row_lo = r0 >= 0 ? (int)r0 : 0;      // masked tokens still load a real row (row 0)
-            row_hi = r1 >= 0 ? (int)r1 : 0;
+            // a masked token repeats the row of the tile's first valid token: rows outside the
+            // selection are never read, whatever they hold
+            int stand_in = 0;
+            if (m0)
+                stand_in = __shfl_sync(0xffffffffu, (int)r0, __ffs(m0) - 1);
+            else if (m1)
+                stand_in = __shfl_sync(0xffffffffu, (int)r1, __ffs(m1) - 1);
+            row_lo = r0 >= 0 ? (int)r0 : stand_in;
+            row_hi = r1 >= 0 ? (int)r1 : stand_in;
             const int base = __shfl_sync(0xffffffffu, row_lo, 0);
             contig = __all_sync(0xffffffffu, r0 == (int64_t)base + lane && r1 == (int64_t)base + 32 + lane);
         };
@@ -644,7 +647,7 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
             tc_fence_after();
             const float lt = l + __shfl_xor_sync(0xffffffffu, l, 16);
             const float inv = lt > 0.f ? 1.f / lt : 0.f;
-            const int h = h0 + row;
+            const int h = row;
             const bool store = h < p.heads;
             const size_t u = p.splits == 1 ? ((size_t)b * p.heads + h) : (((size_t)b * p.splits + s) * p.heads + h);
 #pragma unroll 1
@@ -830,8 +833,7 @@ inline bool tc_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cached)
 
 inline omni_status_t tc_launch(const CUtensorMap *maps, const DecodeParams &p, cudaStream_t stream)
 {
-    const int head_groups = (p.heads + kTcHeads - 1) / kTcHeads;
-    const unsigned grid = (unsigned)(p.batch * p.splits * head_groups);
+    const unsigned grid = (unsigned)(p.batch * p.splits);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kTcThreads);
