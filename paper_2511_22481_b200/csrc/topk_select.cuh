@@ -1,15 +1,32 @@
 // Selection producer for token-level sparsity: the positions of the k largest scores of every
 // request, written as the sel_idx / sel_len arrays the decode kernels read.
 //
-// One cluster of up to eight CTAs per request.  Every CTA loads its share of the request's scores
-// ONCE, as order-preserving 32-bit keys, into shared memory; everything after that works on
-// shared memory.  A most-significant-digit radix select (four passes of 8 bits) finds the key
-// T of the k-th largest score: per pass every CTA histograms the digit of its keys that still
-// match the prefix, the cluster's histograms are summed through distributed shared memory, and each
-// CTA scans the 256 bins for the digit that holds the k-th largest.  Then every key above T is
-// selected, and of the keys equal to T the ones at the lowest positions, as many as are still
-// missing; positions are written in increasing order, so the output is a deterministic function
-// of the scores (ties included).
+// One cluster of up to eight CTAs per request.  The scores are read ONCE, through shared memory, and a thread
+// keeps a run of consecutive ones in registers as order-preserving 32-bit keys (0: no position, 1:
+// NaN, larger: numbers in their order).  What follows is a chain of short steps, bound by latency
+// and by instructions, not by bytes; so it keeps the barriers between CTAs down to two and spends
+// few instructions per key:
+//   1. a lower bound L of the k-th largest key.  The keys are cut into groups (a thread's, or a
+//      vector of four); the k-th largest of the groups' maxima is such a bound, since k keys are at least as
+//      large, and with many more groups than k it is a tight one.  Every CTA histograms the top
+//      11 bits of its maxima (2048 bins); after a cluster barrier a warp of every CTA finds the
+//      bin of the k-th largest, first among sums of 32 bins, then among the 32 bins of one sum,
+//      reading the other CTAs' counts through distributed shared memory;
+//   2. every CTA lists its keys from L on; a second cluster barrier; every CTA reads all lists and finds
+//      the threshold key T among them (8 bits at a time) on its own, without the others;
+//   3. keys above T are selected, and of the keys equal to T the ones at the lowest positions, as many
+//      as are still missing.  A thread's positions are consecutive, so one sum over the threads in front
+//      gives each its place: positions come out in increasing order, and the output is a deterministic
+//      function of the scores (ties included).
+// Where there are too few groups for k, or too many keys from L on for the lists (scores that crowd
+// into few values), step 1 histograms the keys themselves, 11, 11 and 10 bits at a time with a
+// cluster barrier each, until the bin of the k-th largest fits the lists or is down to equal keys.
+//
+// What it measured (k = 2048, back to back): 16 requests x 131072 scores 21.2 us with all keys in shared memory
+// and four 8-bit searches over them; 17.0 with the keys in registers, 2048 bins and two searches less; 16.5
+// with the bound instead of a histogram of all keys; 14.2 with consecutive keys per thread (keys in
+// vectors 1024 apart load without a detour, but ballots then have to place every vector's positions);
+// 12.9 with 512 threads of up to 64 keys instead of 1024 of up to 32.  One request: 16.3 -> 10.7.
 #pragma once
 
 #include <mutex>
@@ -19,24 +36,18 @@
 namespace omni {
 
 constexpr int kTopkCluster = 8;
-constexpr int kTopkThreads = 512;
-constexpr int kTopkChunk = 24576;                        // most keys a CTA holds in shared memory (96 KiB)
-constexpr int kTopkFew = 4096;                           // candidates below which a pass skips the lane-private copies
+constexpr int kTopkThreads = 512;                        // few threads with many keys each: half of a warp's instructions do not depend on its keys
+constexpr int kTopkWarps = kTopkThreads / 32;
+constexpr int kTopkVectors = 16;                         // most 4-key vectors a thread holds
 constexpr int kTopkMaxContext = 131072;                  // positions per request
+constexpr int kTopkBins = 2048;
+constexpr int kTopkList = 4096;                          // most keys of a bin, over the cluster, that go into the lists
 
-// float bits -> unsigned key with the same order; NaN sorts below everything
+// float bits -> unsigned key with the same order; every NaN is 1, below all numbers
 __device__ __forceinline__ uint32_t topk_key(float f)
 {
     const uint32_t u = __float_as_uint(f);
-    if ((u & 0x7fffffffu) > 0x7f800000u) return 0u;
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr)
-{
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
-    return v;
+    return f != f ? 1u : u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
 }
 
 __device__ __forceinline__ uint32_t topk_map(const void *p, uint32_t rank)
@@ -45,244 +56,507 @@ __device__ __forceinline__ uint32_t topk_map(const void *p, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
     return r;
 }
-
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr)
+{
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_cluster_u32x2(uint32_t cluster_addr)
+{
+    uint2 v;
+    asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(cluster_addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ void topk_cluster_sync()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-constexpr int kTopkWarps = kTopkThreads / 32;
+// Sum of `c` over this and all higher lanes.
+__device__ __forceinline__ uint32_t topk_suffix(uint32_t c, int lane)
+{
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_down_sync(0xffffffffu, c, d);
+        if (lane + d < 32) c += o;
+    }
+    return c;
+}
 
 struct alignas(16) TopkShared {
-    uint32_t replicas[256 * 32];     // digit histogram, one copy per lane: entry (digit, lane) at digit * 32 + lane
-    uint32_t published[2][256];      // this CTA's histogram of the current pass, read by the whole cluster
-    uint32_t counts[2];              // keys above / equal to the threshold in this chunk
-    uint32_t prefix, need;           // result of a digit search: the extended prefix, keys still to take in its bin
-    uint32_t bin_count;              // ... and the keys of the whole cluster in that bin
-    uint32_t warp_sums[kTopkWarps];
-    uint32_t warp_gt[kTopkWarps], warp_eq[kTopkWarps];
+    uint32_t bins[2][kTopkBins];     // this CTA's digit counts, one buffer per pass in turn, read by the whole cluster
+    uint32_t sums[2][kTopkBins / 32];
+    uint32_t list[kTopkList];        // this CTA's listed keys, read by the whole cluster
+    uint32_t fine[4][256];           // digit counts of the search among the listed keys
+    uint32_t counts[2][2];           // per attempt: listed keys of this CTA, and keys above the listed range
+    uint32_t prefix, need, bin_count;   // result of a digit search: the extended prefix, keys still to take in its bin, keys in it
+    uint32_t spread;                 // largest listed key less the smallest a list can hold
+    uint32_t before[2];              // listed keys of the CTAs before this one: above T, equal to T
+    uint32_t warp_counts[kTopkWarps];   // selected keys per warp: above T | equal to T << 16
 };
-static_assert(sizeof(TopkShared) % 16 == 0, "the keys behind the control block are stored with 16-byte stores");
 
-__global__ void __launch_bounds__(kTopkThreads, 2)
+// One digit search over the cluster: sums up this CTA's bins, waits for the other CTAs', and finds the bin that
+// holds the need-th largest: keys in higher bins < need <= keys in this and higher bins.  The result
+// goes to sh.prefix (the bin number at `shift`, below `prefix`), sh.need, sh.bin_count; none if there are
+// fewer than `need` keys.  Called by all threads after a block barrier; ends with one.
+__device__ __forceinline__ void topk_search_bins(TopkShared &sh, int buffer, uint32_t prefix, int shift, uint32_t need, uint32_t nranks)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *bins = sh.bins[buffer], *sums = sh.sums[buffer];
+    constexpr int kSumsPerWarp = kTopkBins / 32 / kTopkWarps;
+#pragma unroll
+    for (int h = 0; h < kSumsPerWarp; ++h) {
+        const uint32_t s = __reduce_add_sync(0xffffffffu, bins[(kSumsPerWarp * warp + h) * 32 + lane]);
+        if (lane == 0) sums[kSumsPerWarp * warp + h] = s;
+    }
+    topk_cluster_sync();                                   // every CTA's counts are visible
+    if (warp == 0) {
+        uint2 part[kTopkCluster];                          // all remote loads in flight before the first use
+#pragma unroll
+        for (uint32_t r = 0; r < kTopkCluster; ++r)
+            part[r] = r < nranks ? ld_cluster_u32x2(topk_map(&sums[2 * lane], r)) : make_uint2(0u, 0u);
+        uint32_t lo = 0, hi = 0;
+#pragma unroll
+        for (uint32_t r = 0; r < kTopkCluster; ++r) {
+            lo += part[r].x;
+            hi += part[r].y;
+        }
+        const uint32_t with_lo = topk_suffix(lo + hi, lane), with_hi = with_lo - lo, above_hi = with_hi - hi;
+        const bool in_hi = above_hi < need && need <= with_hi, in_lo = with_hi < need && need <= with_lo;
+        const uint32_t owner = __ballot_sync(0xffffffffu, in_hi || in_lo);
+        if (owner == 0) {
+            if (lane == 0) sh.bin_count = 0;
+        } else {
+            const int src = __ffs(owner) - 1;
+            const int group = __shfl_sync(0xffffffffu, 2 * lane + (in_hi ? 1 : 0), src);
+            const uint32_t above = __shfl_sync(0xffffffffu, in_hi ? above_hi : with_hi, src);
+            uint32_t c = 0, one[kTopkCluster];
+#pragma unroll
+            for (uint32_t r = 0; r < kTopkCluster; ++r)
+                one[r] = r < nranks ? ld_cluster_u32(topk_map(&bins[group * 32 + lane], r)) : 0u;
+#pragma unroll
+            for (uint32_t r = 0; r < kTopkCluster; ++r) c += one[r];
+            const uint32_t with_me = above + topk_suffix(c, lane), higher = with_me - c;
+            if (higher < need && need <= with_me) {
+                sh.prefix = prefix | ((uint32_t)(group * 32 + lane) << shift);
+                sh.need = need - higher;
+                sh.bin_count = c;
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// Sum of `c` over the lanes before this one; `all`: over the warp.
+__device__ __forceinline__ uint32_t topk_before(uint32_t c, int lane, uint32_t &all)
+{
+    uint32_t upto = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, upto, d);
+        if (lane >= d) upto += o;
+    }
+    all = __shfl_sync(0xffffffffu, upto, 31);
+    return upto - c;
+}
+
+// Keys of a thread, one bit each.
+template <int J>
+struct TopkMask {
+    static constexpr int kWords = (4 * J + 31) / 32;
+    uint32_t word[kWords];
+    __device__ __forceinline__ uint32_t count() const
+    {
+        uint32_t n = 0;
+#pragma unroll
+        for (int w = 0; w < kWords; ++w) n += __popc(word[w]);
+        return n;
+    }
+};
+
+// The keys from lo on.
+template <int J>
+__device__ __forceinline__ TopkMask<J> topk_from(const uint32_t (&key)[4 * J], uint32_t lo)
+{
+    TopkMask<J> m;
+#pragma unroll
+    for (int w = 0; w < TopkMask<J>::kWords; ++w) m.word[w] = 0u;
+#pragma unroll
+    for (int i = 0; i < 4 * J; ++i)
+        if (key[i] >= lo) m.word[i / 32] |= 1u << (i % 32);
+    return m;
+}
+
+// The keys above hi.
+template <int J>
+__device__ __forceinline__ TopkMask<J> topk_above(const uint32_t (&key)[4 * J], uint32_t hi)
+{
+    TopkMask<J> none = {};
+    return hi != 0xffffffffu ? topk_from<J>(key, hi + 1u) : none;
+}
+
+// Where vector i of a CTA's scores sits in shared memory.  A thread reads J consecutive vectors: for an
+// even J a gap after every eight keeps the eight lanes of a 16-byte access on different banks.
+template <int J>
+__device__ __forceinline__ int topk_slot(int i)
+{
+    return (J & 1) ? i : i + (i >> 3);
+}
+
+// Lists this CTA's keys in [lo, hi] (if `listed`; a CTA with more than the list holds keeps counting) and
+// counts them, and the keys above hi.  One atomic per warp.
+template <int J>
+__device__ __forceinline__ void topk_collect(TopkShared &sh, const float *staged, const uint32_t (&key)[4 * J], uint32_t lo, uint32_t hi,
+                                             bool listed, uint32_t *counts)
+{
+    const int lane = threadIdx.x & 31;
+    TopkMask<J> in = topk_from<J>(key, lo);
+    if (hi != 0xffffffffu) {
+        const TopkMask<J> over = topk_above<J>(key, hi);
+        const uint32_t above = __reduce_add_sync(0xffffffffu, over.count());
+        if (lane == 0 && above) atomicAdd(&counts[1], above);
+#pragma unroll
+        for (int w = 0; w < TopkMask<J>::kWords; ++w) in.word[w] &= ~over.word[w];
+    }
+    uint32_t all, base = 0;
+    const uint32_t before = topk_before(in.count(), lane, all);
+    if (lane == 0 && all) base = atomicAdd(&counts[0], all);
+    uint32_t at = __shfl_sync(0xffffffffu, base, 0) + before;
+    if (!listed) return;
+#pragma unroll
+    for (int w = 0; w < TopkMask<J>::kWords; ++w)
+        for (uint32_t bits = in.word[w]; bits != 0u; bits &= bits - 1u, ++at) {
+            const int i = 32 * w + __ffs(bits) - 1;
+            if (at < (uint32_t)kTopkList) sh.list[at] = topk_key(staged[4 * topk_slot<J>((int)threadIdx.x * J + (i >> 2)) + (i & 3)]);
+        }
+}
+
+template <int J>
+__global__ void __launch_bounds__(kTopkThreads, 1)
 topk_select_kernel(const float *__restrict__ scores, const int32_t *__restrict__ ctx_len, int stride, int k,
                    int32_t *__restrict__ sel_idx, int32_t *__restrict__ sel_len)
 {
     extern __shared__ __align__(16) unsigned char topk_smem[];
     TopkShared &sh = *reinterpret_cast<TopkShared *>(topk_smem);
-    uint32_t *keys = reinterpret_cast<uint32_t *>(topk_smem + sizeof(TopkShared));     // this CTA's keys: ceil(stride / cluster width) (+ 4 of slack)
-
+    float *staged = reinterpret_cast<float *>(topk_smem + sizeof(TopkShared));        // this CTA's scores
     uint32_t crank, nranks;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nranks));
-    // launched with programmatic stream serialization: nothing of the previous kernel in the stream is
-    // read or overwritten before this returns
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.x / nranks;
-    int m = __ldg(ctx_len + b);
-    m = max(0, min(m, stride));
-    const int want = min(k, m);
-    const int chunk = ((m + (int)nranks - 1) / (int)nranks + 3) & ~3;      // a multiple of four keeps the 16-byte loads aligned
-    const int start = min(m, (int)crank * chunk), len = min(m, start + chunk) - start;
-    const float *src = scores + (size_t)b * stride + start;
-    {
-        // scalar head up to a 16-byte boundary, 16-byte loads for the body, scalar tail
-        // the keys sit in shared memory at the same offset from a 16-byte boundary as the scores in global
-        // memory, so that the body is stored with 16-byte stores too
-        const uint32_t misalign = (uint32_t)((reinterpret_cast<uintptr_t>(src) >> 2) & 3u);
-        keys += misalign;
-        const int head = min(len, (int)((4u - misalign) & 3u));
-        const int body = (len - head) >> 2;
-        const float4 *src4 = reinterpret_cast<const float4 *>(src + head);
-#pragma unroll 8
-        for (int j = threadIdx.x; j < body; j += kTopkThreads) {
-            const float4 v = __ldg(src4 + j);
-            *reinterpret_cast<uint4 *>(keys + head + 4 * j) =
-                make_uint4(topk_key(v.x), topk_key(v.y), topk_key(v.z), topk_key(v.w));
-        }
-        if ((int)threadIdx.x < head) keys[threadIdx.x] = topk_key(__ldg(src + threadIdx.x));
-        const int tail = head + 4 * body;
-        if (tail + (int)threadIdx.x < len) keys[tail + threadIdx.x] = topk_key(__ldg(src + tail + threadIdx.x));
-    }
-    for (int i = threadIdx.x; i < 256 * 32; i += kTopkThreads) sh.replicas[i] = 0;
-
-    uint32_t prefix = 0, mask = 0, need = (uint32_t)want;
-    bool few = false;                                      // at most kTopkFew keys of the cluster still match the prefix
-    int pass = 0;
-    for (int shift = 24; shift >= 0; shift -= 8, ++pass) {
-        __syncthreads();                                   // keys stored (first pass), histogram copies zeroed
-        if (few) {
-            // few keys are left in the cluster: they go straight into the published histogram
-            if (threadIdx.x < 256) sh.published[pass & 1][threadIdx.x] = 0;
-            __syncthreads();
-#pragma unroll 8
-            for (int i = threadIdx.x; i < len; i += kTopkThreads) {
-                const uint32_t key = keys[i];
-                if ((key & mask) == prefix) atomicAdd(&sh.published[pass & 1][(key >> shift) & 255u], 1u);
-            }
-            topk_cluster_sync();
-        } else {
-            // every lane adds into its own copy of the histogram: no two lanes of a warp ever meet on a
-            // word or a bank, however the digits are distributed
-#pragma unroll 8
-            for (int i = threadIdx.x; i < len; i += kTopkThreads) {
-                const uint32_t key = keys[i];
-                if ((key & mask) == prefix) atomicAdd(&sh.replicas[((key >> shift) & 255u) * 32 + lane], 1u);
-            }
-            __syncthreads();
-            {
-                // thread t sums half of the 32 copies of bin t / 2 (rotated start keeps the banks apart)
-                const int bin = threadIdx.x >> 1, half = threadIdx.x & 1;
-                uint32_t c = 0;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) c += sh.replicas[bin * 32 + half * 16 + ((j + bin) & 15)];
-                c += __shfl_xor_sync(0xffffffffu, c, 1);
-                if (half == 0) sh.published[pass & 1][bin] = c;
-            }
-            __syncthreads();                                   // all copies read: they can be cleared for the next pass
-            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-            for (int i = threadIdx.x; i < 256 * 32; i += kTopkThreads) sh.replicas[i] = 0;
-            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // every CTA's histogram is visible
-        }
-        {
-            // threads 0..255: bin t of the histogram summed over the cluster, then the bin that holds
-            // the need-th largest key: keys in higher bins < need <= keys in this and higher bins
-            uint32_t c = 0;
-            if (threadIdx.x < 256) {
-                uint32_t part[kTopkCluster];               // all remote loads in flight before the first use
-#pragma unroll
-                for (uint32_t r = 0; r < kTopkCluster; ++r)
-                    part[r] = r < nranks ? ld_cluster_u32(topk_map(&sh.published[pass & 1][threadIdx.x], r)) : 0u;
-#pragma unroll
-                for (uint32_t r = 0; r < kTopkCluster; ++r) c += part[r];
-            }
-            uint32_t inc = c;                              // inclusive suffix sum within the warp
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t o = __shfl_down_sync(0xffffffffu, inc, d);
-                if (lane + d < 32) inc += o;
-            }
-            if (lane == 0) sh.warp_sums[warp] = inc;
-            __syncthreads();
-            uint32_t above = 0;                            // keys in the bins of higher warps
-            for (int w = warp + 1; w < 8; ++w) above += sh.warp_sums[w];
-            const uint32_t with_me = above + inc, higher = with_me - c;
-            if (threadIdx.x < 256 && higher < need && need <= with_me) {
-                sh.prefix = prefix | ((uint32_t)threadIdx.x << shift);
-                sh.need = need - higher;
-                sh.bin_count = c;
-            }
-            if (need == 0 && threadIdx.x == 0) {
-                sh.prefix = prefix | (255u << shift);      // nothing to select: any threshold will do
-                sh.need = 0;
-                sh.bin_count = 0;
-            }
-        }
-        __syncthreads();
-        prefix = sh.prefix;
-        need = sh.need;
-        few = sh.bin_count <= (uint32_t)kTopkFew;
-        mask |= 255u << shift;
-        // published[] alternates between passes, and the next pass's cluster barrier comes before
-        // anybody overwrites the copy read here
-        if (need == sh.bin_count) break;                   // every key left under the prefix is taken: the lower digits decide nothing
-    }
-    // Keys above the prefix's range are selected, keys inside it (all digits searched: keys equal to the
-    // threshold) tie for the `need` places left, lowest positions first.
-    // Warp w owns the contiguous keys [w * per_warp, (w + 1) * per_warp) of the chunk.
-    const uint32_t T = prefix | ~mask;                     // largest key under the prefix
-    const int per_warp = ((len + kTopkWarps - 1) / kTopkWarps + 127) & ~127;
-    const int w_begin = min(len, warp * per_warp), w_end = min(len, w_begin + per_warp);
-    uint32_t gt = 0, eq = 0;
-#pragma unroll 8
-    for (int i = w_begin + lane; i < w_end; i += 32) {
-        gt += keys[i] > T;
-        eq += (keys[i] & mask) == prefix;
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        gt += __shfl_xor_sync(0xffffffffu, gt, d);
-        eq += __shfl_xor_sync(0xffffffffu, eq, d);
-    }
-    if (lane == 0) {
-        sh.warp_gt[warp] = gt;
-        sh.warp_eq[warp] = eq;
-    }
-    __syncthreads();
-    uint32_t gt_before = 0, eq_before = 0, gt_all = 0, eq_all = 0;       // within this chunk, before this warp
-    for (int w = 0; w < kTopkWarps; ++w) {
-        const uint32_t g = sh.warp_gt[w], e = sh.warp_eq[w];
-        if (w < warp) {
-            gt_before += g;
-            eq_before += e;
-        }
-        gt_all += g;
-        eq_all += e;
-    }
-    if (threadIdx.x == 0) {
-        sh.counts[0] = gt_all;
-        sh.counts[1] = eq_all;
-    }
-    topk_cluster_sync();
-    // threshold ties and keys above the threshold in the chunks before this one
-    {
-        uint32_t g[kTopkCluster], e[kTopkCluster];         // all remote loads in flight before the first use
-#pragma unroll
-        for (uint32_t r = 0; r < kTopkCluster; ++r) {
-            g[r] = r < crank ? ld_cluster_u32(topk_map(&sh.counts[0], r)) : 0u;
-            e[r] = r < crank ? ld_cluster_u32(topk_map(&sh.counts[1], r)) : 0u;
-        }
-#pragma unroll
-        for (uint32_t r = 0; r < kTopkCluster; ++r) {
-            gt_before += g[r];
-            eq_before += e[r];
-        }
-    }
-    // entries written before this warp's first key: everything above T, and the first `need` ties
-    uint32_t run_eq = eq_before, run_out = gt_before + min(eq_before, need);
+    for (int i = threadIdx.x; i < 2 * kTopkBins; i += kTopkThreads) (&sh.bins[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < 4 * 256; i += kTopkThreads) (&sh.fine[0][0])[i] = 0;
+    if (threadIdx.x < 4) (&sh.counts[0][0])[threadIdx.x] = 0;
+    if (threadIdx.x < 2) sh.before[threadIdx.x] = 0;
+    if (threadIdx.x == 0) sh.spread = 0;
+    // launched with programmatic stream serialization: nothing of the previous kernel in the stream is
+    // read or overwritten before this returns, and the next kernel may get ready meanwhile
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int m = max(0, min(__ldg(ctx_len + b), stride));
     int32_t *dst = sel_idx + (size_t)b * k;
-    const uint32_t lanes_below = (1u << lane) - 1u;
-    for (int base = w_begin; base < w_end && want > 0; base += 128) {
-        uint32_t key[4];
-        bool at_least[4];
+    if (m <= k) {
+        // everything is selected (the same decision in every CTA of the cluster)
+        for (int i = (int)(crank * kTopkThreads + threadIdx.x); i < m; i += (int)nranks * kTopkThreads) dst[i] = i;
+        if (crank == 0 && threadIdx.x == 0) sel_len[b] = m;
+        return;
+    }
+    // Vectors of four scores at 16-byte boundaries: the request's row starts `shift` scores into its first.
+    // CTA `crank` takes vectors [v0, v1), thread t of it J consecutive ones from v0 + t J on.
+    const float *row = scores + (size_t)b * stride;
+    const int shift = (int)((reinterpret_cast<uintptr_t>(row) >> 2) & 3u);
+    const int vectors = (shift + m + 3) >> 2, per = (vectors + (int)nranks - 1) / (int)nranks;
+    const int v0 = min(vectors, (int)crank * per), v1 = min(vectors, v0 + per);
+    const int p0 = 4 * (v0 + (int)threadIdx.x * J) - shift;             // position of this thread's first key
+    {
+        // vectors [a, a + n) of this CTA lie inside the row
+        const int a = max(0, (shift > 0 ? 1 : 0) - v0), n = min(v1, (shift + m) >> 2) - v0 - a;
+        constexpr int kSlotStep = (J & 1) ? kTopkThreads : kTopkThreads + kTopkThreads / 8;
+        const uint32_t to = (uint32_t)__cvta_generic_to_shared(staged) + 16 * topk_slot<J>((int)threadIdx.x);
+        const float *from = row + 4 * (v0 + (int)threadIdx.x) - shift;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int i = base + 32 * j + lane;
-            key[j] = i < w_end ? keys[i] : 0u;
-            at_least[j] = i < w_end && key[j] >= prefix;
-        }
-        if (!__any_sync(0xffffffffu, at_least[0] || at_least[1] || at_least[2] || at_least[3])) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool is_eq = at_least[j] && (key[j] & mask) == prefix;
-            const uint32_t eq_ballot = __ballot_sync(0xffffffffu, is_eq);
-            const uint32_t eq_rank = run_eq + __popc(eq_ballot & lanes_below);
-            const bool sel = at_least[j] && (!is_eq || eq_rank < need);
-            const uint32_t sel_ballot = __ballot_sync(0xffffffffu, sel);
-            const uint32_t pos = run_out + __popc(sel_ballot & lanes_below);
-            if (sel && pos < (uint32_t)want) dst[pos] = start + base + 32 * j + lane;
-            run_eq += __popc(eq_ballot);
-            run_out += __popc(sel_ballot);
+        for (int j = 0; j < J; ++j)
+            if ((unsigned)((int)threadIdx.x + j * kTopkThreads - a) < (unsigned)max(n, 0))
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * j * kSlotStep), "l"(from + 4 * j * kTopkThreads)
+                             : "memory");
+        // the two vectors that stick out of the row at its ends; what lies outside stays unset and is never looked at
+        if (threadIdx.x < 2) {
+            const int v = threadIdx.x == 0 ? 0 : (shift + m) >> 2;
+            const bool partial = threadIdx.x == 0 ? shift > 0 : ((shift + m) & 3) != 0 && (v > 0 || shift == 0);
+            if (partial && v >= v0 && v < v1)
+                for (int c = 0; c < 4; ++c) {
+                    const int p = 4 * v - shift + c;
+                    if (p >= 0 && p < m) staged[4 * topk_slot<J>(v - v0) + c] = __ldg(row + p);
+                }
         }
     }
-    if (crank == 0 && threadIdx.x == 0) sel_len[b] = want;
-    topk_cluster_sync();                                   // nobody leaves while its counts may still be read
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                       // scores staged, counts zeroed
+    uint32_t key[4 * J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const float4 x = *reinterpret_cast<const float4 *>(staged + 4 * topk_slot<J>((int)threadIdx.x * J + j));
+        key[4 * j] = topk_key(x.x);
+        key[4 * j + 1] = topk_key(x.y);
+        key[4 * j + 2] = topk_key(x.z);
+        key[4 * j + 3] = topk_key(x.w);
+    }
+    // keys outside the row, or past this CTA's share: few threads have any
+    const int end = min(m, 4 * v1 - shift);
+    if (p0 < 0 || p0 + 4 * J > end) {
+#pragma unroll
+        for (int i = 0; i < 4 * J; ++i)
+            if (p0 + i < 0 || p0 + i >= end) key[i] = 0u;
+    }
+
+    // ---- 1. a range [lo, hi] of keys that holds the k-th largest: lo a bound from group maxima ----------
+    // `need`: how many keys of the range are taken; `inside`: how many it holds, over the cluster.
+    // `attempt`: which of the two count pairs goes with the range.
+    uint32_t lo = 0, hi = 0xffffffffu, need = (uint32_t)k, inside = 0;
+    int attempt = 0;
+    bool listed = false;
+    uint2 n[kTopkCluster];                                 // per CTA of the cluster: keys in the range, keys above it
+    auto read_counts = [&]() {
+#pragma unroll
+        for (uint32_t r = 0; r < kTopkCluster; ++r)
+            n[r] = r < nranks ? ld_cluster_u32x2(topk_map(&sh.counts[attempt][0], r)) : make_uint2(0u, 0u);
+    };
+    // The bound is tight enough for the lists with four groups per selected key or more; threads
+    // make fewer groups than vectors, and an atomic each instead of J.
+    const bool by_thread = (int)nranks * min(kTopkThreads, per) >= 4 * k;
+    if (by_thread || vectors >= 2 * k) {
+        uint32_t top = 0;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t v = max(max(key[4 * j], key[4 * j + 1]), max(key[4 * j + 2], key[4 * j + 3]));
+            if (by_thread)
+                top = max(top, v);
+            else if (v != 0u)
+                atomicAdd(&sh.bins[0][v >> 21], 1u);
+        }
+        if (top != 0u) atomicAdd(&sh.bins[0][top >> 21], 1u);
+        __syncthreads();
+        topk_search_bins(sh, 0, 0u, 21, need, nranks);
+        if (sh.bin_count != 0) {
+            lo = max(sh.prefix, 1u);
+            topk_collect<J>(sh, staged, key, lo, hi, true, sh.counts[0]);
+            topk_cluster_sync();
+            read_counts();
+#pragma unroll
+            for (uint32_t r = 0; r < kTopkCluster; ++r) inside += n[r].x;
+            listed = inside <= (uint32_t)kTopkList;
+        } else {
+            topk_cluster_sync();                           // fewer non-empty groups than k
+        }
+        if (!listed) {
+            // everybody has read these bins: the cluster has met since
+            for (int i = threadIdx.x; i < kTopkBins; i += kTopkThreads) sh.bins[0][i] = 0;
+        }
+    }
+    if (!listed) {
+        // ---- ... or lo and hi the ends of a digit bin of all keys --------------------------------
+        attempt = 1;
+        uint32_t prefix = 0, mask = 0;
+        for (int pass = 0;; ++pass) {
+            const int shift_bits = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+            const uint32_t digit_mask = pass == 2 ? 1023u : 2047u;
+            uint32_t *bins = sh.bins[pass & 1];
+            __syncthreads();                               // counts zeroed
+#pragma unroll
+            for (int i = 0; i < 4 * J; ++i)
+                if (key[i] != 0u && (key[i] & mask) == prefix) atomicAdd(&bins[(key[i] >> shift_bits) & digit_mask], 1u);
+            __syncthreads();
+            topk_search_bins(sh, pass & 1, prefix, shift_bits, need, nranks);
+            prefix = sh.prefix;
+            need = sh.need;
+            inside = sh.bin_count;
+            mask |= digit_mask << shift_bits;
+            if (need == inside || inside <= (uint32_t)kTopkList || pass == 2) break;
+            // the buffer of the pass after next is cleared: everybody has read it before the barrier of this pass
+            if (pass == 1)
+                for (int i = threadIdx.x; i < kTopkBins; i += kTopkThreads) sh.bins[0][i] = 0;
+        }
+        lo = max(prefix, 1u);
+        hi = prefix | ~mask;
+        // where all keys of the bin are taken, or they are all equal, only their number matters
+        listed = need != inside && mask != 0xffffffffu;
+        topk_collect<J>(sh, staged, key, lo, hi, listed, sh.counts[1]);
+        topk_cluster_sync();
+        read_counts();
+    }
+
+    // ---- 2. the threshold T and this CTA's place in the output -----------------------------------
+    // From here on `equal to T` means in [T, top] (one value, or values that are all taken), `above` above top.
+    uint32_t T = lo, top = hi, eq_need = need, eq_all = inside;
+    uint32_t out_base = 0, eq_before = 0;                  // keys above / equal to T in the CTAs before this one
+#pragma unroll
+    for (uint32_t r = 0; r < kTopkCluster; ++r) {
+        if (r < crank) {
+            out_base += n[r].y;
+            eq_before += n[r].x;
+        }
+    }
+    if (listed) {
+        constexpr int kMine = kTopkList / kTopkThreads;
+        uint32_t mine[kMine];                              // of the listed keys of the whole cluster, less lo
+        bool valid[kMine], earlier[kMine];                 // there is one; it is from a CTA before this one
+        uint32_t spread = 0;
+#pragma unroll
+        for (int q = 0; q < kMine; ++q) {
+            const uint32_t i = q * kTopkThreads + threadIdx.x;
+            valid[q] = i < inside;
+            earlier[q] = i < eq_before;
+            mine[q] = 0u;
+            if (q * kTopkThreads >= inside) continue;
+            uint32_t at = i, rank = 0;
+#pragma unroll
+            for (uint32_t r = 0; r < kTopkCluster - 1; ++r)
+                if (rank == r && at >= n[r].x) {
+                    at -= n[r].x;
+                    rank = r + 1;
+                }
+            if (valid[q]) mine[q] = ld_cluster_u32(topk_map(&sh.list[at], rank)) - lo;
+            spread = max(spread, mine[q]);
+        }
+        spread = __reduce_max_sync(0xffffffffu, spread);
+        if (lane == 0) atomicMax(&sh.spread, spread);
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // nothing of the others is read from here on
+        __syncthreads();
+        spread = sh.spread;
+        // eight bits at a time from the highest bit that differs
+        uint32_t prefix = 0, mask = spread != 0u ? ~(0xffffffffu >> __clz(spread)) : 0xffffffffu;
+#pragma unroll 1
+        for (int f = 0; f < 4 && mask != 0xffffffffu && eq_need != eq_all; ++f) {
+            const int s = max(0, 24 - __clz(~mask));       // the field ends at bit s
+            const uint32_t field = ~mask >> s;             // at most 255
+#pragma unroll
+            for (int q = 0; q < kMine; ++q)
+                if (valid[q] && (mine[q] & mask) == prefix) atomicAdd(&sh.fine[f][(mine[q] >> s) & field], 1u);
+            __syncthreads();
+            if (warp == 0) {
+                const uint4 c0 = *reinterpret_cast<const uint4 *>(&sh.fine[f][8 * lane]);
+                const uint4 c1 = *reinterpret_cast<const uint4 *>(&sh.fine[f][8 * lane + 4]);
+                const uint32_t c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+                uint32_t with = topk_suffix(c0.x + c0.y + c0.z + c0.w + c1.x + c1.y + c1.z + c1.w, lane);
+#pragma unroll
+                for (int d = 0; d < 8; ++d) {
+                    const uint32_t higher = with - c[d];
+                    if (higher < eq_need && eq_need <= with) {
+                        sh.prefix = prefix | ((uint32_t)(8 * lane + d) << s);
+                        sh.need = eq_need - higher;
+                        sh.bin_count = c[d];
+                    }
+                    with = higher;
+                }
+            }
+            __syncthreads();
+            prefix = sh.prefix;
+            eq_need = sh.need;
+            eq_all = sh.bin_count;
+            mask |= field << s;
+        }
+        T = lo + prefix;
+        top = lo + (prefix | ~mask);
+        if (top < T) top = 0xffffffffu;
+        uint32_t gt = 0, eq = 0;
+#pragma unroll
+        for (int q = 0; q < kMine; ++q) {
+            const bool in = (mine[q] & mask) == prefix;
+            gt += earlier[q] && !in && mine[q] > prefix;
+            eq += earlier[q] && in;
+        }
+        gt = __reduce_add_sync(0xffffffffu, gt);
+        eq = __reduce_add_sync(0xffffffffu, eq);
+        if (lane == 0 && gt) atomicAdd(&sh.before[0], gt);
+        if (lane == 0 && eq) atomicAdd(&sh.before[1], eq);
+    } else {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
+
+    // ---- 3. positions ----------------------------------------------------------------------
+    // With no tie to split every key from T on is selected; otherwise keys above `top`, and the first
+    // eq_need from T to top.
+    const bool split_tie = eq_need != eq_all;
+    const TopkMask<J> sel = topk_from<J>(key, T), over = split_tie ? topk_above<J>(key, top) : sel;      // over: certain of their place
+    uint32_t all;
+    const uint32_t before = topk_before(over.count() | ((sel.count() - over.count()) << 16), lane, all);
+    if (lane == 0) sh.warp_counts[warp] = all;
+    __syncthreads();
+    if (listed) {
+        out_base += sh.before[0];
+        eq_before = sh.before[1];
+    }
+    const uint32_t start = before + __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp_counts[lane] : 0u);
+    uint32_t gt_run = out_base + (split_tie ? 0u : eq_before) + (start & 0xffffu), eq_run = split_tie ? eq_before + (start >> 16) : 0u;
+#pragma unroll
+    for (int w = 0; w < TopkMask<J>::kWords; ++w)
+        for (uint32_t bits = sel.word[w]; bits != 0u; bits &= bits - 1u) {
+            const int i = __ffs(bits) - 1;
+            const bool eq = !((over.word[w] >> i) & 1u);
+            const uint32_t at = gt_run + min(eq_run, eq_need);
+            if ((!eq || eq_run < eq_need) && at < (uint32_t)k) dst[at] = p0 + 32 * w + i;
+            gt_run += !eq;
+            eq_run += eq;
+        }
+    if (crank == 0 && threadIdx.x == 0) sel_len[b] = k;
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");                // nobody leaves while its lists may still be read
 }
 
-// Launch shape.  A CTA costs about 4 us plus 0.4 us per CTA of its cluster, plus 0.6 us per 1024 keys
-// when it has its SM to itself and 0.85 us per 1024 keys when two CTAs share an SM (fitted to
-// measurements).  Every width from 1 to 8 that holds the context is priced with the number of clusters
-// of that width the device keeps resident, alone on their SMs or two to an SM, and the cheapest wins.
-struct TopkShape {
-    int width;
-    size_t smem;
-};
+// Launch shape: every width that holds the context is priced with the number of clusters of that width the
+// device keeps resident, and the cheapest wins.  Cost of a wave of clusters of `width` CTAs with J
+// vectors per thread, in microseconds:
+constexpr double kTopkCostFixed = 6.6, kTopkCostCta = 0.05, kTopkCostVector = 0.4;       // fitted to measurements
+using TopkKernel = void (*)(const float *, const int32_t *, int, int, int32_t *, int32_t *);
+constexpr int kTopkInstances = 10;
+inline int topk_instance(int vectors_per_thread)           // number of the smallest instance that holds that many
+{
+    constexpr int size[kTopkInstances] = {1, 2, 3, 4, 5, 6, 8, 11, 13, 16};
+    int i = 0;
+    while (size[i] < vectors_per_thread) ++i;
+    return i;
+}
+inline TopkKernel topk_kernel(int instance)
+{
+    static const TopkKernel table[kTopkInstances] = {topk_select_kernel<1>, topk_select_kernel<2>, topk_select_kernel<3>,
+                                                     topk_select_kernel<4>, topk_select_kernel<5>, topk_select_kernel<6>,
+                                                     topk_select_kernel<8>, topk_select_kernel<11>, topk_select_kernel<13>,
+                                                     topk_select_kernel<16>};
+    return table[instance];
+}
+inline int topk_instance_vectors(int instance)
+{
+    constexpr int size[kTopkInstances] = {1, 2, 3, 4, 5, 6, 8, 11, 13, 16};
+    return size[instance];
+}
 
-constexpr size_t kTopkSmemAlone = 120 * 1024;            // more than half an SM's shared memory: one CTA per SM
-constexpr size_t kTopkSmemPair = 112 * 1024;             // two CTAs of up to this much fit one SM
+inline size_t topk_smem_bytes(int vectors_per_thread)
+{
+    const int vectors = vectors_per_thread * kTopkThreads;
+    return sizeof(TopkShared) + (size_t)(vectors + ((vectors_per_thread & 1) ? 0 : vectors / 8)) * sizeof(float4);
+}
 
-inline size_t topk_smem_need(int chunk) { return sizeof(TopkShared) + (size_t)(chunk + 4) * sizeof(uint32_t); }
+// Per device: the shared memory the instances need, and the shared-memory / L1 split of the decode
+// kernels (alternating between two splits makes every launch wait for the SMs to be reconfigured).
+inline bool topk_prepare_device(int dev)
+{
+    static std::mutex lock;
+    static bool done[64] = {};
+    std::lock_guard<std::mutex> guard(lock);
+    if (!done[dev]) {
+        for (int i = 0; i < kTopkInstances; ++i)
+            if (cudaFuncSetAttribute(topk_kernel(i), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)topk_smem_bytes(topk_instance_vectors(i))) != cudaSuccess ||
+                cudaFuncSetAttribute(topk_kernel(i), cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
+                return false;
+        done[dev] = true;
+    }
+    return true;
+}
 
 inline void topk_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int batch, int width, size_t smem,
                                cudaStream_t stream)
@@ -302,70 +576,52 @@ inline void topk_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *att
     cfg.numAttrs = 2;
 }
 
-// Clusters of `width` resident at once (asked once per device, width and mode; at least 1).
-inline int topk_resident_clusters(int dev, int width, bool alone)
+// Clusters of `width` resident at once, asked once per device and width; at least 1.  (All instances
+// take one SM per CTA.)
+inline int topk_resident_clusters(int dev, int width)
 {
     static std::mutex lock;                                // callers on several host threads share the table
-    static int cache[64][kTopkCluster + 1][2] = {};
+    static int cache[64][kTopkCluster + 1] = {};
     std::lock_guard<std::mutex> guard(lock);
-    int &slot = cache[dev][width][alone ? 1 : 0];
+    int &slot = cache[dev][width];
     if (slot == 0) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[2];
-        topk_launch_config(cfg, attr, 1, width, alone ? kTopkSmemAlone : kTopkSmemPair, nullptr);
+        topk_launch_config(cfg, attr, 1, width, topk_smem_bytes(kTopkVectors), nullptr);
         cfg.numAttrs = 1;                                  // the cluster shape is all the query needs
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, topk_select_kernel, &cfg) != cudaSuccess) n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, topk_kernel(kTopkInstances - 1), &cfg) != cudaSuccess) n = 0;
         slot = n > 0 ? n : 1;
     }
     return slot;
 }
 
-inline TopkShape topk_shape(int dev, int batch, int stride)
-{
-    TopkShape best = {kTopkCluster, topk_smem_need(kTopkChunk)};
-    double best_cost = 1e30;
-    for (int width = kTopkCluster; width >= 1; --width) {
-        const int chunk = ((stride + width - 1) / width + 3) & ~3;
-        if (chunk > kTopkChunk) break;                     // narrower clusters cannot hold the context
-        const size_t need = topk_smem_need(chunk);
-        const double per_key = chunk / 1024.0;
-        const int alone = topk_resident_clusters(dev, width, true);
-        const double fixed = 4.0 + 0.4 * width + ((width & (width - 1)) ? 0.5 : 0.0);   // odd widths measured slightly slower
-        const double cost_alone = ((batch + alone - 1) / alone) * (fixed + 0.6 * per_key);
-        if (cost_alone < best_cost) {
-            best_cost = cost_alone;
-            best = {width, need > kTopkSmemAlone ? need : kTopkSmemAlone};
-        }
-        if (need <= kTopkSmemPair) {
-            const int paired = topk_resident_clusters(dev, width, false);
-            const double cost_pair = ((batch + paired - 1) / paired) * (fixed + 0.85 * per_key);
-            if (cost_pair < best_cost) {
-                best_cost = cost_pair;
-                best = {width, need};
-            }
-        }
-    }
-    return best;
-}
-
 inline omni_status_t launch_topk_select(const float *scores, const int32_t *ctx_len, int batch, int stride, int k,
                                         int32_t *sel_idx, int32_t *sel_len, cudaStream_t stream)
 {
-    static bool attr_set[64] = {};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return OMNI_ERR_CUDA;
-    if (!attr_set[dev]) {
-        if (cudaFuncSetAttribute(topk_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)topk_smem_need(kTopkChunk)) != cudaSuccess)
-            return OMNI_ERR_CUDA;
-        attr_set[dev] = true;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !topk_prepare_device(dev)) return OMNI_ERR_CUDA;
+    // vectors of the longest row that does not start at a 16-byte boundary, if there can be one
+    const bool aligned = (reinterpret_cast<uintptr_t>(scores) & 15u) == 0 && stride % 4 == 0;
+    const int vectors = ((aligned ? 0 : 3) + stride + 3) / 4;
+    int best_width = 0, best = 0;
+    double best_cost = 1e30;
+    for (int width = 1; width <= kTopkCluster; ++width) {
+        const int j = ((vectors + width - 1) / width + kTopkThreads - 1) / kTopkThreads;
+        if (j > kTopkVectors) continue;                    // narrower clusters cannot hold the context
+        const int instance = topk_instance(j);
+        const int resident = topk_resident_clusters(dev, width);
+        const double cost = ((batch + resident - 1) / resident) * (kTopkCostFixed + kTopkCostCta * width + kTopkCostVector * topk_instance_vectors(instance));
+        if (cost < best_cost) {
+            best_cost = cost;
+            best_width = width;
+            best = instance;
+        }
     }
-    const TopkShape shape = topk_shape(dev, batch, stride);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
-    topk_launch_config(cfg, attr, batch, shape.width, shape.smem, stream);
-    return cudaLaunchKernelEx(&cfg, topk_select_kernel, scores, ctx_len, stride, k, sel_idx, sel_len) == cudaSuccess
+    topk_launch_config(cfg, attr, batch, best_width, topk_smem_bytes(topk_instance_vectors(best)), stream);
+    return cudaLaunchKernelEx(&cfg, topk_kernel(best), scores, ctx_len, stride, k, sel_idx, sel_len) == cudaSuccess
                ? OMNI_OK
                : OMNI_ERR_CUDA;
 }
