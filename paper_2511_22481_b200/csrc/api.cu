@@ -613,11 +613,10 @@ omni_status_t omni_kv_append_rolling(const omni_mla_desc_t *desc, void *kv_cache
     if ((int64_t)desc->max_pages_per_req < rolling_sink_pages(n_sink) + rolling_ring_pages(n_recent)) return OMNI_ERR_SHAPE;
     if (!aligned(kv_cache, 128) || !aligned(new_rows, 16) || !aligned(page_table, 4) || !aligned(ctx_len, 4))
         return OMNI_ERR_ALIGN;
-    append_rolling_kernel<<<(unsigned)desc->batch, 72, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<__nv_bfloat16 *>(kv_cache), page_table, ctx_len, static_cast<const __nv_bfloat16 *>(new_rows),
-        desc->max_pages_per_req, desc->num_pages, (int)rolling_sink_pages(n_sink), (int)rolling_ring_pages(n_recent),
-        device_status);
-    return cudaPeekAtLastError() == cudaSuccess ? OMNI_OK : OMNI_ERR_CUDA;
+    return launch_overlapped(append_rolling_kernel, (unsigned)desc->batch, 72, static_cast<cudaStream_t>(stream),
+                             static_cast<__nv_bfloat16 *>(kv_cache), page_table, ctx_len, static_cast<const __nv_bfloat16 *>(new_rows),
+                             desc->max_pages_per_req, desc->num_pages, (int)rolling_sink_pages(n_sink),
+                             (int)rolling_ring_pages(n_recent), device_status);
 }
 
 omni_status_t omni_sparse_mla_combine(const omni_mla_desc_t *desc, int32_t max_splits,

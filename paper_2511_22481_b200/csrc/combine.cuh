@@ -136,6 +136,10 @@ __global__ void __launch_bounds__(72) append_rolling_kernel(__nv_bfloat16 *__res
                                                             int max_pages, int64_t num_pages, int sink_pages,
                                                             int ring_pages, int32_t *status)
 {
+    // launched as a programmatic dependent between two decode steps: the launch gaps on either side would
+    // cost more than the copy (the step it precedes waits for this one before it reads)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.x;
     const int32_t t = __ldg(ctx_len + b);
     int64_t row = -1;
