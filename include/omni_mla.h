@@ -365,12 +365,13 @@ omni_status_t omni_sparse_mla_resolve_rows(const omni_mla_desc_t *desc,
  *                            omni_sparse_mla_host_staging_bytes(desc), 256-byte aligned
  *                            (the size includes split-KV scratch for the two-part schedule below)
  * Everything is ordered on `stream`: the host buffers may be read after the stream is
- * synchronised.  From a batch of a few megabytes of q and out on (at least 4 requests), the
- * call runs the batch as two parts: the second part's q copy and, later, its kernel and copies
- * out go to a stream the library creates once per device, which waits for `stream` at the
- * start and which `stream` waits for at the end, so that copies in, kernels and copies out of
- * the two parts overlap (PCIe carries both directions at once).  `workspace` is used only when
- * the batch runs as one part.
+ * synchronised.  With pinned, 16-byte aligned buffers (all six) the kernels read the index arrays and
+ * write out and lse in place.  From a batch of a few megabytes of q and out on (at least 4
+ * requests), the call runs the batch as two to four parts: q, part after part, is copied on a
+ * stream the library creates, which waits for `stream` at the start and which `stream` waits for
+ * at the end, so that copies in, kernels and results out of the parts overlap (PCIe carries both
+ * directions at once); other host memory is copied both ways, a large batch as two parts.
+ * `workspace` is used only when the batch runs as one part.
  */
 size_t omni_sparse_mla_host_staging_bytes(const omni_mla_desc_t *desc);
 omni_status_t omni_sparse_mla_decode_host(const omni_mla_desc_t *desc, const void *q_host,

@@ -2,10 +2,12 @@
 // workspace carving and kernel launches.  Nothing here allocates device memory.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "combine.cuh"
 #include "common.cuh"
+#include "host_gather.cuh"
 #include "simt_decode.cuh"
 #include "tc_decode.cuh"
 #include "tc2_decode.cuh"
@@ -665,10 +667,19 @@ omni_status_t omni_sparse_mla_resolve_rows(const omni_mla_desc_t *desc,
 }
 
 
-// The host-buffer entry point splits a large batch into two parts so that the second part's
-// host-to-device copies run under the first half's kernel, and the first half's device-to-host
-// copies under the second half's kernel (PCIe carries both directions at once).  The second half
-// runs on a stream of the library's own, which forks from and joins back into the caller's.
+// The host-buffer entry point moves q and the index arrays in and out and lse back over PCIe, which carries
+// both directions at once.  With pinned buffers, which is what they are for, one kernel reads the index arrays (see
+// host_gather.cuh).  A small batch runs as one part: that kernel reads q too, and the decode
+// kernels store out and lse straight into the host buffers (a copy out would start only after their last
+// store, and costs 4-7 us of its own): one request of 16 heads 49 -> 20 us, four of 128 77 -> 47.
+// A large batch runs as up to four parts: on one stream of the library's the copy engine brings q,
+// part after part, on another it takes the results of a part back, and the kernels run on the
+// caller's stream, which both fork from and join back into.  The copy engines do it there because
+// reads and writes of the SMs over PCIe hold each other up (5 MB each way: 201 us together, 125 with
+// the copy engine reading); only the last part, which has PCIe to itself, stores its results in
+// place.  32 requests: 203 -> 178 us, of which 125 are the transfers if both directions overlapped
+// throughout.
+// Other host memory goes through copies, a large batch in two halves.
 static size_t host_copy_bytes(const omni_mla_desc_t *desc)
 {
     const size_t B = desc->batch, H = desc->num_heads;
@@ -700,10 +711,11 @@ static size_t host_half_workspace(const omni_mla_desc_t *desc, int half)
 // Side streams of the host-buffer entry point: a few per device, chosen by the caller's stream, so
 // that calls in flight on different streams do not queue their second halves behind one another.
 constexpr int kHostSideStreams = 4;
-static cudaStream_t host_side_stream(cudaStream_t caller)
+static cudaStream_t host_side_stream(cudaStream_t caller, int which = 0)
 {
     static std::mutex lock;
-    static cudaStream_t streams[64][kHostSideStreams] = {};
+    static cudaStream_t all[2][64][kHostSideStreams] = {};
+    cudaStream_t(*streams)[kHostSideStreams] = all[which];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
     const uintptr_t h = reinterpret_cast<uintptr_t>(caller);
@@ -714,13 +726,90 @@ static cudaStream_t host_side_stream(cudaStream_t caller)
     return streams[dev][slot];
 }
 
+// Parts of a large batch in pinned buffers.  The last part is the smallest: its kernel and its results are what
+// nothing overlaps.  Where the kernels take longer than the transfers, parts only cost efficiency:
+// two halves keep the first transfer in and the last one out short.  Returns how many, their sizes in `size`.
+constexpr int kHostParts = 4;
+static int host_parts(const omni_mla_desc_t *desc, int *size)
+{
+    const int B = desc->batch;
+    size[0] = B;
+    // one part up to 3.5 MB of q and out (12 requests of 128 heads: 105 us either way, 20: 152 against 142)
+    if (!host_pipelined(desc) || (size_t)B * desc->num_heads * (kDqk + kDv) * 2 <= (size_t)(3584u << 10)) return 1;
+    const double tiles = (desc->max_sel + kTile - 1) / kTile;
+    const double kernel_us = 0.9 * B * tiles / 74, copy_us = (double)B * desc->num_heads * (kDqk * 2) / 50e3;
+    if (B < 8 || kernel_us > copy_us) {
+        size[0] = (B + 1) / 2;
+        size[1] = B - size[0];
+        return 2;
+    }
+    size[3] = B / 8;
+    size[2] = B / 4;
+    size[1] = (B - size[3] - size[2]) / 2;
+    size[0] = B - size[3] - size[2] - size[1];
+    return 4;
+}
+
+static size_t host_part_workspace(const omni_mla_desc_t *desc)
+{
+    int size[kHostParts];
+    const int n = host_parts(desc, size);
+    size_t need = 0;
+    for (int i = 0; i < n; ++i) {
+        omni_mla_desc_t d = *desc;
+        d.batch = size[i];
+        const size_t w = workspace_need(&d, choose_splits(&d, device_info().sm_count));
+        need = w > need ? w : need;
+    }
+    return align_up(need, 256);
+}
+
 size_t omni_sparse_mla_host_staging_bytes(const omni_mla_desc_t *desc)
 {
     if (!desc_ok(desc)) return 0;
     size_t n = host_copy_bytes(desc);
-    if (host_pipelined(desc)) n += host_half_workspace(desc, 0) + host_half_workspace(desc, 1);
+    if (host_pipelined(desc)) {
+        const size_t halves = host_half_workspace(desc, 0) + host_half_workspace(desc, 1), parts = host_part_workspace(desc);
+        n += halves > parts ? halves : parts;
+    }
     return n;
 }
+
+// Whether kernels can use a host buffer in place: pinned from its first to its last byte, at the same address
+// on the device, 16-byte aligned.
+static bool mapped_host(const void *p, size_t bytes)
+{
+    if (!aligned(p, 16)) return false;
+    const void *ends[2] = {p, static_cast<const char *>(p) + bytes - 1};
+    for (const void *e : ends) {
+        cudaPointerAttributes at = {};
+        if (cudaPointerGetAttributes(&at, e) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (at.type != cudaMemoryTypeHost || at.devicePointer != e) return false;
+    }
+    return true;
+}
+
+// Events that order a call's streams: one set per host thread and device.  A recorded event may be recorded
+// again while an earlier wait on it is still pending, so a set serves every call of its thread.
+struct HostEvents {
+    cudaEvent_t ev[64][2 * kHostParts + 1] = {};
+    ~HostEvents()
+    {
+        for (auto &device : ev)
+            for (cudaEvent_t e : device)
+                if (e) cudaEventDestroy(e);
+    }
+    cudaEvent_t *of(int dev)
+    {
+        if (dev < 0 || dev >= 64) return nullptr;
+        for (cudaEvent_t &e : ev[dev])
+            if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
+        return ev[dev];
+    }
+};
 
 omni_status_t omni_sparse_mla_decode_host(const omni_mla_desc_t *desc, const void *q_host,
                                           const void *kv_cache,
@@ -775,6 +864,75 @@ omni_status_t omni_sparse_mla_decode_host(const omni_mla_desc_t *desc, const voi
     };
 
     cudaStream_t side = host_pipelined(desc) ? host_side_stream(stream) : nullptr;
+    if (mapped_host(q_host, B * rq) && mapped_host(page_table_host, B * rpt) && mapped_host(sel_idx_host, B * rsi) &&
+        mapped_host(sel_len_host, B * rsl) && mapped_host(out_host, B * rout) && mapped_host(lse_host, B * rlse)) {
+        int size[kHostParts];
+        int parts = host_parts(desc, size), dev = -1;
+        static thread_local HostEvents pool;
+        cudaStream_t back = parts > 1 ? host_side_stream(stream, 1) : nullptr;
+        cudaEvent_t *ev = side && back && cudaGetDevice(&dev) == cudaSuccess ? pool.of(dev) : nullptr;
+        auto gather = [&](const GatherParts &g) {
+            size_t vectors = 0;
+            for (const GatherPart &a : g.part) vectors += a.bytes / 16;
+            const unsigned blocks = (unsigned)std::min<size_t>(16, vectors / (kGatherThreads * kGatherAhead) + 1);
+            return launch_overlapped(host_gather_kernel, blocks, kGatherThreads, stream, g);
+        };
+        if (!ev) {
+            const omni_status_t st =
+                gather({{{page_table_host, dpt, B * rpt}, {sel_idx_host, dsi, B * rsi}, {sel_len_host, dsl, B * rsl}, {q_host, dq, B * rq}}});
+            if (st != OMNI_OK) return st;
+            return omni_sparse_mla_decode(desc, dq, kv_cache, reinterpret_cast<int32_t *>(dpt), reinterpret_cast<int32_t *>(dsi),
+                                          reinterpret_cast<int32_t *>(dsl), out_host, lse_host, workspace, workspace_bytes,
+                                          device_status, stream);
+        }
+        // side:   q of part 0 | q of part 1 | ...
+        // caller: indices     | kernels 0   | kernels 1     | ... | join
+        // back:                             | out of part 0 | ...
+        cudaEvent_t *in_done = ev, *part_done = ev + kHostParts, start = ev[2 * kHostParts];
+        if (cudaEventRecord(start, stream) != cudaSuccess || cudaStreamWaitEvent(side, start, 0) != cudaSuccess) return OMNI_ERR_CUDA;
+        // indices of more than a megabyte or so come with the parts that use them
+        const bool indices_at_once = B * (rpt + rsi + rsl) <= (size_t)(1u << 20);
+        bool ok = true;
+        size_t b0 = 0;
+        for (int i = 0; i < parts; b0 += size[i], ++i) {
+            if (!indices_at_once) {
+                const size_t n = size[i];
+                ok = ok && h2d(dpt + b0 * rpt, reinterpret_cast<const char *>(page_table_host) + b0 * rpt, n * rpt, side) &&
+                     h2d(dsi + b0 * rsi, reinterpret_cast<const char *>(sel_idx_host) + b0 * rsi, n * rsi, side) &&
+                     h2d(dsl + b0 * rsl, reinterpret_cast<const char *>(sel_len_host) + b0 * rsl, n * rsl, side);
+            }
+            ok = ok && copy_q(b0, size[i], side);
+            ok = cudaEventRecord(in_done[i], side) == cudaSuccess && ok;
+        }
+        omni_status_t st = ok ? OMNI_OK : OMNI_ERR_CUDA;
+        if (st == OMNI_OK && indices_at_once)
+            st = gather({{{page_table_host, dpt, B * rpt}, {sel_idx_host, dsi, B * rsi}, {sel_len_host, dsl, B * rsl}, {nullptr, nullptr, 0}}});
+        const size_t part_ws = host_part_workspace(desc);
+        b0 = 0;
+        for (int i = 0; i < parts; b0 += size[i], ++i) {
+            // (after an error the waits still join the streams)
+            if (cudaStreamWaitEvent(stream, in_done[i], 0) != cudaSuccess) st = OMNI_ERR_CUDA;
+            if (st != OMNI_OK) continue;
+            omni_mla_desc_t d = *desc;
+            d.batch = size[i];
+            const bool last = i == parts - 1;
+            char *to = static_cast<char *>(out_host) + b0 * rout;
+            st = omni_sparse_mla_decode(&d, dq + b0 * rq, kv_cache, reinterpret_cast<int32_t *>(dpt + b0 * rpt),
+                                        reinterpret_cast<int32_t *>(dsi + b0 * rsi), reinterpret_cast<int32_t *>(dsl + b0 * rsl),
+                                        last ? to : dout + b0 * rout,
+                                        reinterpret_cast<float *>((last ? reinterpret_cast<char *>(lse_host) : dlse) + b0 * rlse), half_ws,
+                                        part_ws, device_status, stream);
+            if (st == OMNI_OK && !last &&
+                (cudaEventRecord(part_done[i], stream) != cudaSuccess || cudaStreamWaitEvent(back, part_done[i], 0) != cudaSuccess ||
+                 cudaMemcpyAsync(to, dout + b0 * rout, size[i] * rout, cudaMemcpyDeviceToHost, back) != cudaSuccess ||
+                 // (lse of all parts but the last in one copy)
+                 (i == parts - 2 && cudaMemcpyAsync(lse_host, dlse, (b0 + size[i]) * rlse, cudaMemcpyDeviceToHost, back) != cudaSuccess)))
+                st = OMNI_ERR_CUDA;
+        }
+        if (cudaEventRecord(start, back) != cudaSuccess || cudaStreamWaitEvent(stream, start, 0) != cudaSuccess)
+            st = st != OMNI_OK ? st : OMNI_ERR_CUDA;
+        return st;
+    }
     if (!side) {
         if (!copy_q(0, B, stream) || !copy_indices(stream)) return OMNI_ERR_CUDA;
         return decode_and_copy_out(*desc, 0, workspace, workspace_bytes, stream);
