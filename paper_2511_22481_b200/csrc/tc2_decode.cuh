@@ -3,40 +3,48 @@
 // A cluster of two CTAs owns all heads of one (request, split): CTA r serves heads
 // [64r, 64r+64).  The pair issues cta_group::2 MMAs with M = 128 (64 rows per CTA), which run
 // the tensor pipe of each SM at full rate where a lone M = 64 MMA runs it at half rate, and it
-// halves the operand bytes each SM must hold.  Per 64-token tile:
-//   S = Q K^T   M=128, N=64 tokens, K=576: every CTA supplies its 64 Q rows and the K rows of
-//               ITS 32 tokens of the tile ("K role": 32 tokens x 576 columns, 36 KiB)
-//   O += P V    M=128, N=256 per instruction (two of them), K=64 tokens: every CTA supplies its
-//               64 P rows and, for all 64 tokens, ITS 256 value columns ("V role": 64 tokens x
-//               256 columns, 32 KiB; CTA r holds columns [256r, 256r+256))
+// halves the operand bytes each SM must hold.  Per tile of 128 tokens, two units of 64:
+//   S = Q K^T   M=128, N=128 tokens, K=576: every CTA supplies its 64 Q rows and the K rows of
+//               ITS unit of the tile ("K role": 64 tokens x 576 columns, 72 KiB)
+//   O += P V    per unit: M=128, N=256 per instruction (two of them), K=64 tokens: every CTA
+//               supplies its 64 P rows and, for all 64 tokens, ITS 256 value columns ("V role":
+//               64 tokens x 256 columns, 32 KiB; CTA r holds columns [256r, 256r+256))
 // The two roles overlap only in a quarter of the tile, at different addresses in the two CTAs,
 // so each role is loaded on its own (1.9x the tile's bytes cross L2 -> shared memory, which L2
 // sustains; each byte leaves HBM once because the pair runs together).
 //
-// Both roles, P and S are double buffered, so the loads of tile i+2 are in flight while tile i
-// is consumed and Q K^T of tile i+1 overlaps the softmax of tile i.  Every refill is ONE 3-D TMA
-// box {64 columns, rows, panels}: the copy engine sustains only about 4 M instructions/s per SM,
-// so 8 KiB boxes cap an SM near 32 GB/s while 32-72 KiB boxes reach 90-150 GB/s.  Tiles that are
-// not 64 consecutive pool rows are gathered row by row with cp.async (see below).
+// What bounds it: a score MMA over N = 64 tokens is bound by its operand reads from shared memory (24
+// clocks for 16 clocks of math), over N = 128 by the math (32 clocks), so a tile of 128 tokens costs
+// the tensor core 2176 clocks where two of 64 cost 2750; and it reads 23 % fewer operand bytes,
+// which is power, and long runs are held back by the power limit.  From there on it is the refill of the
+// operands: there is room for one tile of K rows and one of V columns, about one HBM latency of
+// work, so each is refilled piece by piece as it is used up: K in three groups of three column panels,
+// V in its two units.  Where 64 pairs read 17 units each (32 requests x 33 units), HBM delivers at its rate
+// throughout the main loop, and what is left is the start and the end of a launch.  Against tiles
+// of 64 tokens with two whole stages, both measured in one call: 32 requests x 33 units 25.6 ->
+// 24.5 us, 64 x 33 43.2 -> 40.7, 128 x 64 156 -> 147, one request of 128 units 16.4 -> 15.7.
+//
+// The loads of a piece are requested as soon as its last reader retires, S is triple buffered, and
+// Q K^T runs up to two tiles ahead of P V.  Every piece is ONE 3-D TMA box {64 columns, 64 rows,
+// panels}: requesting one costs a warp 50 to 90 clocks.  Units that are not 64 consecutive pool rows
+// are gathered row by row with cp.async (see below).
 //
 // All MMAs are issued by warp 1 of CTA 0 in "whatever is ready" order: the whole warp runs the
 // loop with warp-uniform control flow and one elected lane issues each instruction (a lone
 // diverged thread cannot feed the tensor pipe: it needs ~110 clocks per MMA, the elected form
 // issues one every 25-64 clocks).  Completion is broadcast to both CTAs with multicast commits.
 //
-// Warps per CTA: 0 K-role producer, 1 MMA issuer (CTA 0 only) + tensor-memory owner,
-// 2-5 and 8-11 softmax / epilogue (two groups of four warps that take the tiles in turn: warps
-// 2-5 the even tiles, 8-11 the odd ones, 32 of a tile's 64 tokens per thread; all eight share
-// the epilogue), 6 V-role producer, 7 L2 prefetcher (CTA 0 only): shared memory holds
-// only two tiles, about one HBM latency of work, so each whole page is pulled into L2 one tile
-// before its K-role load and the shared-memory refills start from a line already on its way.
+// Warps per CTA: 0 K-role producer, 1 MMA issuer (CTA 0 only) + tensor-memory owner, 2-5 and 8-11
+// softmax / epilogue (a thread serves one head row and 32 of a tile's 128 tokens), 6 V-role
+// producer, 7 L2 prefetcher: the rows of each unit are pulled into L2 ahead of their K-role load, so
+// that the shared-memory refills start from a line already on its way.
 //
 // Tensor memory per CTA (a 64-row slice of an M=128 pair accumulator keeps columns [0, N/2) in
 // lanes 0-63 and columns [N/2, N) in lanes 64-127):
 //   columns   0..255  O: two N=256 accumulators; lane L, column x  <->  head row L%64,
 //                        value column 256*(L/64) + x
-//   columns 256..287  S buffer 0: lane L, column x <-> head row L%64, token 32*(L/64) + x
-//   columns 288..319, 320..351  S buffers 1, 2 (Q K^T runs two tiles ahead of P V)
+//   columns 256..319  S buffer 0: lane L, column x <-> head row L%64, token 64*(L/64) + x
+//   columns 320..383, 384..447  S buffers 1, 2
 //
 // Splits of a request are merged in one of three ways chosen by the host: inside a cluster of
 // two pairs (two splits, see cluster_merge_exchange), by a separate merge kernel over fp32
@@ -51,52 +59,51 @@
 
 namespace omni {
 
-constexpr int kC2Tile = 64;                              // tokens per tile of the pair
+constexpr int kC2Tile = 64;                              // tokens per unit: the granule of splits, index handling and P V
 constexpr int kC2Threads = 384;
-// Tiles the L2 prefetch runs ahead of the K-role loads.  Measured on B200: the further ahead, the
-// slower (1: 30.4 us, 5: 32.3 us, 12: 35.0 us per step on the batch-32 benchmark shape; the same
-// order at batch 128): a line prefetched long before its use is often gone again by then.
-constexpr int kPrefetchAhead = 1;
-constexpr int kC2KBytes = kPanels * 32 * 128;            // K role: 9 panels x [32 tokens x 128 B]
-constexpr int kC2KPanel = 32 * 128;
+// Units the L2 prefetch of scattered rows runs ahead of that of whole pages.  A page is prefetched when the K
+// loads of the tile in front of its own have been requested: a prefetch that competes with the loads of
+// an earlier tile delays them (requested one tile earlier 25.8 us per step of 32 requests x 33 units, just
+// before those loads 25.5, just after them 24.5).
+constexpr int kScatterAhead = 2;
+constexpr int kC2GroupPanels = 3;                        // K role: refilled in three groups of three panels
+constexpr int kC2Groups = kPanels / kC2GroupPanels;
+constexpr int kC2GroupBytes = kC2GroupPanels * kPanelBytes;   // [64 tokens x 128 B] x 3
 constexpr int kC2VBytes = 4 * kPanelBytes;               // V role: 4 panels x [64 tokens x 128 B]
 constexpr int kC2SmemQ = 0;                              // 9 panels x [64 heads x 128 B]
-constexpr int kC2SmemK = kC2SmemQ + kTileBytes;          // 2 stages
-constexpr int kC2SmemV = kC2SmemK + 2 * kC2KBytes;       // 2 stages
-constexpr int kC2SmemP = kC2SmemV + 2 * kC2VBytes;       // 2 buffers x [64 heads x 128 B]
+constexpr int kC2SmemK = kC2SmemQ + kTileBytes;          // 9 panels x [64 tokens x 128 B]
+constexpr int kC2SmemV = kC2SmemK + kTileBytes;          // 2 stages
+constexpr int kC2SmemP = kC2SmemV + 2 * kC2VBytes;       // 2 units x [64 heads x 128 B]
 constexpr int kC2SmemCtl = kC2SmemP + 2 * kPanelBytes;
 constexpr int kC2SmemCtlBytes = 3072;
 constexpr int kC2SmemBytes = kC2SmemCtl + kC2SmemCtlBytes;   // no alignment slack: the base is checked at run time
 constexpr uint32_t kC2ColS = 256;
-// Validity masks travel from the K producer to the softmax warps through a small ring.  The
-// producer writes the mask of tile i+1 once the score MMAs of tile i-2 have retired, and those
-// were issued only after every softmax warp had read the scores of tile i-5 (three score
-// buffers), i.e. after tile i-6 was finished: seven tiles can be live, so the ring holds eight.
-constexpr int kMaskRing = 8;
+// Validity masks travel from the K producer to the softmax warps through a small ring, in units.  The
+// producer resolves up to tile t + 2 once the score MMAs of tile t have retired.  Those were issued only
+// after every softmax warp had read the scores of tile t - 3 (three score buffers), i.e. after tile
+// t - 4 was finished: six tiles can be live, and the ring holds eight.
+constexpr int kMaskRing = 16;
 
 struct C2Control {
-    uint64_t q_full;
-    uint64_t k_full[2];
-    uint64_t k_empty[2];
+    uint64_t k_full[kC2Groups];          // per tile; those of the first tile wait for q's panels too
+    uint64_t k_empty[kC2Groups];
     uint64_t v_full[2];
     uint64_t s_full[3];
     uint64_t s_empty[3];
-    uint64_t p_full[2];
-    uint64_t pv_done[2];                 // P V of a tile retired: frees its V stage and its P buffer
+    uint64_t p_full;                     // both P units of a tile are written (and O rescaled)
+    uint64_t pv_done[2];                 // P V of a unit retired: frees its V stage and its P unit
     uint64_t x_bar;                      // all softmax threads: exchange of the final row sums
     uint64_t exit_bar;                   // both CTAs of the pair are done with tensor memory
-    uint64_t valid_mask[kMaskRing];      // per tile: validity of its 64 tokens
-    float xchg[2][4][64];                // row maxima: [group][2 * parity of the group's tile + token half][head row]; at the end the slots a group no longer uses carry its partial row sums
+    uint64_t valid_mask[kMaskRing];      // per unit: validity of its 64 tokens
+    float xchg[2][4][64];                // row maxima: [tile parity][quarter of the tile's tokens][head row]; at the end the parity no longer in use carries the partial row sums
     uint32_t tmem_base;
     uint32_t abort;
     uint32_t merge_flag;
     uint32_t xfail;                      // cluster merge: some wait of this CTA ran out (decided CTA-wide)
-    int32_t k_progress;                  // tiles whose K loads the producer has started (L2 prefetch pacing)
+    int32_t k_progress;                  // units whose K loads have been requested (L2 prefetch pacing)
     uint64_t recv_bar;                   // cluster merge: the partner's block has arrived
     uint64_t ready_bar;                  // cluster merge: the partner's main loop is over
-    uint64_t xg_bar[2];                  // row-maximum exchange inside either softmax group
-    uint64_t ref_bar;                    // the reference maxima after a tile are published (4 warps of its group)
-    float ref[2][64];                    // [tile parity][head row]: running reference maximum after that tile
+    uint64_t xg_bar;                     // row-maximum exchange of a tile
 };
 static_assert(sizeof(C2Control) <= kC2SmemCtlBytes, "control block too large");
 static_assert(kC2SmemBytes <= 232448, "shared memory budget");
@@ -128,6 +135,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 // epilogue to be acknowledged (about 9 us here).
 __device__ __forceinline__ void cluster_sync_relaxed()
 {
+    __syncwarp();                        // the aligned forms want whole warps
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
@@ -137,6 +145,7 @@ __device__ __forceinline__ void cluster_sync_relaxed()
 // written before it.
 __device__ __forceinline__ void cluster_sync_after_init()
 {
+    __syncwarp();                        // the aligned forms want whole warps
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -169,12 +178,13 @@ __device__ __forceinline__ void cp_async_wait()
 {
     asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
 }
-// All lanes: wait for this lane's copies of the stage (all but the `newer` most recent groups),
-// make them visible to the tensor core's proxy, then lane 0 credits `bytes` to the barrier.
-__device__ __noinline__ void retire_gathered_stage(uint32_t bar_cluster_addr, uint32_t bytes, bool newer_in_flight,
-                                                      int lane)
+// All lanes: wait for this lane's copies of the stage (all but the `newer` most recent groups of them, at
+// most two), make them visible to the tensor core's proxy, then lane 0 credits `bytes` to the barrier.
+__device__ __noinline__ void retire_gathered_stage(uint32_t bar_cluster_addr, uint32_t bytes, int newer, int lane)
 {
-    if (newer_in_flight)
+    if (newer >= 2)
+        cp_async_wait<2>();
+    else if (newer == 1)
         cp_async_wait<1>();
     else
         cp_async_wait<0>();
@@ -192,40 +202,29 @@ __device__ __noinline__ void retire_gathered_stage(uint32_t bar_cluster_addr, ui
     }
 }
 
-// The two gathers are kept out of line so that the producers' loops stay as small as they are
-// for selections that never need them.
-// K role: 32 rows x 9 panels; eight lanes per row, four rows per instruction; chunk c of row r
-// lands at chunk c ^ (r % 8) of its 128-byte line.
-__device__ __noinline__ void gather_k_rows(uint32_t dst, const char *kv_bytes, int own_row, int lane)
-{
-    const int ch = lane & 7;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        const int r = 4 * g + (lane >> 3);
-        const int src_row = __shfl_sync(0xffffffffu, own_row, r);
-        const char *src = kv_bytes + (size_t)src_row * (kDqk * 2) + ch * 16;
-        const uint32_t d = dst + r * 128 + ((ch ^ (r & 7)) << 4);
-#pragma unroll
-        for (int c = 0; c < kPanels; ++c) cp_async16(d + c * (32 * 128), src + c * 128);
-    }
-    cp_async_commit();
-}
-
-// V role: 64 rows x the four panels of this CTA's value columns (`kv_cols` points at the first).
-__device__ __noinline__ void gather_v_rows(uint32_t dst, const char *kv_cols, int row_lo, int row_hi, int lane)
+// Gathers 64 rows x kCount panels, `cols` pointing at the first panel of row 0: eight lanes per row, four rows
+// per instruction, chunk c of row r lands at chunk c ^ (r % 8) of its 128-byte line.  Kept out of
+// line so that the producers' loops stay as small as they are for selections that never need it.
+template <int kCount>
+__device__ __noinline__ void gather_rows(uint32_t dst, const char *cols, int row_lo, int row_hi, int lane)
 {
     const int ch = lane & 7;
 #pragma unroll
     for (int g = 0; g < 16; ++g) {
         const int r = 4 * g + (lane >> 3);
-        const int a = __shfl_sync(0xffffffffu, row_lo, r & 31), c2 = __shfl_sync(0xffffffffu, row_hi, r & 31);
-        const int src_row = r < 32 ? a : c2;
-        const char *src = kv_cols + (size_t)src_row * (kDqk * 2) + ch * 16;
+        const int src_row = __shfl_sync(0xffffffffu, g < 8 ? row_lo : row_hi, r & 31);
+        const char *src = cols + (size_t)src_row * (kDqk * 2) + ch * 16;
         const uint32_t d = dst + r * 128 + ((ch ^ (r & 7)) << 4);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) cp_async16(d + c * kPanelBytes, src + c * 128);
+        for (int c = 0; c < kCount; ++c) cp_async16(d + c * kPanelBytes, src + c * 128);
     }
     cp_async_commit();
+}
+
+// One cache row into L2.
+__device__ __forceinline__ void prefetch_row(const __nv_bfloat16 *kv, int row)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kv + (size_t)row * kDqk), "n"(kDqk * 2) : "memory");
 }
 
 // Pair MMA executed by a whole converged warp: one elected lane issues the instruction.  The
@@ -242,6 +241,21 @@ __device__ __forceinline__ void tc_mma_pair_elect(uint32_t d_tmem, uint32_t a_lo
         "elect.sync _|q, 0xffffffff;\n\t"
         "@q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(kAccumulate ? 1 : 0)
+        : "memory");
+}
+
+// The same with the accumulate flag as a run-time value.
+__device__ __forceinline__ void tc_mma_pair_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                                  uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -591,23 +605,22 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     // ---- set-up: barriers and tensor memory (nothing here touches global memory, so with a
     // programmatic dependent launch it overlaps the tail of the kernel before this one) --------
     if (threadIdx.x == 0) {
-        mbar_init(&ctl->q_full, 1);
-        // arrivals per tile on the pair's score / weight barriers: one per softmax warp that works on
-        // the tile, in either CTA (the four warps of the tile's group)
-        constexpr uint32_t kTileWarps = 8;
-        for (int i = 0; i < 2; ++i) {
+        // arrivals per tile on the pair's score / weight barriers: one per softmax warp, in either CTA
+        constexpr uint32_t kTileWarps = 16;
+        for (int i = 0; i < kC2Groups; ++i) {
             mbar_init(&ctl->k_full[i], 1);
             mbar_init(&ctl->k_empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
             mbar_init(&ctl->v_full[i], 1);
-            mbar_init(&ctl->p_full[i], kTileWarps);
             mbar_init(&ctl->pv_done[i], 1);
-            mbar_init(&ctl->xg_bar[i], 128);
         }
         for (int i = 0; i < 3; ++i) {
             mbar_init(&ctl->s_full[i], 1);
             mbar_init(&ctl->s_empty[i], kTileWarps);
         }
-        mbar_init(&ctl->ref_bar, 4);
+        mbar_init(&ctl->p_full, kTileWarps);
+        mbar_init(&ctl->xg_bar, 256);
         mbar_init(&ctl->x_bar, 256);
         mbar_init(&ctl->exit_bar, 2);
         mbar_init(&ctl->recv_bar, 1);
@@ -640,9 +653,9 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     const bool bad_len = selection.bad;
     int begin, end;
     split_range(n, p.splits, s, begin, end, kC2Tile);
-    const int tiles = (end - begin + kC2Tile - 1) / kC2Tile;
+    const int units = (end - begin + kC2Tile - 1) / kC2Tile, tiles = (units + 1) / 2;
 
-    const bool active = tiles > 0;
+    const bool active = units > 0;
     if (!active && bad_len && threadIdx.x == 0 && crank == 0) flag_status(p.status, OMNI_DEV_BAD_INDEX);
     if (!kClusterMerge && !active) {
         // empty split (the same decision in both CTAs of the pair): zeros and -inf, no pipeline
@@ -654,44 +667,62 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
 
     const int32_t *pt = p.page_table + (size_t)b * p.max_pages;
 
-    // Index pipeline of the producers.  Lane l serves tokens l and l+32 of a tile.  The three
-    // dependent steps (token position -> page id -> pool row) run in different loop iterations,
-    // one tile apart, so no load is consumed in the iteration that issued it.
+    // Index pipeline of the producers.  Lane l serves tokens l and l+32 of a unit.  The three
+    // dependent steps (token position -> page id -> pool row) run in different loop iterations, so no
+    // load is consumed in the iteration that issued it.  A lone warp takes 5-8 clocks an
+    // instruction and a producer has about 1100 clocks a unit, so the common unit (64 consecutive pool
+    // rows) is recognised with one vote and everything else is left to a slower path.
     struct TileIdx {
         int t0, t1;        // token positions (stage 1)
         int pg0, pg1;      // physical page ids, -1 if the position breaks the contract (stage 2)
     };
-    auto stage_tokens = [&](int tile, TileIdx &x) {
-        const int j0 = begin + tile * kC2Tile + lane, j1 = j0 + 32;
-        x.t0 = (tile < tiles && j0 < end) ? selection_at(selection, j0) : -1;
-        x.t1 = (tile < tiles && j1 < end) ? selection_at(selection, j1) : -1;
+    // positions from here on (as unsigned numbers: negative ones too) break the contract
+    const uint32_t t_limit = (uint32_t)min((int64_t)p.max_pages * kPage, (int64_t)1 << 31);
+    const uint32_t page_limit = (uint32_t)p.num_pages;
+    auto stage_tokens = [&](int unit, TileIdx &x) {
+        const int first = begin + unit * kC2Tile;
+        if (kRanges && first >= selection.vstart && first + kC2Tile <= end) {
+            // a unit inside the recent range: 64 consecutive positions of one page, rolled once for all
+            int t = selection.rs + (first - selection.vstart);
+            if ((t & (kPage - 1)) == 0) {
+                if (selection.ring_pages > 0) t = rolling_position(t, selection.sink_pages, selection.ring_pages);
+                x.t0 = t + lane;
+                x.t1 = t + lane + 32;
+                return;
+            }
+        }
+        const int j0 = first + lane, j1 = j0 + 32;
+        x.t0 = j0 < end ? selection_at(selection, j0) : -1;
+        x.t1 = j1 < end ? selection_at(selection, j1) : -1;
     };
     auto stage_pages = [&](TileIdx &x) {
-        x.pg0 = (x.t0 >= 0 && x.t0 / kPage < p.max_pages) ? ldg_index(pt + x.t0 / kPage, selection.keep) : -1;
-        x.pg1 = (x.t1 >= 0 && x.t1 / kPage < p.max_pages) ? ldg_index(pt + x.t1 / kPage, selection.keep) : -1;
+        x.pg0 = (uint32_t)x.t0 < t_limit ? ldg_index(pt + (x.t0 >> 6), selection.keep) : -1;
+        x.pg1 = (uint32_t)x.t1 < t_limit ? ldg_index(pt + (x.t1 >> 6), selection.keep) : -1;
     };
+    static_assert(kPage == 64, "positions are split by shifts");
     // row_lo / row_hi: pool rows of tokens lane and lane+32 (a masked token repeats the row of the
-    // tile's first valid token: real cache contents, multiplied by a weight of exactly zero);
-    // contig: all 64 tokens valid and in consecutive rows; contig_lo / contig_hi: the same per 32.
-    auto stage_rows = [&](int tile, const TileIdx &x, int &row_lo, int &row_hi, uint64_t &mask, bool &contig,
-                          bool &contig_lo, bool &contig_hi, bool &any_bad) {
-        const int j0 = begin + tile * kC2Tile + lane, j1 = j0 + 32;
-        const bool ok0 = x.pg0 >= 0 && (int64_t)x.pg0 < p.num_pages, ok1 = x.pg1 >= 0 && (int64_t)x.pg1 < p.num_pages;
+    // unit's first valid token: real cache contents, multiplied by a weight of exactly zero);
+    // contig: all 64 tokens valid and in consecutive rows.
+    auto stage_rows = [&](int unit, const TileIdx &x, int &row_lo, int &row_hi, uint64_t &mask, bool &contig,
+                          bool &any_bad) {
+        const bool ok0 = (uint32_t)x.pg0 < page_limit, ok1 = (uint32_t)x.pg1 < page_limit;
+        row_lo = x.pg0 * kPage + (x.t0 & (kPage - 1));
+        row_hi = x.pg1 * kPage + (x.t1 & (kPage - 1));
+        const int base = __shfl_sync(0xffffffffu, row_lo, 0);
+        contig = __all_sync(0xffffffffu, ok0 && ok1 && row_lo == base + lane && row_hi == base + 32 + lane);
+        mask = ~0ull;
+        if (contig) return;
+        const int j0 = begin + unit * kC2Tile + lane, j1 = j0 + 32;
         any_bad |= (j0 < end && !ok0 && !is_padding(selection, x.t0)) || (j1 < end && !ok1 && !is_padding(selection, x.t1));
-        const int r0 = ok0 ? x.pg0 * kPage + x.t0 % kPage : -1, r1 = ok1 ? x.pg1 * kPage + x.t1 % kPage : -1;
-        const uint32_t m0 = __ballot_sync(0xffffffffu, r0 >= 0), m1 = __ballot_sync(0xffffffffu, r1 >= 0);
+        const uint32_t m0 = __ballot_sync(0xffffffffu, ok0), m1 = __ballot_sync(0xffffffffu, ok1);
         mask = (uint64_t)m0 | ((uint64_t)m1 << 32);
         int stand_in = 0;
         if (m0)
-            stand_in = __shfl_sync(0xffffffffu, r0, __ffs(m0) - 1);
+            stand_in = __shfl_sync(0xffffffffu, row_lo, __ffs(m0) - 1);
         else if (m1)
-            stand_in = __shfl_sync(0xffffffffu, r1, __ffs(m1) - 1);
-        row_lo = r0 >= 0 ? r0 : stand_in;
-        row_hi = r1 >= 0 ? r1 : stand_in;
-        const int base_lo = __shfl_sync(0xffffffffu, row_lo, 0), base_hi = __shfl_sync(0xffffffffu, row_hi, 0);
-        contig_lo = __all_sync(0xffffffffu, r0 == base_lo + lane);
-        contig_hi = __all_sync(0xffffffffu, r1 == base_hi + lane);
-        contig = contig_lo && contig_hi && base_hi == base_lo + 32;
+            stand_in = __shfl_sync(0xffffffffu, row_hi, __ffs(m1) - 1);
+        row_lo = ok0 ? row_lo : stand_in;
+        row_hi = ok1 ? row_hi : stand_in;
     };
 
     // what the cluster merge needs from the softmax warps after the main loop
@@ -702,77 +733,105 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         // an empty split inside a merging cluster: no pipeline, but it takes part in the exchange
     } else if (warp == 0) {
         // =========================== K-role producer =====================================
-        // This CTA's K rows are tokens [32*rank, 32*rank+32) of every tile.
-        const uint32_t q_bar = map_to_rank(smem_u32(&ctl->q_full), leader);
+        // This CTA's K rows are unit 2 t + rank of every tile t, refilled in three groups of three panels as the
+        // score MMAs of the tile before retire.
+        const uint32_t k_full_leader = map_to_rank(smem_u32(&ctl->k_full[0]), leader);
         if (lane == 0) {
-            if (rank == 0) mbar_expect_tx(&ctl->q_full, 2 * kTileBytes);
-            // a CTA without heads (64 or fewer in all) takes zeros: the box starts past the last row
-            tma_box3d_pair(smem_base + kC2SmemQ, &q_map, q_bar, head_rows > 0 ? b * p.heads + h0 : p.batch * p.heads, 0);
+#pragma unroll
+            for (int g = 0; g < kC2Groups; ++g) {
+                // a CTA without heads (64 or fewer in all) takes zeros: the box starts past the last row
+                tma_box3d_pair(smem_base + kC2SmemQ + g * kC2GroupBytes, &q_map, k_full_leader + 8 * g,
+                               head_rows > 0 ? b * p.heads + h0 : p.batch * p.heads, g * kC2GroupPanels);
+            }
         }
         bool any_bad = bad_len;
-        TileIdx x1, x2;                      // one and two tiles ahead
-        int row_lo, row_hi;
-        uint64_t mask;
-        bool contig, contig_lo, contig_hi;
-        {
-            // the position loads of the first three tiles go out together, then the two page-id
-            // loads that depend on them: two cache misses in a row before the first copy, not four
-            TileIdx x0;
-            stage_tokens(0, x0);
-            stage_tokens(1, x1);
-            stage_tokens(2, x2);
-            stage_pages(x0);
-            stage_pages(x1);
-            stage_rows(0, x0, row_lo, row_hi, mask, contig, contig_lo, contig_hi, any_bad);
-        }
-        // The mask of a tile is published (store + fence) right after its rows are resolved and
-        // BEFORE the next index loads go out: a fence waits for the loads its thread has in
-        // flight, so a fence placed after them put their whole latency in front of every refill.
-        auto publish_mask = [&](int tile) {
-            if (lane == 0) {
-                ctl->valid_mask[tile % kMaskRing] = mask;
-                __threadfence_block();
+        // index pipeline, a tile (two units) at a time: page ids are one tile, positions two tiles ahead
+        TileIdx x1[2], x2[2];
+        int row_lo = 0, row_hi = 0;          // of this CTA's unit of the tile about to be loaded
+        bool contig = false;
+        // Resolves the rows of a tile and publishes the masks of its units (store + fence), BEFORE the next
+        // index loads go out: a fence waits for the loads its thread has in flight, so a fence placed
+        // after them put their whole latency in front of every refill.
+        auto resolve_tile = [&](int tile, const TileIdx (&x)[2]) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                int lo, hi;
+                uint64_t mask;
+                bool whole;
+                stage_rows(2 * tile + h, x[h], lo, hi, mask, whole, any_bad);
+                if (lane == 0) ctl->valid_mask[(2 * tile + h) % kMaskRing] = mask;
+                if (h == (int)rank) {
+                    row_lo = lo;
+                    row_hi = hi;
+                    contig = whole;
+                }
             }
+            if (lane == 0) __threadfence_block();
         };
-        publish_mask(0);
-        bool ok = true;
-        int pending = -1;                    // stage of a gathered tile whose bytes are not credited yet
-        const char *kv_bytes = reinterpret_cast<const char *>(p.kv);
-        for (int i = 0; ok && i < tiles; ++i) {
-            const int st = i & 1;
-            if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = i;
-            if (i >= 2) ok = mbar_wait(&ctl->k_empty[st], ((i >> 1) - 1) & 1);
-            ok = __all_sync(0xffffffffu, ok) && (*abort_flag == 0);
-            if (!ok) break;
-            const uint32_t bar = map_to_rank(smem_u32(&ctl->k_full[st]), leader);
-            if (lane == 0 && rank == 0) mbar_expect_tx(&ctl->k_full[st], 2 * kC2KBytes);
-            __syncwarp();
-            const uint32_t dst = smem_base + kC2SmemK + st * kC2KBytes;
-            const int own_row = rank ? row_hi : row_lo;
-            bool gathered = false;
-            if (rank ? contig_hi : contig_lo) {
-                if (lane == 0) tma_box3d_pair(dst, &kv_k_map, bar, own_row, 0);
-            } else {
-                // scattered rows: eight lanes per row, four rows per instruction, chunk c of row r
-                // lands at chunk c ^ (r % 8) of its 128-byte line
-                gathered = true;
-                gather_k_rows(dst, kv_bytes, own_row, lane);
+        {
+            // the position loads of the first three tiles go out together, then the page-id loads that
+            // depend on them: two cache misses in a row before the first copy, not four
+            TileIdx x0[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                stage_tokens(h, x0[h]);
+                stage_tokens(2 + h, x1[h]);
+                stage_tokens(4 + h, x2[h]);
             }
-            if (pending >= 0) {
-                retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kC2KBytes, gathered, lane);
-                pending = -1;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                stage_pages(x0[h]);
+                stage_pages(x1[h]);
             }
-            if (gathered) pending = st;
-            // advance the index pipeline: rows of tile i+1, page ids of tile i+2, positions of tile i+3
-            if (i + 1 < tiles) {
-                stage_rows(i + 1, x1, row_lo, row_hi, mask, contig, contig_lo, contig_hi, any_bad);
-                publish_mask(i + 1);
-            }
-            x1 = x2;
-            stage_pages(x1);
-            stage_tokens(i + 3, x2);
+            resolve_tile(0, x0);
         }
-        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kC2KBytes, false, lane);
+        bool ok = true;
+        // gathered groups whose bytes are not credited yet, first in first out: a single scattered group takes
+        // about a memory latency, so all three are requested before the first is waited for
+        int waiting = 0, oldest = 0;
+        auto credit_oldest = [&]() {
+            retire_gathered_stage(k_full_leader + 8 * oldest, kC2GroupBytes, --waiting, lane);
+            oldest = oldest == kC2Groups - 1 ? 0 : oldest + 1;
+        };
+        const char *kv_bytes = reinterpret_cast<const char *>(p.kv);
+        for (int tile = 0; ok && tile < tiles; ++tile) {
+            // the last tile has a single unit when their number is odd: CTA 1 then leaves its half of the K
+            // rows as it is (the scores of those tokens are masked)
+            const bool mine = 2 * tile + (int)rank < units;
+            const uint32_t bytes = (2 * tile + 1 < units ? 2 : 1) * kC2GroupBytes + (tile == 0 ? 2 * kC2GroupBytes : 0);
+#pragma unroll 1
+            for (int g = 0; g < kC2Groups; ++g) {
+                if (tile > 0) {
+                    // nothing to do until the group is free: credit what has landed meanwhile
+                    while (waiting > 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->k_empty[g], (tile - 1) & 1))) credit_oldest();
+                    ok = __all_sync(0xffffffffu, mbar_wait(&ctl->k_empty[g], (tile - 1) & 1));
+                    if (!ok) break;
+                }
+                if (lane == 0 && rank == 0) mbar_expect_tx(&ctl->k_full[g], bytes);
+                if (!mine) continue;
+                const uint32_t dst = smem_base + kC2SmemK + g * kC2GroupBytes;
+                if (contig) {
+                    if (lane == 0) tma_box3d_pair(dst, &kv_k_map, k_full_leader + 8 * g, row_lo, g * kC2GroupPanels);
+                } else {
+                    gather_rows<kC2GroupPanels>(dst, kv_bytes + g * (kC2GroupPanels * 128), row_lo, row_hi, lane);
+                    if (waiting++ == 0) oldest = g;
+                }
+            }
+            if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = 2 * tile + 2;
+            // (before the index work: that fits into the time the score MMAs then take)
+            while (waiting > 0) credit_oldest();
+            ok = ok && (*abort_flag == 0);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            // advance the index pipeline: rows of the next tile, page ids of the one after, positions of the third
+            if (tile + 1 < tiles) resolve_tile(tile + 1, x1);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                x1[h] = x2[h];
+                stage_pages(x1[h]);
+                stage_tokens(2 * tile + 6 + h, x2[h]);
+            }
+        }
         if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = 0x7fffffff;
         if (!ok && lane == 0) {
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_PRODUCER_K);
@@ -786,9 +845,9 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         TileIdx x1, x2;
         int row_lo, row_hi;
         uint64_t mask_unused;
-        bool contig, contig_lo, contig_hi;
+        bool contig;
         {
-            // the position loads of the first three tiles go out together, then the two page-id
+            // the position loads of the first three units go out together, then the two page-id
             // loads that depend on them: two cache misses in a row before the first copy, not four
             TileIdx x0;
             stage_tokens(0, x0);
@@ -796,14 +855,20 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             stage_tokens(2, x2);
             stage_pages(x0);
             stage_pages(x1);
-            stage_rows(0, x0, row_lo, row_hi, mask_unused, contig, contig_lo, contig_hi, any_bad);
+            stage_rows(0, x0, row_lo, row_hi, mask_unused, contig, any_bad);
         }
         bool ok = true;
-        int pending = -1;                    // stage of a gathered tile whose bytes are not credited yet
+        int pending = -1;                    // stage of a gathered unit whose bytes are not credited yet
         const char *kv_bytes = reinterpret_cast<const char *>(p.kv);
-        for (int i = 0; ok && i < tiles; ++i) {
+        for (int i = 0; ok && i < units; ++i) {
             const int st = i & 1;
-            if (i >= 2) ok = mbar_wait(&ctl->pv_done[st], ((i >> 1) - 1) & 1);
+            if (i >= 2) {
+                if (pending >= 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->pv_done[st], ((i >> 1) - 1) & 1))) {
+                    retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, 0, lane);
+                    pending = -1;
+                }
+                ok = mbar_wait(&ctl->pv_done[st], ((i >> 1) - 1) & 1);
+            }
             ok = __all_sync(0xffffffffu, ok) && (*abort_flag == 0);
             if (!ok) break;
             const uint32_t bar = map_to_rank(smem_u32(&ctl->v_full[st]), leader);
@@ -816,69 +881,84 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             } else {
                 // scattered rows: the four panels of this CTA's value columns, 64 tokens
                 gathered = true;
-                gather_v_rows(dst, kv_bytes + (int)rank * 512, row_lo, row_hi, lane);
+                gather_rows<4>(dst, kv_bytes + (int)rank * 512, row_lo, row_hi, lane);
             }
             if (pending >= 0) {
-                retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, gathered, lane);
+                retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, gathered ? 1 : 0, lane);
                 pending = -1;
             }
-            if (gathered) pending = st;
-            if (i + 1 < tiles) stage_rows(i + 1, x1, row_lo, row_hi, mask_unused, contig, contig_lo, contig_hi, any_bad);
+            if (gathered) {
+                pending = st;
+                // the next stage is still in use: credit this one before the index work
+                if (i >= 1 && !__all_sync(0xffffffffu, mbar_test(&ctl->pv_done[st ^ 1], (((i + 1) >> 1) - 1) & 1))) {
+                    retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, 0, lane);
+                    pending = -1;
+                }
+            }
+            if (i + 1 < units) stage_rows(i + 1, x1, row_lo, row_hi, mask_unused, contig, any_bad);
             x1 = x2;
             stage_pages(x1);
             stage_tokens(i + 3, x2);
         }
-        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, false, lane);
+        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, 0, lane);
         if (!ok && lane == 0) {
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_PRODUCER_V);
             *abort_flag = 1;
         }
     } else if (warp == 7) {
-        // =========================== L2 prefetcher (CTA 0 only) ==========================
-        // A hint only: tiles that look like a whole page in order (first position page-aligned,
-        // last position 63 further) get their page prefetched into L2; anything else is left to
-        // the demand loads.  Lane l resolves tiles l, l+32, ... of a batch of 32 in parallel.
-        if (rank == 0) {
-            for (int t0 = 0; t0 < tiles; t0 += 32) {
-                const int t = t0 + lane;
-                const int j0 = begin + t * kC2Tile;
-                int row = -1;
-                if (t < tiles && j0 + kC2Tile <= end) {
-                    const int first = selection_at(selection, j0), last = selection_at(selection, j0 + kC2Tile - 1);
-                    if (first >= 0 && first % kPage == 0 && last == first + kC2Tile - 1 && first / kPage < p.max_pages) {
-                        const int pg = ldg_index(pt + first / kPage, selection.keep);
-                        if (pg >= 0 && (int64_t)pg < p.num_pages) row = pg * kPage;
-                    }
+        // =========================== L2 prefetcher =======================================
+        // A hint only.  CTA r pulls the units that are ITS K rows into L2 ahead of their loads: a whole page in
+        // order (first position page-aligned, last position 63 further) by one tensor prefetch, anything
+        // else row by row.  Lane l looks at the ends of unit r + 2 l, ... of a batch of 32 in parallel.
+        for (int t0 = (int)rank; t0 < units; t0 += 64) {
+            const int t = t0 + 2 * lane;
+            const int j0 = begin + t * kC2Tile;
+            int row = -1;
+            if (t < units && j0 + kC2Tile <= end) {
+                const int first = selection_at(selection, j0), last = selection_at(selection, j0 + kC2Tile - 1);
+                if (first >= 0 && first % kPage == 0 && last == first + kC2Tile - 1 && first / kPage < p.max_pages) {
+                    const int pg = ldg_index(pt + first / kPage, selection.keep);
+                    if (pg >= 0 && (int64_t)pg < p.num_pages) row = pg * kPage;
                 }
-                const int count = min(32, tiles - t0);
-                bool ok = true;
-                // nothing to pace out where no tile of the batch is a whole page (token-level selections)
-                if (!__any_sync(0xffffffffu, row >= 0)) continue;
-                for (int k = 0; ok && k < count; ++k) {
-                    // tile i is prefetched once the K loads of tile i - kPrefetchAhead have started (a
-                    // monotonic counter, polled with a bounded number of naps)
-                    const int i = t0 + k;
-                    const volatile int32_t *progress = &ctl->k_progress;
-                    for (int naps = 0; *progress < i - kPrefetchAhead && *abort_flag == 0; ++naps) {
-                        if (naps > (1 << 22)) {
-                            ok = false;
-                            break;
-                        }
-                        __nanosleep(200);
-                    }
-                    ok = ok && (*abort_flag == 0);
-                    if (ok && lane == k && row >= 0)
-                        asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(&kv_tile_map),
-                                     "r"(0), "r"(row), "r"(0)
-                                     : "memory");
-                }
-                if (!ok) break;
             }
+            __syncwarp();
+            bool ok = true;
+            TileIdx x = {-1, -1, -1, -1};    // of a unit that is not a whole page
+            for (int k = 0; ok && k < 32 && t0 + 2 * k < units; ++k) {
+                const int i = t0 + 2 * k;
+                const bool page = __shfl_sync(0xffffffffu, row, k) >= 0;
+                if (!page) {
+                    stage_tokens(i, x);
+                    stage_pages(x);
+                }
+                // a page is prefetched once the K loads of the tile before have been requested (a monotonic
+                // counter, polled with a bounded number of naps)
+                const volatile int32_t *progress = &ctl->k_progress;
+                for (int naps = 0; *progress < i - (int)rank - (page ? 0 : kScatterAhead) && *abort_flag == 0; ++naps) {
+                    if (naps > (1 << 22)) {
+                        ok = false;
+                        break;
+                    }
+                    __nanosleep(200);
+                }
+                ok = ok && (*abort_flag == 0);
+                ok = __all_sync(0xffffffffu, ok);
+                if (ok && page && lane == k)
+                    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(&kv_tile_map),
+                                 "r"(0), "r"(row), "r"(0)
+                                 : "memory");
+                if (ok && !page && *progress <= i) {      // (not once the unit's own loads are out)
+                    if ((uint32_t)x.pg0 < page_limit) prefetch_row(p.kv, x.pg0 * kPage + (x.t0 & (kPage - 1)));
+                    if ((uint32_t)x.pg1 < page_limit) prefetch_row(p.kv, x.pg1 * kPage + (x.t1 & (kPage - 1)));
+                }
+                __syncwarp();
+            }
+            if (!ok) break;
         }
     } else if (warp == 1) {
         // =========================== MMA issuer (CTA 0 only) =============================
         if (rank == 0) {
-            constexpr uint32_t idesc_qk = instr_desc(128, kC2Tile, 0);
+            constexpr uint32_t idesc_qk = instr_desc(128, 2 * kC2Tile, 0);
             constexpr uint32_t idesc_pv = instr_desc(128, 256, 1);
             const uint64_t q_desc = smem_desc(smem_base + kC2SmemQ, 16, 1024);
             const uint64_t k_desc = smem_desc(smem_base + kC2SmemK, 16, 1024);
@@ -889,34 +969,29 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             // Values that steer the loop are broadcast from lane 0 so that the compiler can see
             // they are warp-uniform and keep the descriptor arithmetic on the uniform datapath;
             // with thread-dependent control flow every MMA costs ~70 clocks to issue instead of ~25.
-            const int tiles_u = __shfl_sync(0xffffffffu, tiles, 0);
+            const int tiles_u = __shfl_sync(0xffffffffu, tiles, 0), units_u = __shfl_sync(0xffffffffu, units, 0);
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
-            // One copy of each issue routine: stage and buffer enter as warp-uniform run-time values
+            // One copy of each issue routine: group, stage and buffer enter as warp-uniform run-time values
             // (every operand of an MMA is then a uniform base plus a compile-time offset), which
             // keeps the issuing warp's code a few kilobytes instead of several tens (an issue loop
             // unrolled over the buffer parities ran config-2-sized launches 5 % slower, token-level
             // ones 8 %: a launch starts with cold instruction caches and this loop is its critical path).
-            auto issue_qk = [&](int kpar, int sbuf) {
-                const uint32_t d = tmem_u + kC2ColS + 32 * sbuf;
-                const uint32_t kb = k_lo + ((kpar * kC2KBytes) >> 4);
-                tc_mma_pair_elect<false>(d, q_lo, kmaj_hi, kb, kmaj_hi, idesc_qk);
+            auto issue_qk = [&](int g, int sbuf) {
+                const uint32_t d = tmem_u + kC2ColS + 64 * sbuf, at = (uint32_t)((g * kC2GroupBytes) >> 4);
+                tc_mma_pair_elect(d, q_lo + at, kmaj_hi, k_lo + at, kmaj_hi, idesc_qk, g != 0 ? 1u : 0u);
 #pragma unroll
-                for (int kk = 1; kk < kDqk / 16; ++kk)
-                    tc_mma_pair_elect<true>(d, q_lo + (((kk >> 2) * kPanelBytes + (kk & 3) * 32) >> 4), kmaj_hi,
-                                            kb + (((kk >> 2) * kC2KPanel + (kk & 3) * 32) >> 4), kmaj_hi, idesc_qk);
-                tc_commit_pair_elect(&ctl->k_empty[kpar], pair_mask);
-                tc_commit_pair_elect(&ctl->s_full[sbuf], pair_mask);
+                for (int kk = 1; kk < 4 * kC2GroupPanels; ++kk) {
+                    const uint32_t off = at + (((kk >> 2) * kPanelBytes + (kk & 3) * 32) >> 4);
+                    tc_mma_pair_elect<true>(d, q_lo + off, kmaj_hi, k_lo + off, kmaj_hi, idesc_qk);
+                }
+                tc_commit_pair_elect(&ctl->k_empty[g], pair_mask);
+                if (g == kC2Groups - 1) tc_commit_pair_elect(&ctl->s_full[sbuf], pair_mask);
             };
             auto issue_pv = [&](int par, bool first) {
                 const uint32_t a = p_lo + ((par * kPanelBytes) >> 4);
                 const uint32_t bd = v_lo + ((par * kC2VBytes) >> 4);
-                if (first) {
-                    tc_mma_pair_elect<false>(tmem_u + kColO, a, kmaj_hi, bd, v_hi, idesc_pv);
-                    tc_mma_pair_elect<false>(tmem_u + kColO + 128, a, kmaj_hi, bd + ((2 * kPanelBytes) >> 4), v_hi, idesc_pv);
-                } else {
-                    tc_mma_pair_elect<true>(tmem_u + kColO, a, kmaj_hi, bd, v_hi, idesc_pv);
-                    tc_mma_pair_elect<true>(tmem_u + kColO + 128, a, kmaj_hi, bd + ((2 * kPanelBytes) >> 4), v_hi, idesc_pv);
-                }
+                tc_mma_pair_elect(tmem_u + kColO, a, kmaj_hi, bd, v_hi, idesc_pv, first ? 0u : 1u);
+                tc_mma_pair_elect(tmem_u + kColO + 128, a, kmaj_hi, bd + ((2 * kPanelBytes) >> 4), v_hi, idesc_pv, first ? 0u : 1u);
 #pragma unroll
                 for (int k = 1; k < 4; ++k) {
                     const uint32_t ak = a + ((k * 32) >> 4), bk = bd + ((k * 2048) >> 4);
@@ -925,45 +1000,46 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 }
                 tc_commit_pair_elect(&ctl->pv_done[par], pair_mask);
             };
-            // S(t) lives in buffer t % 3, K(t) in stage t & 1; Q K^T runs two tiles ahead of P V
-            auto qk_tile = [&](int t) -> bool {
-                const int kpar = t & 1, sbuf = t % 3;
-                bool good = mbar_wait(&ctl->k_full[kpar], (t >> 1) & 1) &&
-                            (t < 3 || mbar_wait(&ctl->s_empty[sbuf], ((t / 3) - 1) & 1));
-                good = __all_sync(0xffffffffu, good);
-                if (!good) return false;
-                tc_fence_after();
-                issue_qk(kpar, sbuf);
-                return true;
-            };
-            auto pv_tile = [&](int i) -> bool {
-                const int par = i & 1;
-                bool good = mbar_wait(&ctl->p_full[par], (i >> 1) & 1) && mbar_wait(&ctl->v_full[par], (i >> 1) & 1);
-                good = __all_sync(0xffffffffu, good);
-                if (!good) return false;
-                tc_fence_after();
-                issue_pv(par, i == 0);
-                return true;
-            };
-            bool ok = mbar_wait(&ctl->q_full, 0);
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok) ok = qk_tile(0);
-            if (ok && tiles_u > 1) ok = qk_tile(1);
-            for (int i = 0; ok && i < tiles_u; ++i) {
-                // if the K rows of tile i+2 have not landed yet while P and V of tile i are ready, P V goes first
-                bool qk_todo = i + 2 < tiles_u;
-                if (qk_todo) {
-                    const int kpar = i & 1;
-                    const bool k_ready = __all_sync(0xffffffffu, mbar_test(&ctl->k_full[kpar], ((i + 2) >> 1) & 1));
-                    const bool pv_ready = __all_sync(0xffffffffu, mbar_test(&ctl->p_full[kpar], (i >> 1) & 1) &&
-                                                                      mbar_test(&ctl->v_full[kpar], (i >> 1) & 1));
-                    if (k_ready || !pv_ready) {
-                        ok = qk_tile(i + 2);
-                        qk_todo = false;
+            // Whatever is ready goes next, scores first (P V first was 1 to 5 % slower): group g of tile t once its
+            // K panels have landed and (first group) the score buffer t % 3 is free; P V of unit u once the
+            // weights of its tile are written and its V rows have landed.
+            bool ok = true;
+            int t = 0, g = 0, u = 0, sbuf = 0, sph = 1;     // sph: parity of the wait on s_empty (the first use passes at once)
+            long long start = 0;
+            uint32_t idle = 0;
+            while (ok && u < units_u) {
+                const bool qk = t < tiles_u && mbar_test(&ctl->k_full[g], t & 1) && (g > 0 || mbar_test(&ctl->s_empty[sbuf], sph));
+                if (__all_sync(0xffffffffu, qk)) {
+                    tc_fence_after();
+                    issue_qk(g, sbuf);
+                    if (++g == kC2Groups) {
+                        g = 0;
+                        ++t;
+                        if (++sbuf == 3) {
+                            sbuf = 0;
+                            sph ^= 1;
+                        }
                     }
+                    idle = 0;
+                    continue;
                 }
-                if (ok) ok = pv_tile(i);
-                if (ok && qk_todo) ok = qk_tile(i + 2);
+                const bool pv = mbar_test(&ctl->p_full, (u >> 1) & 1) && mbar_test(&ctl->v_full[u & 1], (u >> 1) & 1);
+                if (__all_sync(0xffffffffu, pv)) {
+                    tc_fence_after();
+                    issue_pv(u & 1, u == 0);
+                    ++u;
+                    idle = 0;
+                    continue;
+                }
+                // bounded: the clock is read now and then while nothing is ready
+                if ((++idle & 63u) == 0u) {
+                    const long long now = __shfl_sync(0xffffffffu, clock64(), 0);
+                    if (idle == 64u)
+                        start = now;
+                    else
+                        ok = now - start <= kWaitCycles;
+                    ok = ok && __shfl_sync(0xffffffffu, *abort_flag, 0) == 0u;
+                }
             }
             if (!ok && lane == 0) {
                 flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_MMA);
@@ -973,8 +1049,8 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         __syncwarp();
     } else {
         // =========================== softmax + epilogue =================================
-        // Eight warps (2-5 and 8-11): two per tensor-memory lane quarter, one in each of two groups
-        // (sub = 0 for warps 2-5, 1 for warps 8-11).  A thread serves head row L % 64 (L = its
+        // Eight warps (2-5 and 8-11): two per tensor-memory lane quarter (sub = 0 for warps 2-5, 1 for warps
+        // 8-11).  A thread serves head row L % 64 (L = its
         // tensor-memory lane); in the epilogue it owns value columns 256 * (L / 64) + 128 * sub +
         // [0, 128) of that row.
         const int quarter = warp & 3;
@@ -983,19 +1059,18 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         const int half = quarter >> 1;                      // token half of S / column half of O
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         const uint32_t s_empty_leader = map_to_rank(smem_u32(&ctl->s_empty[0]), leader);   // [1], [2] follow at +8, +16
-        const uint32_t p_full_leader0 = map_to_rank(smem_u32(&ctl->p_full[0]), leader);
-        const uint32_t p_full_leader1 = map_to_rank(smem_u32(&ctl->p_full[1]), leader);
+        const uint32_t p_full_leader = map_to_rank(smem_u32(&ctl->p_full), leader);
         float m_ref = -INFINITY, l = 0.f;
         bool ok = true;
-        // Tiles alternate between two groups of four warps (2-5: even tiles, 8-11: odd tiles), so
-        // the chain scores -> weights of one tile overlaps the next tile's instead of all eight warps
-        // marching through every tile together.  In its group a thread serves head row `row` and
-        // the token half `half` of the tile (32 tokens, all 32 score columns of its lane).  The
-        // running reference maximum of a row is shared by the groups through ctl->ref: tile i reads
-        // what tile i-1 left and publishes its own decision at once, before its exponentials.
-        const int grp = sub;
-        for (int i = grp; ok && i < tiles; i += 2) {
-            const int sbuf = i % 3, it = i >> 1;
+        // Every tile is worked on by all eight warps: a thread serves head row `row` and 32 of the 128 tokens,
+        // [64 half + 32 sub, + 32), and the four threads of a row meet over its maximum through shared
+        // memory.  (Two groups of four warps that take the tiles in turn, 64 tokens a thread, overlap one
+        // tile's exchange with the other's exponentials, but the weights of a tile are then ready about 450
+        // clocks later, which every launch pays at its first and at its last tile: one request of 128
+        // units 16.8 us that way, 16.2 this way.)
+        const int tq = half * 2 + sub;                     // quarter of the tile's tokens
+        for (int i = 0; i < tiles; ++i) {
+            const int sbuf = i % 3;
             ok = mbar_wait(&ctl->s_full[sbuf], (i / 3) & 1);
             if (!__all_sync(0xffffffffu, ok)) {
                 ok = false;
@@ -1003,154 +1078,110 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             }
             tc_fence_after();
             uint32_t sv[32];
-            tc_ld32(tmem + lane_base + kC2ColS + 32 * sbuf, sv);
+            tc_ld32(tmem + lane_base + kC2ColS + 64 * sbuf + 32 * sub, sv);
             tc_wait_ld();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(s_empty_leader + 8 * sbuf);
-            const uint32_t valid = (uint32_t)(ctl->valid_mask[i % kMaskRing] >> (32 * half));
-            // x[j] * xs is the scaled score of token j.  A full tile under a positive scale keeps the
-            // raw scores (xs = the scale): the maximum is taken on them and the scale rides on the
-            // fused multiply-add in front of the exponential, one instruction less per token.
-            float x[32];
-            float mt = -INFINITY;
-            float xs = 1.f;
-            if (valid == 0xffffffffu && p.scale_log2 > 0.f) {
+            const uint32_t valid = (uint32_t)(ctl->valid_mask[(2 * i + half) % kMaskRing] >> (32 * sub));
+            // x * xs is the scaled score of a token.  Under a positive scale x is the raw score: the
+            // maximum is taken on them and the scale rides on the fused multiply-add in front of the
+            // exponential, one instruction less per token.
+            float xs = p.scale_log2;
+            if (!(p.scale_log2 > 0.f)) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    x[j] = __uint_as_float(sv[j]);
-                    mt = fmaxf(mt, x[j]);
-                }
-                xs = p.scale_log2;
-                mt *= xs;
-            } else if (valid == 0xffffffffu) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    x[j] = __uint_as_float(sv[j]) * p.scale_log2;
-                    mt = fmaxf(mt, x[j]);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    x[j] = ((valid >> j) & 1u) ? __uint_as_float(sv[j]) * p.scale_log2 : -INFINITY;
-                    mt = fmaxf(mt, x[j]);
-                }
+                for (int j = 0; j < 32; ++j) sv[j] = __float_as_uint(__uint_as_float(sv[j]) * p.scale_log2);
+                xs = 1.f;
             }
-            // the row's other half is served by the thread of the same lane two warps on
-            float *xg = &ctl->xchg[0][0][0] + ((grp * 2 + (it & 1)) * 2) * 64;      // [group][parity][half][row]
-            xg[half * 64 + row] = mt;
-            mbar_arrive(&ctl->xg_bar[grp]);
-            ok = mbar_wait(&ctl->xg_bar[grp], it & 1);
-            if (i > 0) ok = ok && mbar_wait(&ctl->ref_bar, (i - 1) & 1);
+            if (valid != 0xffffffffu) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (!((valid >> j) & 1u)) sv[j] = __float_as_uint(-INFINITY);
+            }
+            float mt4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int j = 0; j < 32; ++j) mt4[j & 3] = fmaxf(mt4[j & 3], __uint_as_float(sv[j]));
+            float mt = fmaxf(fmaxf(mt4[0], mt4[1]), fmaxf(mt4[2], mt4[3])) * xs;
+            float *xg = &ctl->xchg[i & 1][0][row];
+            xg[tq * 64] = mt;
+            mbar_arrive(&ctl->xg_bar);
+            ok = mbar_wait(&ctl->xg_bar, i & 1);
             if (!__all_sync(0xffffffffu, ok)) {
                 ok = false;
                 break;
             }
-            mt = fmaxf(mt, xg[(half ^ 1) * 64 + row]);
-            const float ref_in = i > 0 ? ctl->ref[(i - 1) & 1][row] : -INFINITY;
+            mt = fmaxf(fmaxf(xg[0], xg[64]), fmaxf(xg[128], xg[192]));
             // move the reference only when the tile maximum leaves the window above it
-            float ref_out = ref_in;
+            float factor = 1.f;
             bool moved = false;
-            if (mt > ref_in + kRescaleThreshold || (ref_in == -INFINITY && mt > -INFINITY)) {
-                ref_out = mt;
+            if (mt > m_ref + kRescaleThreshold || (m_ref == -INFINITY && mt > -INFINITY)) {
+                factor = m_ref == -INFINITY ? 0.f : exp2f(m_ref - mt);
+                m_ref = mt;
                 moved = true;
             }
-            if (half == 0) ctl->ref[i & 1][row] = ref_out;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&ctl->ref_bar);
-            // this thread's own sum was last brought to reference m_ref
-            if (ref_out != m_ref) {
-                l *= (m_ref == -INFINITY) ? 0.f : exp2f(m_ref - ref_out);
-                m_ref = ref_out;
-            }
             const float mr = (m_ref == -INFINITY) ? 0.f : m_ref;
-            float sum = 0.f;
+            float sum[2] = {0.f, 0.f};
             uint32_t pk[16];
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
-                const float e0 = fast_exp2(fmaf(x[j], xs, -mr)), e1 = fast_exp2(fmaf(x[j + 1], xs, -mr));
-                sum += e0 + e1;
+                const float e0 = fast_exp2(fmaf(__uint_as_float(sv[j]), xs, -mr));
+                const float e1 = fast_exp2(fmaf(__uint_as_float(sv[j + 1]), xs, -mr));
+                sum[0] += e0;
+                sum[1] += e1;
                 pk[j >> 1] = pack_bf16(e0, e1);
             }
-            l += sum;
-            // this group's P buffer is free once P V of tile i-2 retired; O may be rescaled once P V of tile i-1 did
-            if (i >= 2) {
-                ok = mbar_wait(&ctl->pv_done[grp], ((i >> 1) - 1) & 1);
+            l = l * factor + (sum[0] + sum[1]);
+            // P and O are free once P V of the tile before (its second unit: only the last tile can have a
+            // single one) retired
+            if (i >= 1) {
+                ok = mbar_wait(&ctl->pv_done[1], (i - 1) & 1);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
                     break;
                 }
-            }
-            if (i >= 1 && __any_sync(0xffffffffu, moved)) {
-                ok = mbar_wait(&ctl->pv_done[grp ^ 1], ((i - 1) >> 1) & 1);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                // the four warps of the group cover all 128 lanes: each thread rescales the 256 value columns of its lane
-                const float factor = moved ? ((ref_in == -INFINITY) ? 0.f : exp2f(ref_in - ref_out)) : 1.f;
+                if (__any_sync(0xffffffffu, moved)) {
+                    tc_fence_after();
 #pragma unroll 1
-                for (int c = 0; c < 256; c += 32) {
-                    uint32_t ov[32];
-                    tc_ld32(tmem + lane_base + kColO + c, ov);
-                    tc_wait_ld();
+                    for (int c = 0; c < 128; c += 32) {
+                        uint32_t ov[32];
+                        tc_ld32(tmem + lane_base + kColO + 128 * sub + c, ov);
+                        tc_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * factor);
-                    tc_st32(tmem + lane_base + kColO + c, ov);
+                        for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * factor);
+                        tc_st32(tmem + lane_base + kColO + 128 * sub + c, ov);
+                    }
+                    tc_wait_st();
                 }
-                tc_wait_st();
             }
-            // half a P row: 32 tokens x bf16 = four 16-byte chunks, chunk c stored at c ^ (row % 8)
-            uint8_t *p_row = smem + kC2SmemP + grp * kPanelBytes + row * 128;
+            // half a P row of unit 2 i + half: 32 tokens x bf16 = four 16-byte chunks, chunk c stored at c ^ (row % 8)
+            uint8_t *p_row = smem + kC2SmemP + half * kPanelBytes + row * 128;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int chunk = (half * 4 + c) ^ (row & 7);
-                *reinterpret_cast<uint4 *>(p_row + chunk * 16) =
+            for (int c = 0; c < 4; ++c)
+                *reinterpret_cast<uint4 *>(p_row + (((sub * 4 + c) ^ (row & 7)) << 4)) =
                     make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
-            }
             fence_async_smem();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(grp ? p_full_leader1 : p_full_leader0);
+            if (lane == 0) mbar_arrive_cluster(p_full_leader);
         }
         // The row sums are final as soon as the last tile's weights are written, before its P V has
         // run: their exchange and what follows from them overlap that last P V.
-        if (ok) {
-            // the reference after the last tile is the final one
-            ok = mbar_wait(&ctl->ref_bar, (tiles - 1) & 1);
-            ok = __all_sync(0xffffffffu, ok);
-        }
-        if (ok) {
-            const float ref_final = ctl->ref[(tiles - 1) & 1][row];
-            if (ref_final != m_ref) {
-                l *= (m_ref == -INFINITY) ? 0.f : exp2f(m_ref - ref_final);
-                m_ref = ref_final;
-            }
-        }
-        // Slot of a group's partial row sums: the group's row-maximum slots of the parity it did NOT
-        // use for its last tile.  Every thread of the group has passed the exchange barrier of that
-        // last tile, which each thread reached only after reading the slots of the tile before, so
-        // nobody reads them any more (a group without tiles never used its slots at all).
-        auto sum_slot = [&](int g) -> float * {
-            const int last = (tiles - 1) - ((((tiles - 1) & 1) != g) ? 1 : 0);      // the group's last tile, -1 if none
-            const int parity = last >= 0 ? (((last >> 1) & 1) ^ 1) : 0;
-            return &ctl->xchg[0][0][0] + ((g * 2 + parity) * 2) * 64;                // [half][row]
-        };
+        // Their slots: the parity that the last tile did not use.  Every thread has passed the exchange barrier of
+        // that tile, which it reached only after reading the slots of the tile before.
         float lt = 0.f;
         if (ok) {
-            sum_slot(grp)[half * 64 + row] = l;
+            float *sums = &ctl->xchg[tiles & 1][0][row];
+            sums[tq * 64] = l;
             mbar_arrive(&ctl->x_bar);
             ok = mbar_wait(&ctl->x_bar, 0);
             ok = __all_sync(0xffffffffu, ok);
+            lt = (sums[0] + sums[64]) + (sums[128] + sums[192]);
         }
         if (ok) {
-            const float *s0 = sum_slot(0), *s1 = sum_slot(1);
-            lt = (s0[row] + s0[64 + row]) + (s1[row] + s1[64 + row]);
             cm_inv = lt > 0.f ? 1.f / lt : 0.f;
             cm_lse = lt > 0.f ? (m_ref + log2f(lt)) * kLn2 : -INFINITY;
-            // now the last tile's P V
-            ok = mbar_wait(&ctl->pv_done[(tiles - 1) & 1], ((tiles - 1) >> 1) & 1);
+            // now the last unit's P V
+            ok = mbar_wait(&ctl->pv_done[(units - 1) & 1], ((units - 1) >> 1) & 1);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (kClusterMerge && ok) {
@@ -1279,9 +1310,9 @@ inline bool tc2_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cached)
 {
     const uint64_t rows = (uint64_t)p.num_pages * kPage, qrows = (uint64_t)p.batch * p.heads;
     if (cached)
-        return make_panel_map(&maps[0], p.q, qrows, kTcHeads, kPanels) && make_panel_map(&maps[1], p.kv, rows, 32, kPanels) &&
+        return make_panel_map(&maps[0], p.q, qrows, kTcHeads, kC2GroupPanels) && make_panel_map(&maps[1], p.kv, rows, kTile, kC2GroupPanels) &&
                make_panel_map(&maps[2], p.kv, rows, kTile, 4) && make_panel_map(&maps[3], p.kv, rows, kTile, kPanels);
-    return encode_panel_map(&maps[0], p.q, qrows, kTcHeads, kPanels) && encode_panel_map(&maps[1], p.kv, rows, 32, kPanels) &&
+    return encode_panel_map(&maps[0], p.q, qrows, kTcHeads, kC2GroupPanels) && encode_panel_map(&maps[1], p.kv, rows, kTile, kC2GroupPanels) &&
            encode_panel_map(&maps[2], p.kv, rows, kTile, 4) && encode_panel_map(&maps[3], p.kv, rows, kTile, kPanels);
 }
 

@@ -48,7 +48,7 @@ constexpr int kQ8SmemV = kQ8SmemK + kQ8KStages * kQ8KBytes;
 constexpr int kQ8SmemP = kQ8SmemV + kQ8VStages * kQ8VBytes;     // 2 buffers x [64 heads x (64 hi + 64 lo codes)]
 constexpr int kQ8SmemAux = kQ8SmemP + 2 * kPanelBytes;
 constexpr int kQ8SmemQTemp = kQ8SmemV;                    // 8 bf16 panels of q during set-up: V stages + P buffers
-constexpr int kQ8ScaleRing = 8;                           // as the validity-mask ring
+constexpr int kQ8MaskRing = 8, kQ8ScaleRing = 8, kQ8PrefetchAhead = 1;
 constexpr uint32_t kQ8ColS8 = 256, kQ8ColSr = 352;
 // The weights P' = exp2(y - m) are written as E4M3, whose range is [2^-9, 448].  The reference m is
 // therefore kept below the running maximum of y: it is set kQ8Headroom under the tile maximum
@@ -83,7 +83,7 @@ struct Q8Control {
     uint64_t exit_bar;
     uint64_t recv_bar;
     uint64_t ready_bar;
-    uint64_t valid_mask[kMaskRing];
+    uint64_t valid_mask[kQ8MaskRing];
     float xchg[2][4][64];
     uint32_t tmem_base;
     uint32_t abort;
@@ -349,7 +349,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                 aux->tok_log2[ring][lane + 32] = log2f(sc_hi);
                 aux->tok_rcp[ring][lane] = 1.f / sc_lo;
                 aux->tok_rcp[ring][lane + 32] = 1.f / sc_hi;
-                if (lane == 0) ctl->valid_mask[i % kMaskRing] = mask;
+                if (lane == 0) ctl->valid_mask[i % kQ8MaskRing] = mask;
                 __threadfence_block();
             }
             const uint32_t bar = map_to_rank(smem_u32(&ctl->k_full[st]), leader);
@@ -365,7 +365,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                 gather_k_rows_q8(dst, kv_bytes, own_row, lane);
             }
             if (pending >= 0) {
-                retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kQ8KBytes, gathered, lane);
+                retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kQ8KBytes, gathered ? 1 : 0, lane);
                 pending = -1;
             }
             if (gathered) pending = st;
@@ -378,7 +378,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             stage_pages(x1);
             stage_tokens(i + 3, x2);
         }
-        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kQ8KBytes, false, lane);
+        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kQ8KBytes, 0, lane);
         if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = 0x7fffffff;
         if (!ok && lane == 0) {
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_PRODUCER_K);
@@ -423,7 +423,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                 gather_v_rows_q8(dst, kv_bytes + (int)rank * 256, row_lo, row_hi, lane);
             }
             if (pending >= 0) {
-                retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kQ8VBytes, gathered, lane);
+                retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kQ8VBytes, gathered ? 1 : 0, lane);
                 pending = -1;
             }
             if (gathered) pending = st;
@@ -432,7 +432,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             stage_pages(x1);
             stage_tokens(i + 3, x2);
         }
-        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kQ8VBytes, false, lane);
+        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kQ8VBytes, 0, lane);
         if (!ok && lane == 0) {
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_PRODUCER_V);
             *abort_flag = 1;
@@ -457,7 +457,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                 for (int k = 0; ok && k < count; ++k) {
                     const int i = t0 + k;
                     const volatile int32_t *progress = &ctl->k_progress;
-                    for (int naps = 0; *progress < i - kPrefetchAhead && *abort_flag == 0; ++naps) {
+                    for (int naps = 0; *progress < i - kQ8PrefetchAhead && *abort_flag == 0; ++naps) {
                         if (naps > (1 << 22)) {
                             ok = false;
                             break;
@@ -650,7 +650,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(s_empty_leader + 8 * sbuf);
-            const uint32_t valid = (uint32_t)(ctl->valid_mask[i % kMaskRing] >> (16 * part)) & 0xffffu;
+            const uint32_t valid = (uint32_t)(ctl->valid_mask[i % kQ8MaskRing] >> (16 * part)) & 0xffffu;
             const float4 *ts = reinterpret_cast<const float4 *>(&aux->tok_scale[ring][16 * part]);
             const float4 *tl = reinterpret_cast<const float4 *>(&aux->tok_log2[ring][16 * part]);
             float y[16];

@@ -33,7 +33,7 @@ def test_few_heads_fused_merge(heads):
 @pytest.mark.parametrize("batch,heads", [(1, 3), (6, 74), (6, 75)])
 def test_merge_of_any_number_of_splits(splits, batch, heads):
     """(6, 74): as many blocks as three per SM, (6, 75): more.  Empty splits carry rows of NaN, which must
-    not be read; fp32 sums of at most 70 terms, results rounded to bf16 (half an ulp: 2^-9)."""
+    not be read; fp32 sums of at most 70 terms, results rounded to bf16 (half an ulp: at most 2^-8 of the value)."""
     rng = np.random.default_rng(splits)
     part = rng.standard_normal((batch, splits, heads, 512)).astype(np.float32)
     lse = (rng.standard_normal((batch, splits, heads)) * 3).astype(np.float32)
