@@ -21,9 +21,16 @@
 //    below 448 whatever the data, which is what lets it be written as E4M3: again as two
 //    terms hi + lo, side by side in one 128-byte row of the P buffer, [hi tokens 0..63 | lo tokens
 //    0..63], so that O += [P_hi | P_lo] [V8 ; V8] is four K = 32 steps per accumulator.
-//  * Shared memory.  A K-role stage is 20 KiB and a V-role stage 16 KiB (36 and 32 KiB for bf16
-//    rows), so the same budget holds four K stages and three V stages: twice the tokens in flight.
-//    The bf16 copy of q (latent panels) sits in the V stages and P buffers while it is converted.
+//  * Shared memory.  The K rows of a tile are 40 KiB a CTA and the V columns of a unit 16 KiB (72 and 32
+//    for bf16 rows), so the same budget holds two whole tiles of K and three units of V.  The bf16 copy
+//    of q (latent panels) sits in the V stages and P buffers while it is converted.
+//  * Tensor memory holds two score buffers (of two accumulators each) instead of three.
+//
+// What bounds it: the tensor core takes as long as for bf16 rows (two terms of half the width), and the
+// softmax warps go through about 16 instructions a token in one long chain per tile.  On tiles
+// of 64 tokens that chain took 2100 clocks a tile and nothing overlapped it; on tiles of 128 a thread
+// has twice the independent work for the same chain: 32 requests x 33 units 33.6 -> 28.3 us, 128 x 64
+// 181 -> 148.
 //
 // Work split, merge paths, index handling, time-outs: as in tc2_decode_kernel.
 #pragma once
@@ -36,20 +43,23 @@ namespace omni {
 
 constexpr int kQ8RowBytes = 640;
 constexpr int kQ8Panels = 5;                              // four panels of 128 codes, one of 64 bf16 rope columns
-constexpr int kQ8KStages = 4, kQ8VStages = 3;
-constexpr int kQ8KPanel = 32 * 128;
-constexpr int kQ8KBytes = kQ8Panels * kQ8KPanel;          // K role: 32 tokens x 640 B
+constexpr int kQ8KStages = 2, kQ8VStages = 3;
+constexpr int kQ8KBytes = kQ8Panels * kPanelBytes;        // K role: 64 tokens x 640 B
 constexpr int kQ8VBytes = 2 * kPanelBytes;                // V role: 64 tokens x 256 codes
 constexpr int kQ8SmemQHi = 0;                             // 4 panels x [64 heads x 128 codes]
 constexpr int kQ8SmemQLo = 4 * kPanelBytes;
 constexpr int kQ8SmemQRope = 8 * kPanelBytes;             // [64 heads x 64 bf16]
 constexpr int kQ8SmemK = kTileBytes;
 constexpr int kQ8SmemV = kQ8SmemK + kQ8KStages * kQ8KBytes;
-constexpr int kQ8SmemP = kQ8SmemV + kQ8VStages * kQ8VBytes;     // 2 buffers x [64 heads x (64 hi + 64 lo codes)]
+constexpr int kQ8SmemP = kQ8SmemV + kQ8VStages * kQ8VBytes;     // 2 units x [64 heads x (64 hi + 64 lo codes)]
 constexpr int kQ8SmemAux = kQ8SmemP + 2 * kPanelBytes;
 constexpr int kQ8SmemQTemp = kQ8SmemV;                    // 8 bf16 panels of q during set-up: V stages + P buffers
-constexpr int kQ8MaskRing = 8, kQ8ScaleRing = 8, kQ8PrefetchAhead = 1;
-constexpr uint32_t kQ8ColS8 = 256, kQ8ColSr = 352;
+// Masks and scales travel from the K producer to the softmax warps through rings.  Those of tile t + 2 are
+// written once the score MMAs of tile t have retired; these were issued only after every softmax warp
+// had read the scores of tile t - 2 (two score buffers), i.e. after tile t - 3 was finished: five
+// tiles can be live.
+constexpr int kQ8Ring = 5;
+constexpr uint32_t kQ8ColS8 = 256, kQ8ColSr = 384;        // two buffers of 64 columns each
 // The weights P' = exp2(y - m) are written as E4M3, whose range is [2^-9, 448].  The reference m is
 // therefore kept below the running maximum of y: it is set kQ8Headroom under the tile maximum
 // whenever that maximum has risen more than kQ8RescaleWindow above it, so the largest weight
@@ -58,10 +68,10 @@ constexpr uint32_t kQ8ColS8 = 256, kQ8ColSr = 352;
 constexpr float kQ8Headroom = 8.f, kQ8RescaleWindow = 8.75f;
 
 struct Q8Aux {
-    float q_scale[64];                        // a[row]
-    float tok_scale[kQ8ScaleRing][64];        // scale of each token of a tile
-    float tok_log2[kQ8ScaleRing][64];         // its base-2 logarithm
-    float tok_rcp[kQ8ScaleRing][64];          // its reciprocal
+    float q_scale[64];                    // a[row]
+    float tok_scale[kQ8Ring][128];        // scale of each token of a tile
+    float tok_log2[kQ8Ring][128];         // its base-2 logarithm
+    float tok_rcp[kQ8Ring][128];          // its reciprocal
 };
 static_assert(kQ8SmemQRope + kPanelBytes == kTileBytes, "q area");
 static_assert(kQ8SmemAux + (int)sizeof(Q8Aux) <= kC2SmemCtl, "auxiliary arrays must end below the control block");
@@ -75,15 +85,15 @@ struct Q8Control {
     uint64_t k_empty[kQ8KStages];
     uint64_t v_full[kQ8VStages];
     uint64_t v_empty[kQ8VStages];
-    uint64_t s_full[3];
-    uint64_t s_empty[3];
-    uint64_t p_full[2];
-    uint64_t p_free[2];                  // P V of a tile retired: its P buffer may be rewritten, O may be rescaled
+    uint64_t s_full[2];
+    uint64_t s_empty[2];
+    uint64_t p_full;                     // both P units of a tile are written (and O rescaled)
+    uint64_t pv_done[2];                 // P V of a unit retired: its P unit may be rewritten, O may be rescaled
     uint64_t x_bar;
     uint64_t exit_bar;
     uint64_t recv_bar;
     uint64_t ready_bar;
-    uint64_t valid_mask[kQ8MaskRing];
+    uint64_t valid_mask[kQ8Ring][2];     // [tile][unit]
     float xchg[2][4][64];
     uint32_t tmem_base;
     uint32_t abort;
@@ -112,6 +122,20 @@ __device__ __forceinline__ void tc_mma8_pair_elect(uint32_t d_tmem, uint32_t a_l
         "elect.sync _|q, 0xffffffff;\n\t"
         "@q tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %5, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(kAccumulate ? 1 : 0)
+        : "memory");
+}
+
+__device__ __forceinline__ void tc_mma8_pair_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                                   uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -145,37 +169,26 @@ __device__ __forceinline__ void split_e4m3(const float (&v)[16], uint4 &hi, uint
     lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// Row gathers of the 8-bit layout (see gather_k_rows / gather_v_rows): 640-byte rows, K role
-// 32 rows x 5 panels, V role 64 rows x the two panels of this CTA's value columns.
-__device__ __noinline__ void gather_k_rows_q8(uint32_t dst, const char *kv_bytes, int own_row, int lane)
-{
-    const int ch = lane & 7;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        const int r = 4 * g + (lane >> 3);
-        const int src_row = __shfl_sync(0xffffffffu, own_row, r);
-        const char *src = kv_bytes + (size_t)src_row * kQ8RowBytes + ch * 16;
-        const uint32_t d = dst + r * 128 + ((ch ^ (r & 7)) << 4);
-#pragma unroll
-        for (int c = 0; c < kQ8Panels; ++c) cp_async16(d + c * kQ8KPanel, src + c * 128);
-    }
-    cp_async_commit();
-}
-
-__device__ __noinline__ void gather_v_rows_q8(uint32_t dst, const char *kv_cols, int row_lo, int row_hi, int lane)
+// Row gathers of the 8-bit layout (see gather_rows): 64 rows of 640 bytes, kCount panels.
+template <int kCount>
+__device__ __noinline__ void gather_rows_q8(uint32_t dst, const char *cols, int row_lo, int row_hi, int lane)
 {
     const int ch = lane & 7;
 #pragma unroll
     for (int g = 0; g < 16; ++g) {
         const int r = 4 * g + (lane >> 3);
-        const int a = __shfl_sync(0xffffffffu, row_lo, r & 31), c2 = __shfl_sync(0xffffffffu, row_hi, r & 31);
-        const int src_row = r < 32 ? a : c2;
-        const char *src = kv_cols + (size_t)src_row * kQ8RowBytes + ch * 16;
+        const int src_row = __shfl_sync(0xffffffffu, g < 8 ? row_lo : row_hi, r & 31);
+        const char *src = cols + (size_t)src_row * kQ8RowBytes + ch * 16;
         const uint32_t d = dst + r * 128 + ((ch ^ (r & 7)) << 4);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) cp_async16(d + c * kPanelBytes, src + c * 128);
+        for (int c = 0; c < kCount; ++c) cp_async16(d + c * kPanelBytes, src + c * 128);
     }
     cp_async_commit();
+}
+
+__device__ __forceinline__ void prefetch_row_q8(const char *kv, int row)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(kv + (size_t)row * kQ8RowBytes), "n"(kQ8RowBytes) : "memory");
 }
 
 // Two instances, as for the bf16 kernel: with and without the in-cluster merge of two splits, each
@@ -219,14 +232,12 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             mbar_init(&ctl->v_full[i], 1);
             mbar_init(&ctl->v_empty[i], 1);
         }
-        for (int i = 0; i < 3; ++i) {
+        for (int i = 0; i < 2; ++i) {
             mbar_init(&ctl->s_full[i], 1);
             mbar_init(&ctl->s_empty[i], 16);
+            mbar_init(&ctl->pv_done[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&ctl->p_full[i], 16);
-            mbar_init(&ctl->p_free[i], 1);
-        }
+        mbar_init(&ctl->p_full, 16);
         mbar_init(&ctl->x_bar, 256);
         mbar_init(&ctl->exit_bar, 2);
         mbar_init(&ctl->recv_bar, 1);
@@ -255,9 +266,9 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
     const bool bad_len = selection.bad;
     int begin, end;
     split_range(n, p.splits, s, begin, end, kC2Tile);
-    const int tiles = (end - begin + kC2Tile - 1) / kC2Tile;
+    const int units = (end - begin + kC2Tile - 1) / kC2Tile, tiles = (units + 1) / 2;
 
-    const bool active = tiles > 0;
+    const bool active = units > 0;
     if (!active && bad_len && threadIdx.x == 0 && crank == 0) flag_status(p.status, OMNI_DEV_BAD_INDEX);
     if (!kClusterMerge && !active) c2_store_empty(p, b, s, h0, head_rows, warp, lane);
 
@@ -266,39 +277,42 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
     const int32_t *pt = p.page_table + (size_t)b * p.max_pages;
     const char *kv_bytes = reinterpret_cast<const char *>(p.kv);
 
-    // Index pipeline of the producers: as in tc2_decode_kernel (lane l serves tokens l and l+32).
+    // Index pipeline of the producers: as in tc2_decode_kernel (lane l serves tokens l and l+32 of a unit).
     struct TileIdx {
         int t0, t1;
         int pg0, pg1;
     };
-    auto stage_tokens = [&](int tile, TileIdx &x) {
-        const int j0 = begin + tile * kC2Tile + lane, j1 = j0 + 32;
-        x.t0 = (tile < tiles && j0 < end) ? selection_at(selection, j0) : -1;
-        x.t1 = (tile < tiles && j1 < end) ? selection_at(selection, j1) : -1;
+    const uint32_t t_limit = (uint32_t)min((int64_t)p.max_pages * kPage, (int64_t)1 << 31);
+    const uint32_t page_limit = (uint32_t)p.num_pages;
+    auto stage_tokens = [&](int unit, TileIdx &x) {
+        const int j0 = begin + unit * kC2Tile + lane, j1 = j0 + 32;
+        x.t0 = j0 < end ? selection_at(selection, j0) : -1;
+        x.t1 = j1 < end ? selection_at(selection, j1) : -1;
     };
     auto stage_pages = [&](TileIdx &x) {
-        x.pg0 = (x.t0 >= 0 && x.t0 / kPage < p.max_pages) ? ldg_index(pt + x.t0 / kPage, selection.keep) : -1;
-        x.pg1 = (x.t1 >= 0 && x.t1 / kPage < p.max_pages) ? ldg_index(pt + x.t1 / kPage, selection.keep) : -1;
+        x.pg0 = (uint32_t)x.t0 < t_limit ? ldg_index(pt + (x.t0 >> 6), selection.keep) : -1;
+        x.pg1 = (uint32_t)x.t1 < t_limit ? ldg_index(pt + (x.t1 >> 6), selection.keep) : -1;
     };
-    auto stage_rows = [&](int tile, const TileIdx &x, int &row_lo, int &row_hi, uint64_t &mask, bool &contig,
-                          bool &contig_lo, bool &contig_hi, bool &any_bad) {
-        const int j0 = begin + tile * kC2Tile + lane, j1 = j0 + 32;
-        const bool ok0 = x.pg0 >= 0 && (int64_t)x.pg0 < p.num_pages, ok1 = x.pg1 >= 0 && (int64_t)x.pg1 < p.num_pages;
-        any_bad |= (j0 < end && !ok0 && !is_padding(selection, x.t0)) || (j1 < end && !ok1 && !is_padding(selection, x.t1));
-        const int r0 = ok0 ? x.pg0 * kPage + x.t0 % kPage : -1, r1 = ok1 ? x.pg1 * kPage + x.t1 % kPage : -1;
-        const uint32_t m0 = __ballot_sync(0xffffffffu, r0 >= 0), m1 = __ballot_sync(0xffffffffu, r1 >= 0);
+    auto stage_rows = [&](int unit, const TileIdx &x, int &row_lo, int &row_hi, uint64_t &mask, bool &contig,
+                          bool &any_bad) {
+        const bool ok0 = (uint32_t)x.pg0 < page_limit, ok1 = (uint32_t)x.pg1 < page_limit;
+        row_lo = x.pg0 * kPage + (x.t0 & (kPage - 1));
+        row_hi = x.pg1 * kPage + (x.t1 & (kPage - 1));
+        const int base = __shfl_sync(0xffffffffu, row_lo, 0);
+        contig = __all_sync(0xffffffffu, ok0 && ok1 && row_lo == base + lane && row_hi == base + 32 + lane);
+        mask = ~0ull;
+        if (contig) return;
+        const int j0 = begin + unit * kC2Tile + lane, j1 = j0 + 32;
+        any_bad |= (j0 < end && !ok0) || (j1 < end && !ok1);
+        const uint32_t m0 = __ballot_sync(0xffffffffu, ok0), m1 = __ballot_sync(0xffffffffu, ok1);
         mask = (uint64_t)m0 | ((uint64_t)m1 << 32);
         int stand_in = 0;
         if (m0)
-            stand_in = __shfl_sync(0xffffffffu, r0, __ffs(m0) - 1);
+            stand_in = __shfl_sync(0xffffffffu, row_lo, __ffs(m0) - 1);
         else if (m1)
-            stand_in = __shfl_sync(0xffffffffu, r1, __ffs(m1) - 1);
-        row_lo = r0 >= 0 ? r0 : stand_in;
-        row_hi = r1 >= 0 ? r1 : stand_in;
-        const int base_lo = __shfl_sync(0xffffffffu, row_lo, 0), base_hi = __shfl_sync(0xffffffffu, row_hi, 0);
-        contig_lo = __all_sync(0xffffffffu, r0 == base_lo + lane);
-        contig_hi = __all_sync(0xffffffffu, r1 == base_hi + lane);
-        contig = contig_lo && contig_hi && base_hi == base_lo + 32;
+            stand_in = __shfl_sync(0xffffffffu, row_hi, __ffs(m1) - 1);
+        row_lo = ok0 ? row_lo : stand_in;
+        row_hi = ok1 ? row_hi : stand_in;
     };
 
     float cm_lse = -INFINITY, cm_inv = 0.f;
@@ -314,71 +328,100 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             tma_box3d(smem_base + kQ8SmemQTemp, &q_nope_map, &ctl->q_full, b * p.heads + h0, 0);
             tma_box3d(smem_base + kQ8SmemQRope, &q_rope_map, &ctl->q_full, b * p.heads + h0, 8);
         }
+        // This CTA's K rows are unit 2 t + rank of every tile t.
         bool any_bad = bad_len;
-        TileIdx x1, x2;
-        int row_lo, row_hi;
-        uint64_t mask;
-        bool contig, contig_lo, contig_hi;
-        float sc_lo, sc_hi;                  // scales of the rows of the tile about to be loaded
+        TileIdx x1[2], x2[2];
+        int row_lo = 0, row_hi = 0;          // of this CTA's unit of the tile about to be loaded
+        bool contig = false;
+        uint64_t mask[2];
+        float sc[2][2];                      // scales of the rows of that tile: [unit][token half]
+        auto resolve_tile = [&](int tile, const TileIdx (&x)[2]) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                int lo, hi;
+                bool whole;
+                stage_rows(2 * tile + h, x[h], lo, hi, mask[h], whole, any_bad);
+                // a unit without tokens has no row whose scale could be read
+                sc[h][0] = mask[h] ? __ldg(p.kv_scale + lo) : 1.f;
+                sc[h][1] = mask[h] ? __ldg(p.kv_scale + hi) : 1.f;
+                if (h == (int)rank) {
+                    row_lo = lo;
+                    row_hi = hi;
+                    contig = whole;
+                }
+            }
+        };
         {
-            TileIdx x0;
-            stage_tokens(0, x0);
-            stage_tokens(1, x1);
-            stage_tokens(2, x2);
-            stage_pages(x0);
-            stage_pages(x1);
-            stage_rows(0, x0, row_lo, row_hi, mask, contig, contig_lo, contig_hi, any_bad);
-            sc_lo = __ldg(p.kv_scale + row_lo);
-            sc_hi = __ldg(p.kv_scale + row_hi);
+            TileIdx x0[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                stage_tokens(h, x0[h]);
+                stage_tokens(2 + h, x1[h]);
+                stage_tokens(4 + h, x2[h]);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                stage_pages(x0[h]);
+                stage_pages(x1[h]);
+            }
+            resolve_tile(0, x0);
         }
         bool ok = true;
         int pending = -1;
+        const uint32_t k_full_leader = map_to_rank(smem_u32(&ctl->k_full[0]), leader);
         for (int i = 0; ok && i < tiles; ++i) {
-            const int st = i % kQ8KStages;
-            if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = i;
-            if (i >= kQ8KStages) ok = mbar_wait(&ctl->k_empty[st], ((i / kQ8KStages) - 1) & 1);
+            const int st = i & 1;
+            if (i >= 2) {
+                if (pending >= 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->k_empty[st], ((i >> 1) - 1) & 1))) {
+                    retire_gathered_stage(k_full_leader + 8 * pending, kQ8KBytes, 0, lane);
+                    pending = -1;
+                }
+                ok = mbar_wait(&ctl->k_empty[st], ((i >> 1) - 1) & 1);
+            }
             ok = __all_sync(0xffffffffu, ok) && (*abort_flag == 0);
             if (!ok) break;
             {
                 // what the softmax warps need to know about tile i, published before its copy is
                 // requested: which tokens count, and every token's scale, its logarithm and reciprocal
-                const int ring = i % kQ8ScaleRing;
-                aux->tok_scale[ring][lane] = sc_lo;
-                aux->tok_scale[ring][lane + 32] = sc_hi;
-                aux->tok_log2[ring][lane] = log2f(sc_lo);
-                aux->tok_log2[ring][lane + 32] = log2f(sc_hi);
-                aux->tok_rcp[ring][lane] = 1.f / sc_lo;
-                aux->tok_rcp[ring][lane + 32] = 1.f / sc_hi;
-                if (lane == 0) ctl->valid_mask[i % kQ8MaskRing] = mask;
+                const int ring = i % kQ8Ring;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float s1 = sc[k >> 1][k & 1];
+                    aux->tok_scale[ring][32 * k + lane] = s1;
+                    aux->tok_log2[ring][32 * k + lane] = log2f(s1);
+                    aux->tok_rcp[ring][32 * k + lane] = 1.f / s1;
+                }
+                if (lane < 2) ctl->valid_mask[ring][lane] = lane ? mask[1] : mask[0];
                 __threadfence_block();
+                __syncwarp();
             }
-            const uint32_t bar = map_to_rank(smem_u32(&ctl->k_full[st]), leader);
-            if (lane == 0 && rank == 0) mbar_expect_tx(&ctl->k_full[st], 2 * kQ8KBytes);
-            __syncwarp();
-            const uint32_t dst = smem_base + kQ8SmemK + st * kQ8KBytes;
-            const int own_row = rank ? row_hi : row_lo;
+            if (lane == 0 && rank == 0) mbar_expect_tx(&ctl->k_full[st], (2 * i + 1 < units ? 2 : 1) * kQ8KBytes);
+            // the last tile has a single unit when their number is odd: CTA 1 then leaves its rows as they are
             bool gathered = false;
-            if (rank ? contig_hi : contig_lo) {
-                if (lane == 0) tma_box3d_pair(dst, &kv_k_map, bar, own_row, 0);
-            } else {
-                gathered = true;
-                gather_k_rows_q8(dst, kv_bytes, own_row, lane);
+            if (2 * i + (int)rank < units) {
+                const uint32_t dst = smem_base + kQ8SmemK + st * kQ8KBytes;
+                if (contig) {
+                    if (lane == 0) tma_box3d_pair(dst, &kv_k_map, k_full_leader + 8 * st, row_lo, 0);
+                } else {
+                    gathered = true;
+                    gather_rows_q8<kQ8Panels>(dst, kv_bytes, row_lo, row_hi, lane);
+                }
             }
+            if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = 2 * i + 2;
             if (pending >= 0) {
-                retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kQ8KBytes, gathered ? 1 : 0, lane);
+                retire_gathered_stage(k_full_leader + 8 * pending, kQ8KBytes, gathered ? 1 : 0, lane);
                 pending = -1;
             }
             if (gathered) pending = st;
-            if (i + 1 < tiles) {
-                stage_rows(i + 1, x1, row_lo, row_hi, mask, contig, contig_lo, contig_hi, any_bad);
-                sc_lo = __ldg(p.kv_scale + row_lo);
-                sc_hi = __ldg(p.kv_scale + row_hi);
+            if (i + 1 < tiles) resolve_tile(i + 1, x1);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                x1[h] = x2[h];
+                stage_pages(x1[h]);
+                stage_tokens(2 * i + 6 + h, x2[h]);
             }
-            x1 = x2;
-            stage_pages(x1);
-            stage_tokens(i + 3, x2);
         }
-        if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->k_full[pending]), leader), kQ8KBytes, 0, lane);
+        if (pending >= 0) retire_gathered_stage(k_full_leader + 8 * pending, kQ8KBytes, 0, lane);
         if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = 0x7fffffff;
         if (!ok && lane == 0) {
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_PRODUCER_K);
@@ -392,7 +435,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
         TileIdx x1, x2;
         int row_lo, row_hi;
         uint64_t mask_unused;
-        bool contig, contig_lo, contig_hi;
+        bool contig;
         {
             TileIdx x0;
             stage_tokens(0, x0);
@@ -400,15 +443,21 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             stage_tokens(2, x2);
             stage_pages(x0);
             stage_pages(x1);
-            stage_rows(0, x0, row_lo, row_hi, mask_unused, contig, contig_lo, contig_hi, any_bad);
+            stage_rows(0, x0, row_lo, row_hi, mask_unused, contig, any_bad);
         }
         // the V stages hold the temporary copy of q until the softmax warps have converted it
         bool ok = mbar_wait(&ctl->q_conv, 0);
         ok = __all_sync(0xffffffffu, ok);
         int pending = -1;
-        for (int i = 0; ok && i < tiles; ++i) {
+        for (int i = 0; ok && i < units; ++i) {
             const int st = i % kQ8VStages;
-            if (i >= kQ8VStages) ok = mbar_wait(&ctl->v_empty[st], ((i / kQ8VStages) - 1) & 1);
+            if (i >= kQ8VStages) {
+                if (pending >= 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->v_empty[st], ((i / kQ8VStages) - 1) & 1))) {
+                    retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kQ8VBytes, 0, lane);
+                    pending = -1;
+                }
+                ok = mbar_wait(&ctl->v_empty[st], ((i / kQ8VStages) - 1) & 1);
+            }
             ok = __all_sync(0xffffffffu, ok) && (*abort_flag == 0);
             if (!ok) break;
             const uint32_t bar = map_to_rank(smem_u32(&ctl->v_full[st]), leader);
@@ -420,14 +469,14 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                 if (lane == 0) tma_box3d_pair(dst, &kv_v_map, bar, row_lo, 2 * (int)rank);
             } else {
                 gathered = true;
-                gather_v_rows_q8(dst, kv_bytes + (int)rank * 256, row_lo, row_hi, lane);
+                gather_rows_q8<2>(dst, kv_bytes + (int)rank * 256, row_lo, row_hi, lane);
             }
             if (pending >= 0) {
                 retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kQ8VBytes, gathered ? 1 : 0, lane);
                 pending = -1;
             }
             if (gathered) pending = st;
-            if (i + 1 < tiles) stage_rows(i + 1, x1, row_lo, row_hi, mask_unused, contig, contig_lo, contig_hi, any_bad);
+            if (i + 1 < units) stage_rows(i + 1, x1, row_lo, row_hi, mask_unused, contig, any_bad);
             x1 = x2;
             stage_pages(x1);
             stage_tokens(i + 3, x2);
@@ -438,46 +487,55 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             *abort_flag = 1;
         }
     } else if (warp == 7) {
-        // =========================== L2 prefetcher (CTA 0 only) ==========================
-        if (rank == 0) {
-            for (int t0 = 0; t0 < tiles; t0 += 32) {
-                const int t = t0 + lane;
-                const int j0 = begin + t * kC2Tile;
-                int row = -1;
-                if (t < tiles && j0 + kC2Tile <= end) {
-                    const int first = selection_at(selection, j0), last = selection_at(selection, j0 + kC2Tile - 1);
-                    if (first >= 0 && first % kPage == 0 && last == first + kC2Tile - 1 && first / kPage < p.max_pages) {
-                        const int pg = ldg_index(pt + first / kPage, selection.keep);
-                        if (pg >= 0 && (int64_t)pg < p.num_pages) row = pg * kPage;
-                    }
+        // =========================== L2 prefetcher (as in tc2_decode_kernel) =============
+        for (int t0 = (int)rank; t0 < units; t0 += 64) {
+            const int t = t0 + 2 * lane;
+            const int j0 = begin + t * kC2Tile;
+            int row = -1;
+            if (t < units && j0 + kC2Tile <= end) {
+                const int first = selection_at(selection, j0), last = selection_at(selection, j0 + kC2Tile - 1);
+                if (first >= 0 && first % kPage == 0 && last == first + kC2Tile - 1 && first / kPage < p.max_pages) {
+                    const int pg = ldg_index(pt + first / kPage, selection.keep);
+                    if (pg >= 0 && (int64_t)pg < p.num_pages) row = pg * kPage;
                 }
-                const int count = min(32, tiles - t0);
-                bool ok = true;
-                if (!__any_sync(0xffffffffu, row >= 0)) continue;
-                for (int k = 0; ok && k < count; ++k) {
-                    const int i = t0 + k;
-                    const volatile int32_t *progress = &ctl->k_progress;
-                    for (int naps = 0; *progress < i - kQ8PrefetchAhead && *abort_flag == 0; ++naps) {
-                        if (naps > (1 << 22)) {
-                            ok = false;
-                            break;
-                        }
-                        __nanosleep(200);
-                    }
-                    ok = ok && (*abort_flag == 0);
-                    if (ok && lane == k && row >= 0)
-                        asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(&kv_page_map),
-                                     "r"(0), "r"(row), "r"(0)
-                                     : "memory");
-                }
-                if (!ok) break;
             }
+            __syncwarp();
+            bool ok = true;
+            TileIdx x = {-1, -1, -1, -1};    // of a unit that is not a whole page
+            for (int k = 0; ok && k < 32 && t0 + 2 * k < units; ++k) {
+                const int i = t0 + 2 * k;
+                const bool page = __shfl_sync(0xffffffffu, row, k) >= 0;
+                if (!page) {
+                    stage_tokens(i, x);
+                    stage_pages(x);
+                }
+                const volatile int32_t *progress = &ctl->k_progress;
+                for (int naps = 0; *progress < i - (int)rank - (page ? 0 : kScatterAhead) && *abort_flag == 0; ++naps) {
+                    if (naps > (1 << 22)) {
+                        ok = false;
+                        break;
+                    }
+                    __nanosleep(200);
+                }
+                ok = ok && (*abort_flag == 0);
+                ok = __all_sync(0xffffffffu, ok);
+                if (ok && page && lane == k)
+                    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(&kv_page_map),
+                                 "r"(0), "r"(row), "r"(0)
+                                 : "memory");
+                if (ok && !page && *progress <= i) {
+                    if ((uint32_t)x.pg0 < page_limit) prefetch_row_q8(kv_bytes, x.pg0 * kPage + (x.t0 & (kPage - 1)));
+                    if ((uint32_t)x.pg1 < page_limit) prefetch_row_q8(kv_bytes, x.pg1 * kPage + (x.t1 & (kPage - 1)));
+                }
+                __syncwarp();
+            }
+            if (!ok) break;
         }
     } else if (warp == 1) {
         // =========================== MMA issuer (CTA 0 only) =============================
         if (rank == 0) {
-            constexpr uint32_t idesc_qk8 = instr_desc_e4m3(128, kC2Tile, 0);
-            constexpr uint32_t idesc_qkr = instr_desc(128, kC2Tile, 0);
+            constexpr uint32_t idesc_qk8 = instr_desc_e4m3(128, 2 * kC2Tile, 0);
+            constexpr uint32_t idesc_qkr = instr_desc(128, 2 * kC2Tile, 0);
             constexpr uint32_t idesc_pv8 = instr_desc_e4m3(128, 256, 1);
             const uint64_t q_desc = smem_desc(smem_base + kQ8SmemQHi, 16, 1024);
             const uint64_t k_desc = smem_desc(smem_base + kQ8SmemK, 16, 1024);
@@ -485,24 +543,24 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             const uint64_t v_desc = smem_desc(smem_base + kQ8SmemV, kPanelBytes, 1024);
             const uint32_t q_lo = (uint32_t)q_desc, k_lo = (uint32_t)k_desc, p_lo = (uint32_t)p_desc, v_lo = (uint32_t)v_desc;
             const uint32_t kmaj_hi = (uint32_t)(q_desc >> 32), v_hi = (uint32_t)(v_desc >> 32);
-            const int tiles_u = __shfl_sync(0xffffffffu, tiles, 0);
+            const int tiles_u = __shfl_sync(0xffffffffu, tiles, 0), units_u = __shfl_sync(0xffffffffu, units, 0);
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             // S8(t) = [Q_hi | Q_lo] [K8 ; K8]^T: two terms x 16 steps of 32 codes; Sr(t) = Q_rope K_rope^T: 4 steps of 16 bf16
             auto issue_qk = [&](int kst, int sbuf) {
-                const uint32_t d8 = tmem_u + kQ8ColS8 + 32 * sbuf, dr = tmem_u + kQ8ColSr + 32 * sbuf;
+                const uint32_t d8 = tmem_u + kQ8ColS8 + 64 * sbuf, dr = tmem_u + kQ8ColSr + 64 * sbuf;
                 const uint32_t kb = k_lo + ((kst * kQ8KBytes) >> 4);
                 tc_mma8_pair_elect<false>(d8, q_lo, kmaj_hi, kb, kmaj_hi, idesc_qk8);
 #pragma unroll
                 for (int kk = 1; kk < 32; ++kk) {
                     const int term = kk >> 4, c = kk & 15;
                     tc_mma8_pair_elect<true>(d8, q_lo + ((term * kQ8SmemQLo + (c >> 2) * kPanelBytes + (c & 3) * 32) >> 4), kmaj_hi,
-                                             kb + (((c >> 2) * kQ8KPanel + (c & 3) * 32) >> 4), kmaj_hi, idesc_qk8);
+                                             kb + (((c >> 2) * kPanelBytes + (c & 3) * 32) >> 4), kmaj_hi, idesc_qk8);
                 }
-                tc_mma_pair_elect<false>(dr, q_lo + (kQ8SmemQRope >> 4), kmaj_hi, kb + ((4 * kQ8KPanel) >> 4), kmaj_hi, idesc_qkr);
+                tc_mma_pair_elect<false>(dr, q_lo + (kQ8SmemQRope >> 4), kmaj_hi, kb + ((4 * kPanelBytes) >> 4), kmaj_hi, idesc_qkr);
 #pragma unroll
                 for (int kk = 1; kk < 4; ++kk)
                     tc_mma_pair_elect<true>(dr, q_lo + ((kQ8SmemQRope + kk * 32) >> 4), kmaj_hi,
-                                            kb + ((4 * kQ8KPanel + kk * 32) >> 4), kmaj_hi, idesc_qkr);
+                                            kb + ((4 * kPanelBytes + kk * 32) >> 4), kmaj_hi, idesc_qkr);
                 tc_commit_pair_elect(&ctl->k_empty[kst], pair_mask);
                 tc_commit_pair_elect(&ctl->s_full[sbuf], pair_mask);
             };
@@ -511,13 +569,8 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             auto issue_pv = [&](int vst, int pbuf, bool first) {
                 const uint32_t a = p_lo + ((pbuf * kPanelBytes) >> 4);
                 const uint32_t bd = v_lo + ((vst * kQ8VBytes) >> 4);
-                if (first) {
-                    tc_mma8_pair_elect<false>(tmem_u + kColO, a, kmaj_hi, bd, v_hi, idesc_pv8);
-                    tc_mma8_pair_elect<false>(tmem_u + kColO + 128, a, kmaj_hi, bd + (kPanelBytes >> 4), v_hi, idesc_pv8);
-                } else {
-                    tc_mma8_pair_elect<true>(tmem_u + kColO, a, kmaj_hi, bd, v_hi, idesc_pv8);
-                    tc_mma8_pair_elect<true>(tmem_u + kColO + 128, a, kmaj_hi, bd + (kPanelBytes >> 4), v_hi, idesc_pv8);
-                }
+                tc_mma8_pair_elect(tmem_u + kColO, a, kmaj_hi, bd, v_hi, idesc_pv8, first ? 0u : 1u);
+                tc_mma8_pair_elect(tmem_u + kColO + 128, a, kmaj_hi, bd + (kPanelBytes >> 4), v_hi, idesc_pv8, first ? 0u : 1u);
 #pragma unroll
                 for (int k = 1; k < 4; ++k) {
                     const uint32_t ak = a + ((k * 32) >> 4), bk = bd + (((k & 1) * 4096) >> 4);
@@ -525,35 +578,45 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                     tc_mma8_pair_elect<true>(tmem_u + kColO + 128, ak, kmaj_hi, bk + (kPanelBytes >> 4), v_hi, idesc_pv8);
                 }
                 tc_commit_pair_elect(&ctl->v_empty[vst], pair_mask);
-                tc_commit_pair_elect(&ctl->p_free[pbuf], pair_mask);
+                tc_commit_pair_elect(&ctl->pv_done[pbuf], pair_mask);
             };
-            auto qk_tile = [&](int t) -> bool {
-                const int kst = t % kQ8KStages, sbuf = t % 3;
-                bool good = mbar_wait(&ctl->k_full[kst], (t / kQ8KStages) & 1) &&
-                            (t < 3 || mbar_wait(&ctl->s_empty[sbuf], ((t / 3) - 1) & 1));
-                good = __all_sync(0xffffffffu, good);
-                if (!good) return false;
-                tc_fence_after();
-                issue_qk(kst, sbuf);
-                return true;
-            };
-            auto pv_tile = [&](int i) -> bool {
-                const int vst = i % kQ8VStages, pbuf = i & 1;
-                bool good = mbar_wait(&ctl->p_full[pbuf], (i >> 1) & 1) && mbar_wait(&ctl->v_full[vst], (i / kQ8VStages) & 1);
-                good = __all_sync(0xffffffffu, good);
-                if (!good) return false;
-                tc_fence_after();
-                issue_pv(vst, pbuf, i == 0);
-                return true;
-            };
+            // as in tc2_decode_kernel: whatever is ready goes next, scores first
             bool ok = mbar_wait(&ctl->q_ready, 0);
             ok = __all_sync(0xffffffffu, ok);
             if (ok) tc_fence_after();
-            if (ok) ok = qk_tile(0);
-            if (ok && tiles_u > 1) ok = qk_tile(1);
-            for (int i = 0; ok && i < tiles_u; ++i) {
-                if (i + 2 < tiles_u) ok = qk_tile(i + 2);
-                if (ok) ok = pv_tile(i);
+            int t = 0, u = 0, vst = 0, vph = 0;
+            long long start = 0;
+            uint32_t idle = 0;
+            while (ok && u < units_u) {
+                const int sbuf = t & 1;
+                const bool qk = t < tiles_u && mbar_test(&ctl->k_full[sbuf], (t >> 1) & 1) && mbar_test(&ctl->s_empty[sbuf], ((t >> 1) & 1) ^ 1);
+                if (__all_sync(0xffffffffu, qk)) {
+                    tc_fence_after();
+                    issue_qk(sbuf, sbuf);
+                    ++t;
+                    idle = 0;
+                    continue;
+                }
+                const bool pv = mbar_test(&ctl->p_full, (u >> 1) & 1) && mbar_test(&ctl->v_full[vst], vph);
+                if (__all_sync(0xffffffffu, pv)) {
+                    tc_fence_after();
+                    issue_pv(vst, u & 1, u == 0);
+                    ++u;
+                    if (++vst == kQ8VStages) {
+                        vst = 0;
+                        vph ^= 1;
+                    }
+                    idle = 0;
+                    continue;
+                }
+                if ((++idle & 63u) == 0u) {
+                    const long long now = __shfl_sync(0xffffffffu, clock64(), 0);
+                    if (idle == 64u)
+                        start = now;
+                    else
+                        ok = now - start <= kWaitCycles;
+                    ok = ok && __shfl_sync(0xffffffffu, *abort_flag, 0) == 0u;
+                }
             }
             if (!ok && lane == 0) {
                 flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_MMA);
@@ -570,8 +633,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
         const int part = half * 2 + sub;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         const uint32_t s_empty_leader = map_to_rank(smem_u32(&ctl->s_empty[0]), leader);
-        const uint32_t p_full_leader0 = map_to_rank(smem_u32(&ctl->p_full[0]), leader);
-        const uint32_t p_full_leader1 = map_to_rank(smem_u32(&ctl->p_full[1]), leader);
+        const uint32_t p_full_leader = map_to_rank(smem_u32(&ctl->p_full), leader);
         bool ok = true;
         float a_row = 1.f;
         {
@@ -635,39 +697,46 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             a_row = aux->q_scale[row];
         }
         float m_ref = -INFINITY, l = 0.f;
+        // this thread: head row `row`, tokens [64 half + 32 sub, + 32) of every tile, i.e. quarter `part`
+        const float ac = a_row * p.scale_log2;
         for (int i = 0; ok && i < tiles; ++i) {
-            const int buf = i & 1, sbuf = i % 3, ring = i % kQ8ScaleRing;
-            ok = mbar_wait(&ctl->s_full[sbuf], (i / 3) & 1);
+            const int sbuf = i & 1, ring = i % kQ8Ring;
+            ok = mbar_wait(&ctl->s_full[sbuf], (i >> 1) & 1);
             if (!__all_sync(0xffffffffu, ok)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
-            uint32_t s8[16], sr[16];
-            tc_ld16(tmem + lane_base + kQ8ColS8 + 32 * sbuf + 16 * sub, s8);
-            tc_ld16(tmem + lane_base + kQ8ColSr + 32 * sbuf + 16 * sub, sr);
+            uint32_t s8[32], sr[32];
+            tc_ld32(tmem + lane_base + kQ8ColS8 + 64 * sbuf + 32 * sub, s8);
+            tc_ld32(tmem + lane_base + kQ8ColSr + 64 * sbuf + 32 * sub, sr);
             tc_wait_ld();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(s_empty_leader + 8 * sbuf);
-            const uint32_t valid = (uint32_t)(ctl->valid_mask[i % kQ8MaskRing] >> (16 * part)) & 0xffffu;
-            const float4 *ts = reinterpret_cast<const float4 *>(&aux->tok_scale[ring][16 * part]);
-            const float4 *tl = reinterpret_cast<const float4 *>(&aux->tok_log2[ring][16 * part]);
-            float y[16];
-            float mt = -INFINITY;
+            const uint32_t valid = (uint32_t)(ctl->valid_mask[ring][half] >> (32 * sub));
+            const float4 *ts = reinterpret_cast<const float4 *>(&aux->tok_scale[ring][32 * part]);
+            const float4 *tl = reinterpret_cast<const float4 *>(&aux->tok_log2[ring][32 * part]);
+            float y[32];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
+            for (int g = 0; g < 8; ++g) {
                 const float4 sc = ts[g], lg = tl[g];
                 const float scv[4] = {sc.x, sc.y, sc.z, sc.w}, lgv[4] = {lg.x, lg.y, lg.z, lg.w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int j = 4 * g + k;
-                    const float xv = (__uint_as_float(s8[j]) * (a_row * scv[k]) + __uint_as_float(sr[j])) * p.scale_log2;
-                    const bool on = (valid >> j) & 1u;
-                    y[j] = on ? xv + lgv[k] : -INFINITY;
-                    mt = fmaxf(mt, y[j]);
+                    y[j] = fmaf(__uint_as_float(s8[j]), ac * scv[k], fmaf(__uint_as_float(sr[j]), p.scale_log2, lgv[k]));
                 }
             }
+            if (valid != 0xffffffffu) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (!((valid >> j) & 1u)) y[j] = -INFINITY;
+            }
+            float mt4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int j = 0; j < 32; ++j) mt4[j & 3] = fmaxf(mt4[j & 3], y[j]);
+            float mt = fmaxf(fmaxf(mt4[0], mt4[1]), fmaxf(mt4[2], mt4[3]));
             ctl->xchg[i & 1][part][row] = mt;
             mbar_arrive(&ctl->x_bar);
             ok = mbar_wait(&ctl->x_bar, i & 1);
@@ -686,60 +755,61 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                 moved = true;
             }
             const float mr = (m_ref == -INFINITY) ? 0.f : m_ref;
-            const float4 *tr = reinterpret_cast<const float4 *>(&aux->tok_rcp[ring][16 * part]);
-            float sum = 0.f;
-            float pw[16];
+            const float4 *tr = reinterpret_cast<const float4 *>(&aux->tok_rcp[ring][32 * part]);
+            float sum[2] = {0.f, 0.f};
+            uint4 p_hi[2], p_lo[2];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const float4 rc = tr[g];
-                const float rcv[4] = {rc.x, rc.y, rc.z, rc.w};
+            for (int c = 0; c < 2; ++c) {
+                float pw[16];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int j = 4 * g + k;
-                    pw[j] = fast_exp2(y[j] - mr);                    // p * scale_t, below 448; 0 for a masked token
-                    sum += ((valid >> j) & 1u) ? pw[j] * rcv[k] : 0.f;      // p
+                for (int g = 0; g < 4; ++g) {
+                    const float4 rc = tr[4 * c + g];
+                    const float rcv[4] = {rc.x, rc.y, rc.z, rc.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int j = 4 * g + k;
+                        pw[j] = fast_exp2(y[16 * c + j] - mr);       // p * scale_t, below 448; 0 for a masked token
+                        sum[k & 1] = fmaf(pw[j], rcv[k], sum[k & 1]);   // p (a masked token repeats a selected row's scale)
+                    }
                 }
+                split_e4m3(pw, p_hi[c], p_lo[c]);
             }
-            l = l * factor + sum;
-            uint4 p_hi, p_lo;
-            split_e4m3(pw, p_hi, p_lo);
-            // the P buffer is free once P V of tile i-2 retired; O may be rescaled once P V of tile i-1 did
-            if (i >= 2) {
-                ok = mbar_wait(&ctl->p_free[buf], ((i >> 1) - 1) & 1);
+            l = l * factor + (sum[0] + sum[1]);
+            // P and O are free once P V of the tile before retired
+            if (i >= 1) {
+                ok = mbar_wait(&ctl->pv_done[1], (i - 1) & 1);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
                     break;
                 }
-            }
-            if (i >= 1 && __any_sync(0xffffffffu, moved)) {
-                ok = mbar_wait(&ctl->p_free[buf ^ 1], ((i - 1) >> 1) & 1);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
+                if (__any_sync(0xffffffffu, moved)) {
+                    tc_fence_after();
 #pragma unroll 1
-                for (int c = 0; c < 128; c += 32) {
-                    uint32_t ov[32];
-                    tc_ld32(tmem + lane_base + kColO + 128 * sub + c, ov);
-                    tc_wait_ld();
+                    for (int c = 0; c < 128; c += 32) {
+                        uint32_t ov[32];
+                        tc_ld32(tmem + lane_base + kColO + 128 * sub + c, ov);
+                        tc_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * factor);
-                    tc_st32(tmem + lane_base + kColO + 128 * sub + c, ov);
+                        for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * factor);
+                        tc_st32(tmem + lane_base + kColO + 128 * sub + c, ov);
+                    }
+                    tc_wait_st();
                 }
-                tc_wait_st();
             }
-            // this thread's 16 tokens: hi codes in 16-byte chunk `part`, lo codes in chunk 4 + part of the row
-            uint8_t *p_row = smem + kQ8SmemP + buf * kPanelBytes + row * 128;
-            *reinterpret_cast<uint4 *>(p_row + ((part ^ (row & 7)) << 4)) = p_hi;
-            *reinterpret_cast<uint4 *>(p_row + (((4 + part) ^ (row & 7)) << 4)) = p_lo;
+            // a P row of unit 2 i + half: hi codes of its 64 tokens in chunks 0-3, lo codes in chunks 4-7
+            uint8_t *p_row = smem + kQ8SmemP + half * kPanelBytes + row * 128;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                *reinterpret_cast<uint4 *>(p_row + (((2 * sub + c) ^ (row & 7)) << 4)) = p_hi[c];
+                *reinterpret_cast<uint4 *>(p_row + (((4 + 2 * sub + c) ^ (row & 7)) << 4)) = p_lo[c];
+            }
             fence_async_smem();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(buf ? p_full_leader1 : p_full_leader0);
+            if (lane == 0) mbar_arrive_cluster(p_full_leader);
         }
         if (ok) {
-            ok = mbar_wait(&ctl->p_free[(tiles - 1) & 1], ((tiles - 1) >> 1) & 1);
+            ok = mbar_wait(&ctl->pv_done[(units - 1) & 1], ((units - 1) >> 1) & 1);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (ok) {
@@ -931,11 +1001,11 @@ inline bool tc2q8_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cache
     if (cached)
         return cached_map(&maps[0], p.q, qrows, kTcHeads, 8, 1, encode_panel_map) &&
                cached_map(&maps[1], p.q, qrows, kTcHeads, 1, 1, encode_panel_map) &&
-               cached_map(&maps[2], p.kv, rows, 32, kQ8Panels, 2, encode_q8_panel_map) &&
+               cached_map(&maps[2], p.kv, rows, kTile, kQ8Panels, 2, encode_q8_panel_map) &&
                cached_map(&maps[3], p.kv, rows, kTile, 2, 2, encode_q8_panel_map) &&
                cached_map(&maps[4], p.kv, rows, kTile, kQ8Panels, 2, encode_q8_panel_map);
     return encode_panel_map(&maps[0], p.q, qrows, kTcHeads, 8) && encode_panel_map(&maps[1], p.q, qrows, kTcHeads, 1) &&
-           encode_q8_panel_map(&maps[2], p.kv, rows, 32, kQ8Panels) && encode_q8_panel_map(&maps[3], p.kv, rows, kTile, 2) &&
+           encode_q8_panel_map(&maps[2], p.kv, rows, kTile, kQ8Panels) && encode_q8_panel_map(&maps[3], p.kv, rows, kTile, 2) &&
            encode_q8_panel_map(&maps[4], p.kv, rows, kTile, kQ8Panels);
 }
 
