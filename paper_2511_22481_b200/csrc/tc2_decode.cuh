@@ -101,8 +101,9 @@ struct C2Control {
     uint32_t merge_flag;
     uint32_t xfail;                      // cluster merge: some wait of this CTA ran out (decided CTA-wide)
     int32_t k_progress;                  // units whose K loads have been requested (L2 prefetch pacing)
-    uint64_t recv_bar;                   // cluster merge: the partner's block has arrived
+    uint64_t recv_bar[4];                // cluster merge: the partner's chunks have arrived
     uint64_t ready_bar;                  // cluster merge: the partner's main loop is over
+    uint64_t taken_bar;                  // cluster merge: the partner's softmax warps have received this CTA's block
     uint64_t xg_bar;                     // row-maximum exchange of a tile
 };
 static_assert(sizeof(C2Control) <= kC2SmemCtlBytes, "control block too large");
@@ -128,15 +129,6 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
     // default (CTA-scope release) semantics: a cluster-scope release costs ~0.6 us per arrive here,
     // and what must be ordered before it is already ordered by the tcgen05 / async-proxy fences
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-
-// Execution-only rendezvous of the pair (no memory ordering): used before the tensor-memory
-// release, where the release-ordered form would first wait for every global store of the
-// epilogue to be acknowledged (about 9 us here).
-__device__ __forceinline__ void cluster_sync_relaxed()
-{
-    __syncwarp();                        // the aligned forms want whole warps
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 // Rendezvous of the cluster after the barriers were initialised.  The initialising thread has
@@ -278,13 +270,19 @@ __device__ __forceinline__ void tc_commit_pair_elect(uint64_t *bar, uint16_t bot
 // split 0 finishes value columns [0,128) and [256,384), split 1 the other two quarters: these are
 // the columns of softmax warps 2-5 and 8-11 in tensor memory, so in either CTA one warp per
 // scheduler is a "sender" (its columns are finished by the partner) and one a "keeper":
-//   1. the senders normalise their half by the row sums and write it, followed by the
-//      log-sum-exp of the split for every head row, to one block of shared memory, which four
-//      bulk shared-memory-to-shared-memory copies take to the partner, each as soon as its
-//      quarter of the block is written;
-//   2. the keepers wait for the partner's block, weigh their own half (still in tensor memory)
-//      and the received one by exp(lse_split - lse_total), add them and store bf16 rows as whole
-//      128-byte lines through warp-private staging tiles.
+//   1. the senders normalise their half by the row sums and write it to a block of shared memory, behind
+//      the log-sum-exp of the split for every head row, which four bulk shared-memory-to-shared-memory
+//      copies take to the partner, each as soon as its quarter of the block is written;
+//   2. every softmax warp finishes 64 columns of its tensor-memory lane quarter as the quarters of the
+//      partner's block come in (each has a barrier of its own): it weighs its own half (still in tensor
+//      memory) and the received one by exp(lse_split - lse_total), adds them and stores bf16 rows
+//      as whole 128-byte lines through warp-private staging tiles.
+// What bounds it: the block takes about 4000 clocks through the network between SMs (17 bytes a clock), so
+// everything else overlaps it; with one barrier for the whole block, and the cluster's last
+// rendezvous behind the stores, the exchange took 7800 clocks after the later main loop, now 5800 (28.2 ->
+// 27.6 us per step of 32 requests x 33 units).  Its barriers are mbarriers: an aligned cluster barrier in
+// one branch of the kernel makes the compiler give up warp uniformity everywhere, 11 KB more code and
+// a main loop 1.6 times slower.
 // The copy lands in shared memory that held the partner's operand tiles, so it is not sent
 // before the partner has said that its main loop is over (`ready_bar`, a remote arrive that the
 // partner fires as soon as its last P V has retired, while this CTA is still staging).
@@ -294,12 +292,13 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
                                                        uint32_t tmem, int b, int s, uint32_t crank, int h0,
                                                        int head_rows, bool active, bool main_ok, float cm_lse, float cm_inv)
 {
-    // The block travels as four chunks, so that the copy of one overlaps the staging of the next:
-    // chunk q holds, for every head row, the q-th 32 columns of both 128-column runs that are sent.
+    // The block travels as four chunks, so that the copy of one overlaps the staging of the next and the mixing
+    // of the one before: chunk q holds, for every head row, the q-th 32 columns of both 128-column runs
+    // that are sent.  The log-sum-exps go with the first.
     constexpr uint32_t kChunkPitch = 2 * 128 + 16;       // row-per-lane 16-byte accesses do not conflict
     constexpr uint32_t kChunkBytes = 64 * kChunkPitch;   // 17,408
-    constexpr uint32_t kRowsBytes = 4 * kChunkBytes;
-    constexpr uint32_t kBlockBytes = kRowsBytes + 256;   // + 64 log-sum-exps: 69,888
+    constexpr uint32_t kLseBytes = 256;
+    constexpr uint32_t kBlockBytes = kLseBytes + 4 * kChunkBytes;      // 69,888
     constexpr uint32_t kStagePitch = 144, kStageBytes = 32 * kStagePitch;
     static_assert(2 * kBlockBytes + 8 * kStageBytes <= 221184, "exchange tiles must end below the control block and the 8-bit kernel's auxiliary arrays");
     uint8_t *send = smem, *stages = smem + kBlockBytes, *recv = smem + kBlockBytes + 8 * kStageBytes;
@@ -324,8 +323,22 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
     tc_fence_after();
     if (sub != s) {
         // ---- sender: this thread's 128 value columns are finished by the other split ----------
-        if (half == 0) reinterpret_cast<float *>(send + kRowsBytes)[row] = cm_lse;
-        bool ready = true;                                // (sending warp) the partner's operand tiles are dead
+        if (half == 0) reinterpret_cast<float *>(send)[row] = cm_lse;
+        // (sending warp) chunks go out as soon as they are staged and the partner's operand tiles are dead; a
+        // split that finishes first has staged all of them by the time it hears that
+        int sent = 0;
+        auto send_chunks = [&](int upto) {
+#pragma unroll 1
+            for (; sent <= upto; ++sent) {
+                const uint32_t from = sent == 0 ? 0u : kLseBytes + sent * kChunkBytes, bytes = kChunkBytes + (sent == 0 ? kLseBytes : 0u);
+                const uint32_t dst = map_to_rank(smem_u32(recv + from), partner);
+                const uint32_t bar = map_to_rank(smem_u32(&ctl->recv_bar[sent]), partner);
+                if (lane == 0)
+                    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(dst), "r"(smem_u32(send + from)), "r"(bytes), "r"(bar)
+                                 : "memory");
+            }
+        };
 #pragma unroll 1
         for (int q = 0; q < 4; ++q) {
             uint32_t ov[32];
@@ -334,7 +347,7 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
                 tc_ld32(tmem + lane_base + kColO + 128 * sub + q * 32, ov);
                 tc_wait_ld();
             }
-            uint4 *o = reinterpret_cast<uint4 *>(send + q * kChunkBytes + (size_t)row * kChunkPitch + half * 128);
+            uint4 *o = reinterpret_cast<uint4 *>(send + kLseBytes + q * kChunkBytes + (size_t)row * kChunkPitch + half * 128);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 // an empty or fully masked split contributes exact zeros
@@ -347,45 +360,38 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
             }
             fence_async_smem();                           // the bulk copy reads what the threads wrote
             asm volatile("bar.sync 2, 128;" ::: "memory"); // the four sending warps
-            if (quarter == 0) {
-                if (q == 0) {
-                    ready = mbar_wait(&ctl->ready_bar, 0);
-                    ready = __all_sync(0xffffffffu, ready);
-                    if (!ready && lane == 0) {
-                        *xfail = 1u;
-                        flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_SOFTMAX);
-                    }
-                }
-                if (ready && lane == 0) {
-                    const uint32_t bytes = q == 3 ? kChunkBytes + 256 : kChunkBytes;       // the last one takes the log-sum-exps along
-                    const uint32_t dst = map_to_rank(smem_u32(recv + q * kChunkBytes), partner);
-                    const uint32_t bar = map_to_rank(smem_u32(&ctl->recv_bar), partner);
-                    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(dst), "r"(smem_u32(send + q * kChunkBytes)), "r"(bytes), "r"(bar)
-                                 : "memory");
-                }
+            if (quarter == 0 && __all_sync(0xffffffffu, mbar_test(&ctl->ready_bar, 0))) send_chunks(q);
+        }
+        if (quarter == 0 && sent < 4) {
+            bool ready = mbar_wait(&ctl->ready_bar, 0);
+            ready = __all_sync(0xffffffffu, ready);
+            if (ready) send_chunks(3);
+            if (!ready && lane == 0) {
+                *xfail = 1u;
+                flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_SOFTMAX);
             }
         }
     } else if (quarter == 0 && lane == 0) {
-        mbar_expect_tx(&ctl->recv_bar, kBlockBytes);
+        for (int q = 0; q < 4; ++q) mbar_expect_tx(&ctl->recv_bar[q], kChunkBytes + (q == 0 ? kLseBytes : 0u));
     }
 
     // ---- finish: the columns kept here (those of the warps with sub == s) never left tensor
-    // memory.  Once the partner's block is in, all eight warps take part: a warp can read any
-    // column of its tensor-memory lane quarter, so the keeping warp of a quarter finishes the
-    // first 64 of its 128 columns and the sending warp of the same quarter, its block gone, the
-    // other 64.  A thread mixes its accumulator row with the received one and the warp writes the
-    // bf16 rows out as whole 128-byte lines through its private staging tile.
-    {
-        bool got = mbar_wait(&ctl->recv_bar, 0);
+    // memory.  All eight warps take part: a warp can read any column of its tensor-memory lane
+    // quarter, so the keeping warp of a quarter finishes the first 64 of its 128 columns (chunks 0 and 1)
+    // and the sending warp of the same quarter, its block gone, the other 64 (chunks 2 and 3).  A thread
+    // mixes its accumulator row with the received one and the warp writes the bf16 rows out as
+    // whole 128-byte lines through its private staging tile.
+    auto received = [&](int q) {
+        bool got = mbar_wait(&ctl->recv_bar[q], 0);
         got = __all_sync(0xffffffffu, got);
         if (!got && lane == 0) {
             *xfail = 1u;
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_SOFTMAX);
         }
-    }
+    };
+    received(0);
     // weights of the two splits for this head row, final log-sum-exp
-    const float other = reinterpret_cast<const float *>(recv + kRowsBytes)[row];
+    const float other = reinterpret_cast<const float *>(recv)[row];
     const float mx = fmaxf(cm_lse, other);
     float total = -INFINITY, w_own = 0.f, w_other = 0.f;
     if (mx > -INFINITY) {
@@ -403,11 +409,13 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
     const int row0 = (quarter & 1) * 32;                                  // first head row of this warp
     uint8_t *gq = reinterpret_cast<uint8_t *>(p.out + ((size_t)b * p.heads + h0 + row0) * kDv + half * 256 + col);
     const int rows_here = max(0, min(32, head_rows - row0));
-    const uint8_t *theirs = recv + (sub == s ? 0 : 2) * kChunkBytes + (size_t)row * kChunkPitch + half * 128;
+    const int first_chunk = sub == s ? 0 : 2;
+    const uint8_t *theirs = recv + kLseBytes + first_chunk * kChunkBytes + (size_t)row * kChunkPitch + half * 128;
     uint4 *mine = reinterpret_cast<uint4 *>(buf + lane * kStagePitch);
     tc_fence_after();
-#pragma unroll
+#pragma unroll 1
     for (int c2 = 0; c2 < 2; ++c2) {
+        received(first_chunk + c2);
         uint32_t ov[32];
         if (use_own) {
             tc_ld32(tmem + lane_base + kColO + col + c2 * 32, ov);
@@ -429,6 +437,9 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
             mine[c2 * 4 + j] = w;
         }
     }
+    // this warp has seen its chunks land: once all eight have said so, the partner may leave
+    __syncwarp();
+    if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&ctl->taken_bar), partner));
     __syncwarp();
     uint4 v[8];
 #pragma unroll
@@ -623,8 +634,9 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         mbar_init(&ctl->xg_bar, 256);
         mbar_init(&ctl->x_bar, 256);
         mbar_init(&ctl->exit_bar, 2);
-        mbar_init(&ctl->recv_bar, 1);
+        for (int i = 0; i < 4; ++i) mbar_init(&ctl->recv_bar[i], 1);
         mbar_init(&ctl->ready_bar, 1);
+        mbar_init(&ctl->taken_bar, 8);
         ctl->abort = 0;
         ctl->xfail = 0;
         ctl->k_progress = 0;
@@ -1235,13 +1247,13 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     }
     if (warp == 1) {
         mbar_wait(&ctl->exit_bar, 0);
+        // the bulk copies sent to the partner read this CTA's shared memory: it has to stay until they are in
+        // (a cluster barrier here would wait for the partner's last stores too)
+        if (kClusterMerge) mbar_wait(&ctl->taken_bar, 0);
         __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
-    // the bulk copy a CTA sent to its partner reads this CTA's shared memory: nobody leaves
-    // before every CTA of the cluster has received its block
-    if (kClusterMerge) cluster_sync_relaxed();
     // ---- split merge by whichever CTA finishes a (request, head half) last ---------------
     if (!kClusterMerge && p.splits > 1 && p.counters != nullptr)
         merge_if_last(p, b, (int)rank, 2, h0, head_rows, reinterpret_cast<float *>(smem), &ctl->merge_flag);

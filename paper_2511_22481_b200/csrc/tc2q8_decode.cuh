@@ -91,8 +91,9 @@ struct Q8Control {
     uint64_t pv_done[2];                 // P V of a unit retired: its P unit may be rewritten, O may be rescaled
     uint64_t x_bar;
     uint64_t exit_bar;
-    uint64_t recv_bar;
+    uint64_t recv_bar[4];
     uint64_t ready_bar;
+    uint64_t taken_bar;
     uint64_t valid_mask[kQ8Ring][2];     // [tile][unit]
     float xchg[2][4][64];
     uint32_t tmem_base;
@@ -240,8 +241,9 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
         mbar_init(&ctl->p_full, 16);
         mbar_init(&ctl->x_bar, 256);
         mbar_init(&ctl->exit_bar, 2);
-        mbar_init(&ctl->recv_bar, 1);
+        for (int i = 0; i < 4; ++i) mbar_init(&ctl->recv_bar[i], 1);
         mbar_init(&ctl->ready_bar, 1);
+        mbar_init(&ctl->taken_bar, 8);
         ctl->abort = 0;
         ctl->xfail = 0;
         ctl->k_progress = 0;
@@ -851,11 +853,11 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
     }
     if (warp == 1) {
         mbar_wait(&ctl->exit_bar, 0);
+        if (kClusterMerge) mbar_wait(&ctl->taken_bar, 0);
         __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
-    if (kClusterMerge) cluster_sync_relaxed();
     if (!kClusterMerge && p.splits > 1 && p.counters != nullptr)
         merge_if_last(p, b, (int)rank, 2, h0, head_rows, reinterpret_cast<float *>(smem), &ctl->merge_flag);
 }
