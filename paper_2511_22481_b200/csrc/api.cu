@@ -104,38 +104,47 @@ bool merge_in_cluster(const omni_mla_desc_t *d, int splits, int resident_merge_c
     return d->batch <= resident_merge_clusters;
 }
 
-// Pick the number of split-KV partitions per request.  The kernel's work units run in waves over
-// the SMs.  In units of one tile time (64 tokens), as measured: a unit costs a fixed part of about
-// 6 (set-up, first-tile latency, epilogue) plus one per granule; a unit that writes fp32 partial
-// results to global memory for a later merge costs about 6 more when the grid runs in several
-// waves (256 KiB written and read back against 72 KiB per tile; about 2 within one wave, where
-// they stay in L2), and so does the merge kernel at the end.  Two splits merged inside a
-// cluster of two CTA pairs avoid the partial results and pay about 5 for the exchange.  A tile of the
-// single-CTA kernel takes twice as long, and the merge of its few heads about 4.
-// Minimise waves * (granules per unit + fixed parts) + merge.
+// Pick the number of split-KV partitions per request: minimise waves * (units per split + fixed part) + merge.
+// The kernel's work runs in waves over the SMs, and the unit of cost is the time of 64 tokens (0.65 to
+// 0.9 us, by how many pairs read).  Fitted to 460 measured (heads, batch, units, splits), whole pages
+// and scattered tokens, which the host cannot tell apart:
+//  * two splits merged inside a cluster of two CTA pairs cost about 3.5;
+//  * partial results in global memory and the merge kernel cost about 8 (its launch, latencies), and from 24
+//    partial results on a sixteenth more for each of them (up to 256 KiB written and read back);
+//    5.5 more per wave when there are several, since the partials then compete with the next wave's loads;
+//  * a unit of the single-CTA kernel takes twice as long, and the merge of its few heads costs 5.5.
+// Before, the merge kernel counted as 8 whatever the number of partials and the cluster merge as 5: 4 requests
+// of 16 units ran in 16 splits (17.6 us) instead of 8 (13.3), 16 of them in 4 (17.6) instead of 2 (13.8),
+// 24 x 33 in 3 (26.6) instead of 2 (22.3), 6 x 12 in 16.4 us instead of 11.4.  Up to 8 units a pair keeps a
+// request whole (one launch without any merge).
 int choose_splits(const omni_mla_desc_t *d, int sm_count, int resident_merge_clusters = -1)
 {
     if (d->num_splits >= 1) return d->num_splits;
     if (sm_count <= 0) sm_count = 148;
-    const int granule = use_pair_kernel(d) ? kC2Tile : kTile;
+    constexpr long kUnit = 16;                           // costs are in sixteenths of a unit
+    constexpr int kWholeUnits = 8;
+    const bool pair = use_pair_kernel(d), single = !pair && !(d->flags & OMNI_FLAG_SIMT);
+    const int granule = pair ? kC2Tile : kTile;
     const int granules = (d->max_sel + granule - 1) / granule;
     const long units = (long)d->batch * units_per_request(d);
-    if (use_pair_kernel(d)) sm_count /= 2;               // a work unit occupies two SMs
-    const bool single = !use_pair_kernel(d) && !(d->flags & OMNI_FLAG_SIMT);
+    if (pair) sm_count /= 2;                             // a work unit occupies two SMs
+    const int most = pair && granules <= kWholeUnits ? 1 : kMaxSplits;
     long best_cost = -1;
     int best = 1;
-    for (int s = 1; s <= kMaxSplits && s <= granules; ++s) {
+    for (int s = 1; s <= most && s <= granules; ++s) {
         const long waves = (units * s + sm_count - 1) / sm_count;
         const long per = (granules + s - 1) / s;
         long cost;
-        if (s == 1)
-            cost = waves * ((single ? 2 * per : per) + 6);
-        else if (merge_in_cluster(d, s, resident_merge_clusters))
-            cost = waves * (per + 6) + 5;
-        else if (single)
-            cost = waves * (2 * per + 6 + (waves > 1 ? 6 : 2)) + 4;
+        if (single)
+            cost = waves * (2 * per + 6 + (s > 1 && waves > 1 ? 4 : 0)) * kUnit + (s > 1 ? 88 : 0);
         else
-            cost = waves * (per + 6 + (waves > 1 ? 6 : 2)) + 6;     // partial results stay in L2 within one wave
+            cost = waves * (per + 2) * kUnit;
+        if (!single && s > 1) {
+            if (merge_in_cluster(d, s, resident_merge_clusters))
+                cost += 56;
+            else
+                cost += 124 + std::max(0l, units * s - 24) + (waves > 1 ? 88 * waves : 0);
+        }
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = s;

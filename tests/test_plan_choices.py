@@ -1,0 +1,26 @@
+"""The split plan where it weighs a merge in a cluster, the merge kernel and the number of partial results
+against each other (148 SMs, 33 resident merging clusters).  The counts are the fastest, or within 4 % of
+it, of all those measured at the shape."""
+import math
+
+import pytest
+
+from paper_2511_22481_b200 import binding as B
+from paper_2511_22481_b200 import build as builder
+
+
+@pytest.mark.parametrize("batch,heads,units,want", [
+    (4, 128, 8, (1, 1)),        # the longest request that is never cut
+    (4, 128, 9, (2, 1)),        # the shortest that is
+    (16, 128, 16, (2, 1)), (24, 128, 33, (2, 1)),
+    (33, 128, 33, (2, 1)),      # the last batch whose clusters are all resident
+    (34, 128, 12, (1, 1)),      # the first whose are not
+    (4, 128, 16, (8, 2)),       # few partial results
+    (36, 128, 64, (2, 2)),      # partial results pay all the same
+    (48, 128, 64, (1, 1)),
+    (4, 16, 4, (4, 2)),         # single-CTA kernel
+])
+def test_split_choice(batch, heads, units, want):
+    builder.build()
+    d = B.make_desc(batch, heads, batch * units, units, units * 64, 1.0 / math.sqrt(192.0))
+    assert B.omni_sparse_mla_plan_query(d, 148, 33) == want
