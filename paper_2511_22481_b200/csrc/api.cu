@@ -414,6 +414,8 @@ static omni_status_t check_step_args(const omni_mla_desc_t *desc, const int32_t 
     return OMNI_OK;
 }
 
+constexpr int kNoWorkspaceTokens = 11 * kPage;
+
 // The per-call half: pointer checks, workspace carving, launches.  The selection is an index
 // list (sel_idx, sel_len) or, with sel_idx == nullptr, Eq. 2's ranges (ctx_len, n_sink, n_recent).
 static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table, const int32_t *sel_idx,
@@ -425,7 +427,10 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
     const bool ranges = sel_idx == nullptr;
     omni_status_t args = check_step_args(desc, page_table, sel_idx, sel_len, ctx_len, n_sink, n_recent, rolling, out, lse);
     if (args != OMNI_OK) return args;
-    const int splits = plan.splits;
+    // A short selection that the plan would cut also runs whole, for callers who bring no workspace
+    const bool whole = !workspace && desc->num_splits == 0 && desc->max_sel <= kNoWorkspaceTokens;
+    const int splits = whole ? 1 : plan.splits;
+    const bool cluster_merge = !whole && plan.cluster_merge, fused_merge = !whole && plan.fused_merge;
     if (splits > 1) {
         if (!workspace) return OMNI_ERR_NULL;
         if (!aligned(workspace, 256)) return OMNI_ERR_ALIGN;
@@ -456,9 +461,9 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
     p.part_lse = splits > 1 ? reinterpret_cast<float *>(static_cast<char *>(workspace) + plan.part_out) : nullptr;
     p.status = device_status;
     p.counters = nullptr;
-    p.cluster_merge = plan.cluster_merge;
+    p.cluster_merge = cluster_merge ? 1 : 0;
     p.longest_first = plan.longest_first;
-    if (plan.fused_merge) {
+    if (fused_merge) {
         p.counters = reinterpret_cast<int32_t *>(static_cast<char *>(workspace) + plan.part_out + plan.part_lse);
         if (cudaMemsetAsync(p.counters, 0, plan.counters, stream) != cudaSuccess) return OMNI_ERR_CUDA;
     }

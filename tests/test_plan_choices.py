@@ -4,6 +4,7 @@ it, of all those measured at the shape."""
 import math
 
 import pytest
+import torch
 
 from paper_2511_22481_b200 import binding as B
 from paper_2511_22481_b200 import build as builder
@@ -24,3 +25,19 @@ def test_split_choice(batch, heads, units, want):
     builder.build()
     d = B.make_desc(batch, heads, batch * units, units, units * 64, 1.0 / math.sqrt(192.0))
     assert B.omni_sparse_mla_plan_query(d, 148, 33) == want
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("batch,heads,units", [(4, 128, 9), (3, 128, 11), (4, 16, 4)])
+def test_short_selections_need_no_workspace(batch, heads, units):
+    """Without a workspace the requests stay whole: the bits of one forced split."""
+    from paper_2511_22481_b200 import workloads as W
+    w = W.token_topk("short", 5, batch, heads, 32, units * 64, "cuda")
+    ref = B.plan_for(w, num_splits=1)
+    ref.run(w.q, w.kv_cache, w.page_table, w.sel_idx, w.sel_len)
+    d = B.plan_for(w)
+    assert d.splits > 1
+    out, lse = torch.full_like(ref.out, float("nan")), torch.full_like(ref.lse, float("nan"))
+    B.omni_sparse_mla_decode(d.desc, w.q, w.kv_cache, w.page_table, w.sel_idx, w.sel_len, out, lse)
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref.out) and torch.equal(lse, ref.lse)
