@@ -117,12 +117,15 @@ bool merge_in_cluster(const omni_mla_desc_t *d, int splits, int resident_merge_c
 // of 16 units ran in 16 splits (17.6 us) instead of 8 (13.3), 16 of them in 4 (17.6) instead of 2 (13.8),
 // 24 x 33 in 3 (26.6) instead of 2 (22.3), 6 x 12 in 16.4 us instead of 11.4.  Up to 8 units a pair keeps a
 // request whole (one launch without any merge).
-int choose_splits(const omni_mla_desc_t *d, int sm_count, int resident_merge_clusters = -1)
+struct SplitPlan {
+    int splits, whole;
+};
+SplitPlan split_plan(const omni_mla_desc_t *d, int sm_count, int resident_merge_clusters = -1)
 {
-    if (d->num_splits >= 1) return d->num_splits;
+    if (d->num_splits >= 1) return {d->num_splits, 0};
     if (sm_count <= 0) sm_count = 148;
     constexpr long kUnit = 16;                           // costs are in sixteenths of a unit
-    constexpr int kWholeUnits = 8;
+    constexpr int kWholeUnits = 8, kTailUnits = 64;
     const bool pair = use_pair_kernel(d), single = !pair && !(d->flags & OMNI_FLAG_SIMT);
     const int granule = pair ? kC2Tile : kTile;
     const int granules = (d->max_sel + granule - 1) / granule;
@@ -150,30 +153,50 @@ int choose_splits(const omni_mla_desc_t *d, int sm_count, int resident_merge_clu
             best = s;
         }
     }
-    return best;
+    // One wave of whole requests and a few more: whole, these would keep at most a third of the pairs busy for as
+    // long again, so they are cut into as many pieces as there are pairs.  80 requests x 64 units 134 -> 95 us, 98
+    // x 64 143 -> 117, 76 x 128 225 -> 165.  Where the sizes differ so much that the few run beside the longest ones the
+    // kernel takes them whole after all (c2_request_by_length_rank) and the merge kernel finds nothing to do.  That costs
+    // 2 to 4 us (67 us where sizes run from 8 to 64 units), so the line lies at 64 units.
+    const int tail = d->batch - sm_count;
+    if (pair && tail > 0 && 3 * tail <= sm_count && granules >= kTailUnits && !(d->flags & OMNI_FLAG_FUSED_MERGE)) {
+        const int pieces = std::min(kMaxSplits, sm_count / tail), per = std::max(2, (granules + pieces - 1) / pieces);
+        const int s = (granules + per - 1) / per;
+        const long cost = (granules + 2 + per + 2) * kUnit + 212 + std::max(0, tail * s - 24);
+        if (s > 1 && d->batch <= 256 && cost < best_cost) return {s, sm_count};
+    }
+    return {best, 0};
+}
+
+// Splits of every request, as the queries report them (1 if only the last few are cut).
+int choose_splits(const omni_mla_desc_t *d, int sm_count, int resident_merge_clusters = -1)
+{
+    const SplitPlan plan = split_plan(d, sm_count, resident_merge_clusters);
+    return plan.whole > 0 ? 1 : plan.splits;
 }
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-size_t part_out_bytes(const omni_mla_desc_t *d, int splits)
+size_t part_out_bytes(const omni_mla_desc_t *d, const SplitPlan &plan)
 {
-    return align_up((size_t)d->batch * splits * d->num_heads * kDv * sizeof(float), 256);
+    return align_up((size_t)(d->batch - plan.whole) * plan.splits * d->num_heads * kDv * sizeof(float), 256);
 }
 
-size_t part_lse_bytes(const omni_mla_desc_t *d, int splits)
+size_t part_lse_bytes(const omni_mla_desc_t *d, const SplitPlan &plan)
 {
-    return align_up((size_t)d->batch * splits * d->num_heads * sizeof(float), 256);
+    return align_up((size_t)(d->batch - plan.whole) * plan.splits * d->num_heads * sizeof(float), 256);
 }
 
-// Arrival counters of the in-kernel merge: one per (request, CTA of a pair).
+// Arrival counters of the in-kernel merge: one per (request, CTA of a pair); where only the last requests are cut,
+// which ones these are.
 size_t counter_bytes(const omni_mla_desc_t *d)
 {
     return align_up((size_t)d->batch * 2 * sizeof(int32_t), 256);
 }
 
-size_t workspace_need(const omni_mla_desc_t *d, int splits)
+size_t workspace_need(const omni_mla_desc_t *d, const SplitPlan &plan)
 {
-    return part_out_bytes(d, splits) + part_lse_bytes(d, splits) + counter_bytes(d);
+    return part_out_bytes(d, plan) + part_lse_bytes(d, plan) + counter_bytes(d);
 }
 
 // On request the paired-CTA kernel merges the splits itself (the last CTA to finish a request's
@@ -203,7 +226,7 @@ omni_status_t launch_overlapped(void (*kernel)(KernelArgs...), unsigned blocks, 
 }
 
 omni_status_t launch_combine(int batch, int heads, int max_splits, const float *part_out,
-                             const float *part_lse, const int32_t *num_splits, void *out,
+                             const float *part_lse, const int32_t *num_splits, const int32_t *request, void *out,
                              float *lse, cudaStream_t stream)
 {
     // Keep the shared-memory / L1 split the decode kernel needs: alternating between two splits
@@ -219,7 +242,7 @@ omni_status_t launch_combine(int batch, int heads, int max_splits, const float *
     const int blocks = batch * heads;
     const bool wide = max_splits > kCombineAhead && blocks <= 3 * device_info().sm_count;
     return launch_overlapped(wide ? combine_kernel<4> : combine_kernel<1>, (unsigned)blocks, wide ? 512 : 128, stream, part_out,
-                             part_lse, num_splits, max_splits, heads, static_cast<__nv_bfloat16 *>(out), lse);
+                             part_lse, num_splits, request, max_splits, heads, static_cast<__nv_bfloat16 *>(out), lse);
 }
 
 omni_status_t launch_resolve(const omni_mla_desc_t *d, const int32_t *page_table,
@@ -295,8 +318,10 @@ int32_t omni_sparse_mla_num_splits(const omni_mla_desc_t *desc)
 int32_t omni_sparse_mla_num_launches(const omni_mla_desc_t *desc)
 {
     if (!desc_ok(desc)) return 0;
-    const int s = choose_splits(desc, device_info().sm_count);
+    const SplitPlan plan = split_plan(desc, device_info().sm_count);
+    const int s = plan.splits;
     int n = 1 + ((desc->flags & OMNI_FLAG_VALIDATE) ? 1 : 0);
+    if (plan.whole > 0) return n + 1;
     if (s > 1 && !merge_in_cluster(desc, s) && !(use_pair_kernel(desc) && (desc->flags & OMNI_FLAG_FUSED_MERGE))) ++n;
     return n;
 }
@@ -305,9 +330,11 @@ int32_t omni_sparse_mla_plan_query(const omni_mla_desc_t *desc, int32_t sm_count
                                    int32_t *num_launches)
 {
     if (!desc_ok(desc) || sm_count < 1 || resident_merge_clusters < 0) return 0;
-    const int s = choose_splits(desc, sm_count, resident_merge_clusters);
+    const SplitPlan plan = split_plan(desc, sm_count, resident_merge_clusters);
+    const int s = plan.whole > 0 ? 1 : plan.splits;
     if (num_launches) {
         int n = 1 + ((desc->flags & OMNI_FLAG_VALIDATE) ? 1 : 0);
+        if (plan.whole > 0) ++n;
         if (s > 1 && !merge_in_cluster(desc, s, resident_merge_clusters) &&
             !(use_pair_kernel(desc) && (desc->flags & OMNI_FLAG_FUSED_MERGE)))
             ++n;
@@ -319,7 +346,7 @@ int32_t omni_sparse_mla_plan_query(const omni_mla_desc_t *desc, int32_t sm_count
 size_t omni_sparse_mla_workspace_bytes(const omni_mla_desc_t *desc)
 {
     if (!desc_ok(desc)) return 0;
-    return workspace_need(desc, choose_splits(desc, device_info().sm_count));
+    return workspace_need(desc, split_plan(desc, device_info().sm_count));
 }
 
 // Everything about a decode call that depends only on the descriptor, q and the pool: which
@@ -330,7 +357,7 @@ constexpr uint32_t kPlanMagic = 0x4c504d4fu;
 struct LaunchPlan {
     uint32_t magic;
     int32_t kernel;            // 0 plain-FMA, 1 single-CTA tensor-core, 2 paired-CTA tensor-core, 3 the same over the 8-bit cache
-    int32_t splits;
+    int32_t splits, whole;     // the first `whole` requests are not split
     int32_t cluster_merge, longest_first, fused_merge;
     int32_t device;
     size_t need, part_out, part_lse, counters;
@@ -358,15 +385,17 @@ static omni_status_t build_plan(const omni_mla_desc_t *desc, const void *q, cons
     plan->kv_scale = kv_scale;
     plan->device = dev.index;
     plan->kernel = q8 ? 3 : (desc->flags & OMNI_FLAG_SIMT) ? 0 : use_pair_kernel(desc) ? 2 : 1;
-    const int splits = choose_splits(desc, dev.sm_count);
+    const SplitPlan cut = split_plan(desc, dev.sm_count);
+    const int splits = cut.splits;
     plan->splits = splits;
-    plan->part_out = part_out_bytes(desc, splits);
-    plan->part_lse = part_lse_bytes(desc, splits);
+    plan->whole = cut.whole;
+    plan->part_out = part_out_bytes(desc, cut);
+    plan->part_lse = part_lse_bytes(desc, cut);
     plan->counters = counter_bytes(desc);
-    plan->need = workspace_need(desc, splits);
+    plan->need = workspace_need(desc, cut);
     // Two splits of a request can be merged inside a cluster of two CTA pairs, without partial
     // results in global memory, as long as all those clusters are resident at once.
-    plan->cluster_merge = merge_in_cluster(desc, splits) ? 1 : 0;
+    plan->cluster_merge = (cut.whole == 0 && merge_in_cluster(desc, splits)) ? 1 : 0;
     plan->fused_merge = (splits > 1 && merge_in_kernel(desc)) ? 1 : 0;
     // several waves of work units: start the longest requests first (the kernel ranks them itself)
     plan->longest_first = (plan->kernel >= 2 && !plan->cluster_merge && desc->batch <= 256 &&
@@ -428,7 +457,7 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
     omni_status_t args = check_step_args(desc, page_table, sel_idx, sel_len, ctx_len, n_sink, n_recent, rolling, out, lse);
     if (args != OMNI_OK) return args;
     // A short selection that the plan would cut also runs whole, for callers who bring no workspace
-    const bool whole = !workspace && desc->num_splits == 0 && desc->max_sel <= kNoWorkspaceTokens;
+    const bool whole = !workspace && desc->num_splits == 0 && (desc->max_sel <= kNoWorkspaceTokens || plan.whole > 0);
     const int splits = whole ? 1 : plan.splits;
     const bool cluster_merge = !whole && plan.cluster_merge, fused_merge = !whole && plan.fused_merge;
     if (splits > 1) {
@@ -461,6 +490,8 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
     p.part_lse = splits > 1 ? reinterpret_cast<float *>(static_cast<char *>(workspace) + plan.part_out) : nullptr;
     p.status = device_status;
     p.counters = nullptr;
+    p.whole = whole ? 0 : plan.whole;
+    p.tail_request = p.whole > 0 ? reinterpret_cast<int32_t *>(static_cast<char *>(workspace) + plan.part_out + plan.part_lse) : nullptr;
     p.cluster_merge = cluster_merge ? 1 : 0;
     p.longest_first = plan.longest_first;
     if (fused_merge) {
@@ -490,7 +521,7 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
     if (st != OMNI_OK) return st;
     if (profile) cudaEventRecord(g_profile_after, stream);
     if (splits > 1 && p.counters == nullptr && !p.cluster_merge)
-        return launch_combine(desc->batch, desc->num_heads, splits, p.part_out, p.part_lse, nullptr,
+        return launch_combine(desc->batch - p.whole, desc->num_heads, splits, p.part_out, p.part_lse, nullptr, p.tail_request,
                               out, lse, stream);
     return OMNI_OK;
 }
@@ -645,7 +676,7 @@ omni_status_t omni_sparse_mla_combine(const omni_mla_desc_t *desc, int32_t max_s
         return OMNI_ERR_SHAPE;
     if (!aligned(part_out, 16) || !aligned(out, 8) || !aligned(part_lse, 4) || !aligned(lse, 4))
         return OMNI_ERR_ALIGN;
-    return launch_combine(desc->batch, desc->num_heads, max_splits, part_out, part_lse, num_splits,
+    return launch_combine(desc->batch, desc->num_heads, max_splits, part_out, part_lse, num_splits, nullptr,
                           out, lse, static_cast<cudaStream_t>(stream));
 }
 
@@ -719,7 +750,7 @@ static omni_mla_desc_t host_half_desc(const omni_mla_desc_t *desc, int half)
 static size_t host_half_workspace(const omni_mla_desc_t *desc, int half)
 {
     const omni_mla_desc_t d = host_half_desc(desc, half);
-    return align_up(workspace_need(&d, choose_splits(&d, device_info().sm_count)), 256);
+    return align_up(workspace_need(&d, split_plan(&d, device_info().sm_count)), 256);
 }
 
 // Side streams of the host-buffer entry point: a few per device, chosen by the caller's stream, so
@@ -772,7 +803,7 @@ static size_t host_part_workspace(const omni_mla_desc_t *desc)
     for (int i = 0; i < n; ++i) {
         omni_mla_desc_t d = *desc;
         d.batch = size[i];
-        const size_t w = workspace_need(&d, choose_splits(&d, device_info().sm_count));
+        const size_t w = workspace_need(&d, split_plan(&d, device_info().sm_count));
         need = w > need ? w : need;
     }
     return align_up(need, 256);

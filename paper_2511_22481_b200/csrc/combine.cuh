@@ -19,6 +19,7 @@ template <int kGroups>
 __global__ void __launch_bounds__(128 * kGroups) combine_kernel(const float *__restrict__ part_out,
                                                                 const float *__restrict__ part_lse,
                                                                 const int32_t *__restrict__ num_splits,
+                                                                const int32_t *__restrict__ request,
                                                                 int max_splits, int heads,
                                                                 __nv_bfloat16 *__restrict__ out,
                                                                 float *__restrict__ lse)
@@ -33,6 +34,9 @@ __global__ void __launch_bounds__(128 * kGroups) combine_kernel(const float *__r
     // the kernel that follows may be scheduled early in turn (it waits before it reads)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // which request the b-th set of partial results belongs to; negative: there are none after all
+    const int owner = request ? __ldg(request + b) : b;
+    if (owner < 0) return;
     int ns = num_splits ? __ldg(num_splits + b) : max_splits;
     ns = max(0, min(ns, max_splits));
     // total over all splits, 32 at a time: every warp does it for itself
@@ -94,8 +98,9 @@ __global__ void __launch_bounds__(128 * kGroups) combine_kernel(const float *__r
     uint2 packed;
     packed.x = *reinterpret_cast<uint32_t *>(&lo);
     packed.y = *reinterpret_cast<uint32_t *>(&hi);
-    reinterpret_cast<uint2 *>(out + ((size_t)b * heads + h) * kDv)[col] = packed;
-    if (threadIdx.x == 0) lse[(size_t)b * heads + h] = total;
+    const size_t to = (size_t)owner * heads + h;
+    reinterpret_cast<uint2 *>(out + to * kDv)[col] = packed;
+    if (threadIdx.x == 0) lse[to] = total;
 }
 
 // rows[b][j] = physical row of the j-th selected token (-1 outside sel_len or on a contract

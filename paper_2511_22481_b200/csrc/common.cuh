@@ -37,6 +37,8 @@ struct DecodeParams {
     int64_t num_pages;
     int32_t batch, heads, max_pages, max_sel, splits;
     int32_t cluster_merge;         // 1: two splits, merged inside a cluster of two CTA pairs
+    int32_t whole;                 // the first `whole` requests (in the order they are taken) are not split, only the rest
+    int32_t *tail_request;         // whole > 0: which request the k-th of the rest is, for the merge kernel
     int32_t longest_first;         // 1: work units take the requests in order of decreasing selection size
     float scale_log2;              // softmax_scale * log2(e)
 };

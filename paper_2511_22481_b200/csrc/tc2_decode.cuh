@@ -452,33 +452,82 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
     }
 }
 
-// An empty split (no tokens): zeros and -inf in place of a result.  Called by all threads.
-__device__ __forceinline__ void c2_store_empty(const DecodeParams &p, int b, int s, int h0, int head_rows, int warp, int lane)
+// What a pair works on: split s of `splits` of request b (splits = 0: nothing), whose partial results are those
+// of request `slot`.
+struct C2Unit {
+    int b, s, splits, slot;
+};
+
+// The unit of the pair-th pair.  Only the requests behind the first p.whole are split (whole = 0: all of
+// them); b is their place in the order they are taken in, until c2_name_request.
+__device__ __forceinline__ C2Unit c2_unit(const DecodeParams &p, int pair)
 {
+    C2Unit w;
+    const int behind = pair - p.whole, tail = p.batch - p.whole;
+    w.slot = -1;
+    if (p.whole == 0) {
+        w.splits = p.splits;
+        w.s = pair % p.splits;
+        w.b = pair / p.splits;
+    } else if (behind < 0) {
+        w.splits = 1;
+        w.s = 0;
+        w.b = pair;
+    } else {
+        w.splits = p.splits;
+        w.s = behind / tail;             // first pieces first: they are all there is when nothing is cut
+        w.slot = behind % tail;
+        w.b = p.whole + w.slot;
+    }
+    return w;
+}
+
+// Names the request.  cut: see c2_request_by_length_rank; without it the first piece of a request is all of it.
+// Thread 0 of the pair's first CTA (`first`) tells the merge kernel which request, or that there is nothing to do.
+__device__ __forceinline__ void c2_name_request(const DecodeParams &p, C2Unit &w, int b, bool cut, bool first)
+{
+    w.b = b;
+    if (p.whole == 0) {
+        w.slot = b;
+    } else if (w.slot >= 0) {
+        if (w.s == 0 && first) p.tail_request[w.slot] = cut ? b : -1;
+        if (!cut) w.splits = w.s == 0 ? 1 : 0;
+    }
+}
+
+// An empty split (no tokens): zeros and -inf in place of a result.  Called by all threads.
+__device__ __forceinline__ void c2_store_empty(const DecodeParams &p, const C2Unit &w, int h0, int head_rows, int warp, int lane)
+{
+    if (w.splits == 0) return;
     for (int r = warp; r < head_rows; r += kC2Threads / 32) {
         const int h = h0 + r;
-        if (p.splits == 1) {
-            uint4 *o = reinterpret_cast<uint4 *>(p.out + ((size_t)b * p.heads + h) * kDv);
+        if (w.splits == 1) {
+            uint4 *o = reinterpret_cast<uint4 *>(p.out + ((size_t)w.b * p.heads + h) * kDv);
             for (int i = lane; i < kDv * 2 / 16; i += 32) o[i] = make_uint4(0, 0, 0, 0);
-            if (lane == 0) p.lse[(size_t)b * p.heads + h] = -INFINITY;
+            if (lane == 0) p.lse[(size_t)w.b * p.heads + h] = -INFINITY;
         } else {
-            const size_t u = ((size_t)b * p.splits + s) * p.heads + h;
+            const size_t u = ((size_t)w.slot * p.splits + w.s) * p.heads + h;
             float4 *o = reinterpret_cast<float4 *>(p.part_out + u * kDv);
             for (int i = lane; i < kDv / 4; i += 32) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (lane == 0) p.part_lse[u] = -INFINITY;
         }
     }
-    if (p.splits > 1 && p.counters != nullptr) __threadfence();
+    if (w.splits > 1 && p.counters != nullptr) __threadfence();
 }
 
 // With more work units than the device runs at once, CTAs start in index order, so the requests
 // are taken longest first (ties by index): a long request that started last would otherwise run
 // on alone at the end.  Every CTA ranks the (at most 256) selection sizes itself: request j has
 // rank #{i : n_i > n_j, or n_i = n_j and i < j}, and the pair whose place in the grid is `slot`
-// takes the request of that rank.  lens: shared memory nobody uses yet (batch ints); flag: a
+// takes the request of that rank.  lens: shared memory nobody uses yet (batch + 3 ints); flag: a
 // shared word.  Called by all threads; returns the request.
-__device__ __forceinline__ int c2_request_by_length_rank(const DecodeParams &p, int *lens, uint32_t *flag, int slot)
+// cut: where only the requests behind the first wave are split (p.whole > 0), whether that pays.  Whole,
+// the longest of them would start when the shortest of the first wave ends; only if it then ends after the longest
+// of all, by more than a merge costs (12 units), do pieces help.
+constexpr int kCutGain = 12 * kC2Tile;
+__device__ __forceinline__ int c2_request_by_length_rank(const DecodeParams &p, int *lens, uint32_t *flag, int slot, bool &cut)
 {
+    int *mark = lens + p.batch;                               // sizes of three ranks
     for (int j = threadIdx.x; j < p.batch; j += kC2Threads) lens[j] = load_selection(p, j).n;
     __syncthreads();
     for (int j = threadIdx.x; j < p.batch; j += kC2Threads) {
@@ -486,9 +535,13 @@ __device__ __forceinline__ int c2_request_by_length_rank(const DecodeParams &p, 
         int before = 0;
         for (int i = 0; i < p.batch; ++i) before += (lens[i] > nj) || (lens[i] == nj && i < j);
         if (before == slot) *flag = (uint32_t)j;
+        if (before == 0) mark[0] = nj;
+        if (before == p.whole - 1) mark[1] = nj;
+        if (before == p.whole) mark[2] = nj;
     }
     __syncthreads();
     const int b = (int)*flag;
+    cut = p.whole == 0 || (int64_t)mark[1] + mark[2] > (int64_t)mark[0] + kCutGain;
     __syncthreads();                                          // the shared memory is handed to the producers next
     return b;
 }
@@ -504,7 +557,7 @@ __device__ __forceinline__ int c2_request_by_length_rank(const DecodeParams &p, 
 // CTA-wide barrier is needed, so the stores of one round overlap the tensor-memory reads of the
 // next.  lt: the row's sum of weights; m_ref: its reference maximum (log2 units).
 __device__ __forceinline__ void c2_store_result(const DecodeParams &p, uint8_t *smem, uint32_t tmem, int warp, int lane,
-                                                int b, int s, int h0, int head_rows, float lt, float m_ref)
+                                                const C2Unit &w, int h0, int head_rows, float lt, float m_ref)
 {
     const int quarter = warp & 3;
     const int sub = warp >= 8 ? 1 : 0;
@@ -513,15 +566,16 @@ __device__ __forceinline__ void c2_store_result(const DecodeParams &p, uint8_t *
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
     const float inv = lt > 0.f ? 1.f / lt : 0.f;
     const int h = h0 + row;
-    const bool final_out = p.splits == 1;
-    const size_t u = final_out ? ((size_t)b * p.heads + h) : (((size_t)b * p.splits + s) * p.heads + h);
+    const bool final_out = w.splits == 1;
+    const size_t first = final_out ? (size_t)w.b * p.heads : ((size_t)w.slot * p.splits + w.s) * p.heads;
+    const size_t u = first + h;
     constexpr uint32_t kStagePitch = 144, kStageBytes = 32 * kStagePitch;
     const int widx = sub * 4 + ((warp - 2) & 3);                         // 0..7
     uint8_t *stage = smem + (size_t)widx * 2 * kStageBytes;
     const uint32_t row_bytes = final_out ? kDv * 2 : kDv * 4;
     const int row0 = (quarter & 1) * 32;                                  // first head row of this warp
     // global address of (row0, this warp's first value column)
-    const size_t u0 = final_out ? ((size_t)b * p.heads + h0 + row0) : (((size_t)b * p.splits + s) * p.heads + h0 + row0);
+    const size_t u0 = first + h0 + row0;
     uint8_t *gbase = (final_out ? reinterpret_cast<uint8_t *>(p.out + u0 * kDv)
                                 : reinterpret_cast<uint8_t *>(p.part_out + u0 * kDv)) + part * (row_bytes / 4);
     const int rows_here = max(0, min(32, head_rows - row0));              // rows of this warp that exist
@@ -607,8 +661,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     const uint16_t pair_mask = (uint16_t)(3u << leader);
 
     const int pair = blockIdx.x >> 1;
-    const int s = kClusterMerge ? (int)(crank >> 1) : pair % p.splits;
-    int b = kClusterMerge ? (int)(blockIdx.x >> 2) : pair / p.splits;
+    C2Unit unit = kClusterMerge ? C2Unit{(int)(blockIdx.x >> 2), (int)(crank >> 1), 2, 0} : c2_unit(p, pair);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform
     const int h0 = (int)rank * kTcHeads;
     const int head_rows = min(kTcHeads, p.heads - h0);
@@ -658,20 +711,25 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     // may be scheduled as soon as resources allow; it waits in the same way before it reads.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!kClusterMerge && p.longest_first) b = c2_request_by_length_rank(p, reinterpret_cast<int *>(smem), &ctl->merge_flag, b);
+    if (!kClusterMerge) {
+        bool cut = true;
+        const int request = p.longest_first ? c2_request_by_length_rank(p, reinterpret_cast<int *>(smem), &ctl->merge_flag, unit.b, cut) : unit.b;
+        c2_name_request(p, unit, request, cut, rank == 0 && threadIdx.x == 0);
+    }
+    const int b = unit.b, s = unit.s;
     const Selection selection = load_selection(p, b);
     __builtin_assume(kRanges ? selection.list == nullptr : selection.list != nullptr);
-    const int n = selection.n;
+    const int n = !kClusterMerge && unit.splits == 0 ? 0 : selection.n;
     const bool bad_len = selection.bad;
     int begin, end;
-    split_range(n, p.splits, s, begin, end, kC2Tile);
+    split_range(n, max(unit.splits, 1), s, begin, end, kC2Tile);
     const int units = (end - begin + kC2Tile - 1) / kC2Tile, tiles = (units + 1) / 2;
 
     const bool active = units > 0;
     if (!active && bad_len && threadIdx.x == 0 && crank == 0) flag_status(p.status, OMNI_DEV_BAD_INDEX);
     if (!kClusterMerge && !active) {
         // empty split (the same decision in both CTAs of the pair): zeros and -inf, no pipeline
-        c2_store_empty(p, b, s, h0, head_rows, warp, lane);
+        c2_store_empty(p, unit, h0, head_rows, warp, lane);
     }
 
     const uint32_t tmem = ctl->tmem_base;
@@ -1217,8 +1275,8 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             if (warp == 2 && lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&ctl->ready_bar), crank ^ 2u));
         } else if (!kClusterMerge && ok) {
             tc_fence_after();
-            c2_store_result(p, smem, tmem, warp, lane, b, s, h0, head_rows, lt, m_ref);
-            const bool final_out = p.splits == 1;
+            c2_store_result(p, smem, tmem, warp, lane, unit, h0, head_rows, lt, m_ref);
+            const bool final_out = unit.splits == 1;
             // with the in-kernel merge the partial results must be visible before this CTA is counted
             if (!final_out && p.counters != nullptr) __threadfence();
         }
@@ -1344,7 +1402,7 @@ inline bool tc2_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cached)
 inline omni_status_t tc2_launch(const CUtensorMap *maps, const DecodeParams &p, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.batch * p.splits * 2));
+    cfg.gridDim = dim3((unsigned)((p.whole + (p.batch - p.whole) * p.splits) * 2));
     cfg.blockDim = dim3(kC2Threads);
     cfg.dynamicSmemBytes = kC2SmemBytes;
     cfg.stream = stream;

@@ -214,8 +214,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
     const uint16_t pair_mask = (uint16_t)(3u << leader);
 
     const int pair = blockIdx.x >> 1;
-    const int s = kClusterMerge ? (int)(crank >> 1) : pair % p.splits;
-    int b = kClusterMerge ? (int)(blockIdx.x >> 2) : pair / p.splits;
+    C2Unit unit = kClusterMerge ? C2Unit{(int)(blockIdx.x >> 2), (int)(crank >> 1), 2, 0} : c2_unit(p, pair);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform
     const int h0 = (int)rank * kTcHeads;
     const int head_rows = min(kTcHeads, p.heads - h0);
@@ -261,18 +260,23 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
     tc_fence_after();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!kClusterMerge && p.longest_first) b = c2_request_by_length_rank(p, reinterpret_cast<int *>(smem), &ctl->merge_flag, b);
+    if (!kClusterMerge) {
+        bool cut = true;
+        const int request = p.longest_first ? c2_request_by_length_rank(p, reinterpret_cast<int *>(smem), &ctl->merge_flag, unit.b, cut) : unit.b;
+        c2_name_request(p, unit, request, cut, rank == 0 && threadIdx.x == 0);
+    }
+    const int b = unit.b, s = unit.s;
     const Selection selection = load_selection(p, b);
     __builtin_assume(selection.list != nullptr);
-    const int n = selection.n;
+    const int n = !kClusterMerge && unit.splits == 0 ? 0 : selection.n;
     const bool bad_len = selection.bad;
     int begin, end;
-    split_range(n, p.splits, s, begin, end, kC2Tile);
+    split_range(n, max(unit.splits, 1), s, begin, end, kC2Tile);
     const int units = (end - begin + kC2Tile - 1) / kC2Tile, tiles = (units + 1) / 2;
 
     const bool active = units > 0;
     if (!active && bad_len && threadIdx.x == 0 && crank == 0) flag_status(p.status, OMNI_DEV_BAD_INDEX);
-    if (!kClusterMerge && !active) c2_store_empty(p, b, s, h0, head_rows, warp, lane);
+    if (!kClusterMerge && !active) c2_store_empty(p, unit, h0, head_rows, warp, lane);
 
     const uint32_t tmem = ctl->tmem_base;
     volatile uint32_t *abort_flag = &ctl->abort;
@@ -830,8 +834,8 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             tc_fence_after();
             const float lt = (ctl->xchg[tiles & 1][0][row] + ctl->xchg[tiles & 1][1][row]) +
                              (ctl->xchg[tiles & 1][2][row] + ctl->xchg[tiles & 1][3][row]);
-            c2_store_result(p, smem, tmem, warp, lane, b, s, h0, head_rows, lt, m_ref);
-            if (p.splits != 1 && p.counters != nullptr) __threadfence();
+            c2_store_result(p, smem, tmem, warp, lane, unit, h0, head_rows, lt, m_ref);
+            if (unit.splits != 1 && p.counters != nullptr) __threadfence();
         }
         if (!ok && lane == 0) {
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_SOFTMAX);
@@ -1014,7 +1018,7 @@ inline bool tc2q8_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cache
 inline omni_status_t tc2q8_launch(const CUtensorMap *maps, const DecodeParams &p, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.batch * p.splits * 2));
+    cfg.gridDim = dim3((unsigned)((p.whole + (p.batch - p.whole) * p.splits) * 2));
     cfg.blockDim = dim3(kC2Threads);
     cfg.dynamicSmemBytes = kC2SmemBytes;
     cfg.stream = stream;
