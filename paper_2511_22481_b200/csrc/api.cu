@@ -154,7 +154,7 @@ SplitPlan split_plan(const omni_mla_desc_t *d, int sm_count, int resident_merge_
         }
     }
     // One wave of whole requests and a few more: whole, these would keep at most a third of the pairs busy for as
-    // long again, so they are cut into as many pieces as there are pairs.  80 requests x 64 units 134 -> 95 us, 98
+    // long again, so they are cut into as many pieces as there are pairs.  80 requests x 64 units 134 -> 98 us, 98
     // x 64 143 -> 117, 76 x 128 225 -> 165.  Where the sizes differ so much that the few run beside the longest ones the
     // kernel takes them whole after all (c2_request_by_length_rank) and the merge kernel finds nothing to do.  That costs
     // 2 to 4 us (67 us where sizes run from 8 to 64 units), so the line lies at 64 units.
