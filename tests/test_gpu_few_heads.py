@@ -1,0 +1,21 @@
+"""The single-CTA kernel at the edges of its tiles and of its head rows: partial rows leave eight rows at a time, each
+warp owns sixteen, scores start on the first third of a tile's panels, and a split may be empty."""
+import numpy as np
+import pytest
+
+from paper_2511_22481_b200 import workloads as W
+from parity import check_workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("heads", [1, 8, 9, 16, 17, 31, 32])
+@pytest.mark.parametrize("splits", [1, 2, 5, 13])
+def test_head_rows_and_tiles(heads, splits):
+    rng = np.random.default_rng(heads)
+    lengths = [1, 63, 64, 65, 190, 64 * 13, 64 * 13 + 1]          # with 5 and 13 splits some are empty
+    lists = [np.arange(n) for n in lengths] + [rng.permutation(16 * 64)[:300]]
+    pages = [16] * len(lists)
+    w = W._pack("few heads", 9, heads, pages, W._shuffled_tables(rng, pages, True),
+                [np.asarray(x, dtype=np.int32) for x in lists], "cuda", dict(kind="custom"))
+    check_workload(w, 0, num_splits=splits, what="H=%d S=%d" % (heads, splits))
