@@ -20,6 +20,12 @@
 //   columns 320..383  S buffer 1
 // Every softmax thread owns half a row: lane l of a warp serves head row 16*(warp%4)+l%16 and
 // the token half (of S) / value-column half (of O) l/16.
+//
+// What bounds it is latency: it serves calls of one or two tiles a CTA.  So barriers and tensor memory are set
+// up before the kernel in front of it in the stream has ended, q is requested before the selection's length is known, the
+// scores start on the first third of a tile's panels, and partial rows are stored in whole sectors.  Steps without and with
+// these four: one request of 13 tiles, 16 heads 9.70 -> 9.23 us, 32 heads 10.97 -> 9.46; 8 x 16 tiles of 16
+// heads 11.34 -> 10.67.
 #pragma once
 
 #include <cuda.h>
@@ -37,6 +43,7 @@ constexpr int kPanelBytes = kTile * 128;           // 64 rows x 64 bf16 columns,
 constexpr int kPanels = kDqk / 64;                 // 9 column panels per latent row
 constexpr int kTileBytes = kPanels * kPanelBytes;  // 73,728
 constexpr int kStages = 2;
+constexpr int kGroups = 3, kGroupPanels = kPanels / kGroups, kGroupBytes = kGroupPanels * kPanelBytes;
 constexpr int kPBytes = kTcHeads * kTile * 2;      // 8,192
 constexpr int kSmemQ = 0;
 constexpr int kSmemKV = kSmemQ + kTileBytes;
@@ -52,7 +59,7 @@ constexpr long long kWaitCycles = 1ll << 31;         // about a second of SM clo
 
 struct TcControl {
     uint64_t q_full;
-    uint64_t kv_full[kStages];
+    uint64_t kv_full[kStages][kGroups];  // a third of the tile's panels each: the scores start on the first
     uint64_t kv_empty[kStages];
     uint64_t s_full[2];
     uint64_t s_empty[2];
@@ -303,6 +310,21 @@ __device__ __forceinline__ void tc_ld16x2(uint32_t taddr, uint32_t (&v)[32])
         : "memory");
 }
 
+// 16 lanes x 64 columns: of every 8 columns thread t gets columns 2 (t % 4), + 1 of lane t / 4, then of lane t / 4 + 8.
+__device__ __forceinline__ void tc_ld16x256x8(uint32_t taddr, uint32_t (&v)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr)
+        : "memory");
+}
+
 __global__ void __launch_bounds__(kTcThreads, 1)
 tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap kv_map,
                  const __grid_constant__ CUtensorMap kv_page_map, DecodeParams p)
@@ -315,11 +337,42 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
     const int s = blockIdx.x % p.splits, b = blockIdx.x / p.splits;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform
 
+    // ---- set-up: barriers, tensor memory (nothing here touches global memory, so with a programmatic dependent launch it
+    // overlaps the tail of the kernel before this one) ------------------------------------------
+    if (threadIdx.x == 0) {
+        mbar_init(&ctl->q_full, 1);
+        for (int i = 0; i < kStages; ++i) {
+            for (int g = 0; g < kGroups; ++g) mbar_init(&ctl->kv_full[i][g], 1);
+            mbar_init(&ctl->kv_empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&ctl->s_full[i], 1);
+            mbar_init(&ctl->s_empty[i], 128);
+        }
+        mbar_init(&ctl->p_full, 128);
+        mbar_init(&ctl->pv_done, 1);
+        ctl->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
+                     "r"(kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+
     // Programmatic dependent launch, both ways: nothing in global memory is touched until the
     // kernel before this one in the stream has completed, and the kernel after this one (the split
     // merge) may be scheduled as soon as resources allow; it waits in the same way before it reads.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (warp == 0 && lane == 0) {                           // q needs nothing of the selection
+        mbar_expect_tx(&ctl->q_full, kTileBytes);
+        tma_box3d(smem_base + kSmemQ, &q_map, &ctl->q_full, b * p.heads, 0);
+    }
     const Selection selection = load_selection(p, b);
     const int n = selection.n;
     const bool bad_len = selection.bad;
@@ -344,44 +397,18 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
                 if (lane == 0) p.part_lse[u] = -INFINITY;
             }
         }
-        return;
     }
 
-    // ---- set-up: barriers, tensor memory ------------------------------------------------
-    if (threadIdx.x == 0) {
-        mbar_init(&ctl->q_full, 1);
-        for (int i = 0; i < kStages; ++i) {
-            mbar_init(&ctl->kv_full[i], 1);
-            mbar_init(&ctl->kv_empty[i], 1);
-        }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&ctl->s_full[i], 1);
-            mbar_init(&ctl->s_empty[i], 128);
-        }
-        mbar_init(&ctl->p_full, 128);
-        mbar_init(&ctl->pv_done, 1);
-        ctl->abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
-                     "r"(kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
     volatile uint32_t *abort_flag = &ctl->abort;
 
-    if (warp == 0) {
+    if (tiles == 0) {
+        // (stored above; q has to land before the CTA may leave)
+        if (warp == 0 && !mbar_wait(&ctl->q_full, 0) && lane == 0) flag_status(p.status, OMNI_DEV_TIMEOUT);
+        __syncwarp();
+    } else if (warp == 0) {
         // =========================== producer ===========================================
         const int32_t *pt = p.page_table + (size_t)b * p.max_pages;
-        if (lane == 0) {
-            mbar_expect_tx(&ctl->q_full, kTileBytes);
-            tma_box3d(smem_base + kSmemQ, &q_map, &ctl->q_full, b * p.heads, 0);
-        }
         bool any_bad = bad_len;
         // Lane l serves tokens l and l+32 of a tile.  Token positions are fetched two tiles
         // ahead and turned into pool rows one tile ahead, so neither dependent load sits
@@ -437,13 +464,15 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
             }
             if (lane == 0) {
                 ctl->valid_mask[st] = mask;
-                mbar_expect_tx(&ctl->kv_full[st], kTileBytes);
+                for (int g = 0; g < kGroups; ++g) mbar_expect_tx(&ctl->kv_full[st][g], kGroupBytes);
             }
             __syncwarp();
             const uint32_t stage = smem_base + kSmemKV + st * kTileBytes;
             if (contig) {
-                // 64 consecutive pool rows (a whole page in order): the whole tile is one 3-D box
-                if (lane == 0) tma_box3d(stage, &kv_page_map, &ctl->kv_full[st], row_lo, 0);
+                // 64 consecutive pool rows (a whole page in order): a 3-D box for every third of the panels
+                if (lane == 0)
+                    for (int g = 0; g < kGroups; ++g)
+                        tma_box3d(stage + g * kGroupBytes, &kv_page_map, &ctl->kv_full[st][g], row_lo, g * kGroupPanels);
             } else {
                 // scattered rows: lane g < 16 gathers tokens 4g..4g+3 into rows 4g..4g+3 of every panel
                 int r[4];
@@ -456,7 +485,7 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
                 if (lane < 16) {
 #pragma unroll
                     for (int c = 0; c < kPanels; ++c)
-                        tma_gather4(stage + lane * 512 + c * kPanelBytes, &kv_map, &ctl->kv_full[st], c * 64, r[0], r[1],
+                        tma_gather4(stage + lane * 512 + c * kPanelBytes, &kv_map, &ctl->kv_full[st][c / kGroupPanels], c * 64, r[0], r[1],
                                     r[2], r[3]);
                 }
             }
@@ -467,7 +496,8 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
         if (__any_sync(0xffffffffu, any_bad) && lane == 0) flag_status(p.status, OMNI_DEV_BAD_INDEX);
         if (*abort_flag) {
             // let every copy this warp started land before the CTA can exit
-            for (int i = max(0, issued - kStages); i < issued; ++i) mbar_wait(&ctl->kv_full[i % kStages], (i / kStages) & 1);
+            for (int i = max(0, issued - kStages); i < issued; ++i)
+                for (int g = 0; g < kGroups; ++g) mbar_wait(&ctl->kv_full[i % kStages][g], (i / kStages) & 1);
             mbar_wait(&ctl->q_full, 0);
         }
     } else if (warp == 1) {
@@ -487,18 +517,27 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
             const uint32_t kmaj_hi = (uint32_t)(q_desc >> 32), v_hi = (uint32_t)(v_desc >> 32);
             const int tiles_u = __shfl_sync(0xffffffffu, tiles, 0);
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
-            // S(t) = Q K(t)^T : 36 k-steps of 16 columns; panel c of Q against panel c of the stage
-            auto issue_qk = [&](auto par_tag) {
+            // S(t) = Q K(t)^T : 36 k-steps of 16 columns, a group of panels as soon as it has landed; panel c of Q
+            // against panel c of the stage
+            auto issue_qk = [&](auto par_tag, uint32_t phase) -> bool {
                 constexpr int par = decltype(par_tag)::value;
                 const uint32_t d = tmem_u + kColS + 64 * par;
                 const uint32_t kb = k_lo + ((par * kTileBytes) >> 4);
-                tc_mma_elect<false>(d, q_lo, kmaj_hi, kb, kmaj_hi, idesc_qk);
 #pragma unroll
-                for (int kk = 1; kk < kDqk / 16; ++kk) {
-                    const uint32_t off = ((kk >> 2) * kPanelBytes + (kk & 3) * 32) >> 4;
-                    tc_mma_elect<true>(d, q_lo + off, kmaj_hi, kb + off, kmaj_hi, idesc_qk);
+                for (int g = 0; g < kGroups; ++g) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(&ctl->kv_full[par][g], phase))) return false;
+                    tc_fence_after();
+#pragma unroll
+                    for (int kk = 0; kk < 4 * kGroupPanels; ++kk) {
+                        const uint32_t off = ((g * kGroupPanels + (kk >> 2)) * kPanelBytes + (kk & 3) * 32) >> 4;
+                        if (g == 0 && kk == 0)
+                            tc_mma_elect<false>(d, q_lo, kmaj_hi, kb, kmaj_hi, idesc_qk);
+                        else
+                            tc_mma_elect<true>(d, q_lo + off, kmaj_hi, kb + off, kmaj_hi, idesc_qk);
+                    }
                 }
                 tc_commit_elect(&ctl->s_full[par]);
+                return true;
             };
             // O += P(i) V(i) : the stage read N-major (64-column panels 8192 B apart, 8-token groups
             // 1024 B apart); value columns 0..255 and 256..511 go to the two interleaved accumulators
@@ -527,12 +566,11 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
                 bool good = true;
                 if (i + 1 < tiles_u) {
                     const int t = i + 1;
-                    good = mbar_wait(&ctl->kv_full[par ^ 1], (t >> 1) & 1) &&
-                           (t < 2 || mbar_wait(&ctl->s_empty[par ^ 1], ((t >> 1) - 1) & 1));
+                    good = t < 2 || mbar_wait(&ctl->s_empty[par ^ 1], ((t >> 1) - 1) & 1);
                     good = __all_sync(0xffffffffu, good);
                     if (!good) return false;
                     tc_fence_after();
-                    issue_qk(std::integral_constant<int, par ^ 1>{});
+                    if (!issue_qk(std::integral_constant<int, par ^ 1>{}, (t >> 1) & 1)) return false;
                 }
                 good = mbar_wait(&ctl->p_full, i & 1);
                 good = __all_sync(0xffffffffu, good);
@@ -541,12 +579,8 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
                 issue_pv(par_tag, i == 0);
                 return true;
             };
-            bool ok = mbar_wait(&ctl->q_full, 0) && mbar_wait(&ctl->kv_full[0], 0);
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok) {
-                tc_fence_after();
-                issue_qk(std::integral_constant<int, 0>{});
-            }
+            bool ok = __all_sync(0xffffffffu, mbar_wait(&ctl->q_full, 0));
+            if (ok) ok = issue_qk(std::integral_constant<int, 0>{}, 0);
             for (int i = 0; ok && i < tiles_u; i += 2) {
                 ok = step(std::integral_constant<int, 0>{}, i);
                 if (ok && i + 1 < tiles_u) ok = step(std::integral_constant<int, 1>{}, i + 1);
@@ -650,32 +684,50 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
             const int h = row;
             const bool store = h < p.heads;
             const size_t u = p.splits == 1 ? ((size_t)b * p.heads + h) : (((size_t)b * p.splits + s) * p.heads + h);
+            if (p.splits > 1) {
+                // Partial rows: 16 lanes x 8 columns at a time, of which a thread gets two columns of rows lane / 4 and
+                // lane / 4 + 8, so that four threads write a whole sector.  (With a row to a thread, every store
+                // touches 32 sectors and fills half of each.)
+                const int r0 = quarter * 16 + (lane >> 2);
+                const float inv0 = __shfl_sync(0xffffffffu, inv, lane >> 2), inv1 = __shfl_sync(0xffffffffu, inv, (lane >> 2) + 8);
+                float *o0 = p.part_out + (((size_t)b * p.splits + s) * p.heads + r0) * kDv + 2 * (lane & 3), *o1 = o0 + 8 * kDv;
+                const bool s0 = r0 < p.heads, s1 = r0 + 8 < p.heads;
+                if (quarter * 16 < p.heads) {
 #pragma unroll 1
-            for (int c = 0; c < 256; c += 32) {
-                uint32_t ov[32];
-                __syncwarp();
-                tc_ld32(tmem + lane_base + kColO + c, ov);
-                tc_wait_ld();
-                const int col = half * 256 + c;
-                if (!store) {
-                    // padded head row: nothing to write
-                } else if (p.splits == 1) {
-                    uint4 *o = reinterpret_cast<uint4 *>(p.out + u * kDv + col);
+                    for (int c = 0; c < kDv; c += 64) {
+                        uint32_t ov[32];
+                        tc_ld16x256x8(tmem + lane_base + kColO + (c & 255) + (c >= 256 ? kLane16 : 0u), ov);
+                        tc_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint4 w;
-                        w.x = pack_bf16(__uint_as_float(ov[8 * j]) * inv, __uint_as_float(ov[8 * j + 1]) * inv);
-                        w.y = pack_bf16(__uint_as_float(ov[8 * j + 2]) * inv, __uint_as_float(ov[8 * j + 3]) * inv);
-                        w.z = pack_bf16(__uint_as_float(ov[8 * j + 4]) * inv, __uint_as_float(ov[8 * j + 5]) * inv);
-                        w.w = pack_bf16(__uint_as_float(ov[8 * j + 6]) * inv, __uint_as_float(ov[8 * j + 7]) * inv);
-                        o[j] = w;
+                        for (int j = 0; j < 8; ++j) {
+                            if (s0)
+                                *reinterpret_cast<float2 *>(o0 + c + 8 * j) =
+                                    make_float2(__uint_as_float(ov[4 * j]) * inv0, __uint_as_float(ov[4 * j + 1]) * inv0);
+                            if (s1)
+                                *reinterpret_cast<float2 *>(o1 + c + 8 * j) =
+                                    make_float2(__uint_as_float(ov[4 * j + 2]) * inv1, __uint_as_float(ov[4 * j + 3]) * inv1);
+                        }
                     }
-                } else {
-                    float4 *o = reinterpret_cast<float4 *>(p.part_out + u * kDv + col);
+                }
+            } else {
+#pragma unroll 1
+                for (int c = 0; c < 256; c += 32) {
+                    uint32_t ov[32];
+                    __syncwarp();
+                    tc_ld32(tmem + lane_base + kColO + c, ov);
+                    tc_wait_ld();
+                    if (store) {                            // (a padded head row: nothing to write)
+                        uint4 *o = reinterpret_cast<uint4 *>(p.out + u * kDv + half * 256 + c);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        o[j] = make_float4(__uint_as_float(ov[4 * j]) * inv, __uint_as_float(ov[4 * j + 1]) * inv,
-                                           __uint_as_float(ov[4 * j + 2]) * inv, __uint_as_float(ov[4 * j + 3]) * inv);
+                        for (int j = 0; j < 4; ++j) {
+                            uint4 w;
+                            w.x = pack_bf16(__uint_as_float(ov[8 * j]) * inv, __uint_as_float(ov[8 * j + 1]) * inv);
+                            w.y = pack_bf16(__uint_as_float(ov[8 * j + 2]) * inv, __uint_as_float(ov[8 * j + 3]) * inv);
+                            w.z = pack_bf16(__uint_as_float(ov[8 * j + 4]) * inv, __uint_as_float(ov[8 * j + 5]) * inv);
+                            w.w = pack_bf16(__uint_as_float(ov[8 * j + 6]) * inv, __uint_as_float(ov[8 * j + 7]) * inv);
+                            o[j] = w;
+                        }
+                    }
                 }
             }
             if (store && half == 0) {
@@ -826,9 +878,9 @@ inline bool tc_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cached)
     const uint64_t rows = (uint64_t)p.num_pages * kPage, qrows = (uint64_t)p.batch * p.heads;
     if (cached)
         return make_panel_map(&maps[0], p.q, qrows, kTcHeads, kPanels) && make_row_map(&maps[1], p.kv, rows, 1) &&
-               make_panel_map(&maps[2], p.kv, rows, kTile, kPanels);
+               make_panel_map(&maps[2], p.kv, rows, kTile, kGroupPanels);
     return encode_panel_map(&maps[0], p.q, qrows, kTcHeads, kPanels) && encode_row_map(&maps[1], p.kv, rows, 1, 0) &&
-           encode_panel_map(&maps[2], p.kv, rows, kTile, kPanels);
+           encode_panel_map(&maps[2], p.kv, rows, kTile, kGroupPanels);
 }
 
 inline omni_status_t tc_launch(const CUtensorMap *maps, const DecodeParams &p, cudaStream_t stream)
