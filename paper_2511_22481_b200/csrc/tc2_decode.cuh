@@ -1204,10 +1204,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 for (int j = 0; j < 32; ++j)
                     if (!((valid >> j) & 1u)) sv[j] = __float_as_uint(-INFINITY);
             }
-            float mt4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-            for (int j = 0; j < 32; ++j) mt4[j & 3] = fmaxf(mt4[j & 3], __uint_as_float(sv[j]));
-            float mt = fmaxf(fmaxf(mt4[0], mt4[1]), fmaxf(mt4[2], mt4[3])) * xs;
+            float mt = fmaxf(max32([&](int j) { return __uint_as_float(sv[j]); }), -INFINITY) * xs;
             float *xg = &ctl->xchg[i & 1][0][row];
             xg[tq * 64] = mt;
             mbar_arrive(&ctl->xg_bar);
@@ -1226,17 +1223,18 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 moved = true;
             }
             const float mr = (m_ref == -INFINITY) ? 0.f : m_ref;
-            float sum[2] = {0.f, 0.f};
+            const f32x2 xs2 = pack2(xs, xs), mr2 = pack2(-mr, -mr);
+            f32x2 sums = pack2(0.f, 0.f);
             uint32_t pk[16];
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
-                const float e0 = fast_exp2(fmaf(__uint_as_float(sv[j]), xs, -mr));
-                const float e1 = fast_exp2(fmaf(__uint_as_float(sv[j + 1]), xs, -mr));
-                sum[0] += e0;
-                sum[1] += e1;
+                const float2 y = unpack2(fma2(pack2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1])), xs2, mr2));
+                const float e0 = fast_exp2(y.x), e1 = fast_exp2(y.y);
+                sums = add2(sums, pack2(e0, e1));
                 pk[j >> 1] = pack_bf16(e0, e1);
             }
-            l = l * factor + (sum[0] + sum[1]);
+            const float2 sum = unpack2(sums);
+            l = l * factor + (sum.x + sum.y);
             // P and O are free once P V of the tile before (its second unit: only the last tile can have a
             // single one) retired
             if (i >= 1) {

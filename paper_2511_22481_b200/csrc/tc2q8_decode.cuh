@@ -162,7 +162,10 @@ __device__ __forceinline__ void split_e4m3(const float (&v)[16], uint4 &hi, uint
     for (int k = 0; k < 4; ++k) {
         const uint32_t h0 = e4m3x2(v[4 * k], v[4 * k + 1]), h1 = e4m3x2(v[4 * k + 2], v[4 * k + 3]);
         const float2 b0 = e4m3x2_values(h0), b1 = e4m3x2_values(h1);
-        const uint32_t l0 = e4m3x2(v[4 * k] - b0.x, v[4 * k + 1] - b0.y), l1 = e4m3x2(v[4 * k + 2] - b1.x, v[4 * k + 3] - b1.y);
+        const f32x2 minus = pack2(-1.f, -1.f);            // (v - b is exact, whatever the form)
+        const float2 r0 = unpack2(fma2(pack2(b0.x, b0.y), minus, pack2(v[4 * k], v[4 * k + 1])));
+        const float2 r1 = unpack2(fma2(pack2(b1.x, b1.y), minus, pack2(v[4 * k + 2], v[4 * k + 3])));
+        const uint32_t l0 = e4m3x2(r0.x, r0.y), l1 = e4m3x2(r1.x, r1.y);
         h[k] = h0 | (h1 << 16);
         l[k] = l0 | (l1 << 16);
     }
@@ -728,14 +731,18 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             const float4 *ts = reinterpret_cast<const float4 *>(&aux->tok_scale[ring][32 * part]);
             const float4 *tl = reinterpret_cast<const float4 *>(&aux->tok_log2[ring][32 * part]);
             float y[32];
+            const f32x2 ac2 = pack2(ac, ac), scale2 = pack2(p.scale_log2, p.scale_log2);
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
                 const float4 sc = ts[g], lg = tl[g];
-                const float scv[4] = {sc.x, sc.y, sc.z, sc.w}, lgv[4] = {lg.x, lg.y, lg.z, lg.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < 4; k += 2) {
                     const int j = 4 * g + k;
-                    y[j] = fmaf(__uint_as_float(s8[j]), ac * scv[k], fmaf(__uint_as_float(sr[j]), p.scale_log2, lgv[k]));
+                    const f32x2 rope = fma2(pack2(__uint_as_float(sr[j]), __uint_as_float(sr[j + 1])), scale2, k ? pack2(lg.z, lg.w) : pack2(lg.x, lg.y));
+                    const float2 v = unpack2(fma2(pack2(__uint_as_float(s8[j]), __uint_as_float(s8[j + 1])),
+                                                  mul2(ac2, k ? pack2(sc.z, sc.w) : pack2(sc.x, sc.y)), rope));
+                    y[j] = v.x;
+                    y[j + 1] = v.y;
                 }
             }
             if (valid != 0xffffffffu) {
@@ -743,10 +750,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
                 for (int j = 0; j < 32; ++j)
                     if (!((valid >> j) & 1u)) y[j] = -INFINITY;
             }
-            float mt4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-            for (int j = 0; j < 32; ++j) mt4[j & 3] = fmaxf(mt4[j & 3], y[j]);
-            float mt = fmaxf(fmaxf(mt4[0], mt4[1]), fmaxf(mt4[2], mt4[3]));
+            float mt = fmaxf(max32([&](int j) { return y[j]; }), -INFINITY);
             ctl->xchg[i & 1][part][row] = mt;
             mbar_arrive(&ctl->x_bar);
             ok = mbar_wait(&ctl->x_bar, i & 1);
@@ -766,7 +770,8 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             }
             const float mr = (m_ref == -INFINITY) ? 0.f : m_ref;
             const float4 *tr = reinterpret_cast<const float4 *>(&aux->tok_rcp[ring][32 * part]);
-            float sum[2] = {0.f, 0.f};
+            const f32x2 mr2 = pack2(-mr, -mr);
+            f32x2 sums = pack2(0.f, 0.f);
             uint4 p_hi[2], p_lo[2];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -774,17 +779,19 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
                     const float4 rc = tr[4 * c + g];
-                    const float rcv[4] = {rc.x, rc.y, rc.z, rc.w};
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int k = 0; k < 4; k += 2) {
                         const int j = 4 * g + k;
-                        pw[j] = fast_exp2(y[16 * c + j] - mr);       // p * scale_t, below 448; 0 for a masked token
-                        sum[k & 1] = fmaf(pw[j], rcv[k], sum[k & 1]);   // p (a masked token repeats a selected row's scale)
+                        const float2 d = unpack2(add2(pack2(y[16 * c + j], y[16 * c + j + 1]), mr2));
+                        pw[j] = fast_exp2(d.x);                      // p * scale_t, below 448; 0 for a masked token
+                        pw[j + 1] = fast_exp2(d.y);
+                        sums = fma2(pack2(pw[j], pw[j + 1]), k ? pack2(rc.z, rc.w) : pack2(rc.x, rc.y), sums);   // p (a masked token repeats a selected row's scale)
                     }
                 }
                 split_e4m3(pw, p_hi[c], p_lo[c]);
             }
-            l = l * factor + (sum[0] + sum[1]);
+            const float2 sum = unpack2(sums);
+            l = l * factor + (sum.x + sum.y);
             // P and O are free once P V of the tile before retired
             if (i >= 1) {
                 ok = mbar_wait(&ctl->pv_done[1], (i - 1) & 1);
