@@ -364,7 +364,7 @@ struct LaunchPlan {
     uint32_t magic;
     int32_t kernel;            // 0 plain-FMA, 1 single-CTA tensor-core, 2 paired-CTA tensor-core, 3 the same over the 8-bit cache
     int32_t splits, whole;     // the first `whole` requests are not split
-    int32_t cluster_merge, longest_first, fused_merge;
+    int32_t cluster_merge, longest_first, fused_merge, resident_pairs;
     int32_t device;
     size_t need, part_out, part_lse, counters;
     omni_mla_desc_t desc;
@@ -409,6 +409,7 @@ static omni_status_t build_plan(const omni_mla_desc_t *desc, const void *q, cons
                            (long)desc->batch * splits > dev.sm_count / 2)
                               ? 1
                               : 0;
+    plan->resident_pairs = plan->kernel == 2 ? tc2_resident().pairs : 0;
     DecodeParams shape = {};
     shape.q = static_cast<const __nv_bfloat16 *>(q);
     shape.kv = static_cast<const __nv_bfloat16 *>(kv_cache);
@@ -500,6 +501,7 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
     p.tail_request = p.whole > 0 ? reinterpret_cast<int32_t *>(static_cast<char *>(workspace) + plan.part_out + plan.part_lse) : nullptr;
     p.cluster_merge = cluster_merge ? 1 : 0;
     p.longest_first = plan.longest_first;
+    p.resident_pairs = plan.resident_pairs;
     if (fused_merge) {
         p.counters = reinterpret_cast<int32_t *>(static_cast<char *>(workspace) + plan.part_out + plan.part_lse);
         if (cudaMemsetAsync(p.counters, 0, plan.counters, stream) != cudaSuccess) return OMNI_ERR_CUDA;

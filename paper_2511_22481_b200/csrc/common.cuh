@@ -40,6 +40,7 @@ struct DecodeParams {
     int32_t whole;                 // the first `whole` requests (in the order they are taken) are not split, only the rest
     int32_t *tail_request;         // whole > 0: which request the k-th of the rest is, for the merge kernel
     int32_t longest_first;         // 1: work units take the requests in order of decreasing selection size
+    int32_t resident_pairs;        // CTA pairs that the device holds at once
     float scale_log2;              // softmax_scale * log2(e)
 };
 
@@ -102,7 +103,13 @@ __device__ __forceinline__ int32_t ldg_index(const int32_t *ptr, uint64_t policy
     return v;
 }
 
-__device__ __forceinline__ Selection load_selection(const DecodeParams &p, int b)
+// What the caller says of request b: its number of selected tokens, or (ranges) its context length.
+__device__ __forceinline__ int load_length(const DecodeParams &p, int b)
+{
+    return __ldg((p.sel_idx != nullptr ? p.sel_len : p.ctx_len) + b);
+}
+
+__device__ __forceinline__ Selection make_selection(const DecodeParams &p, int b, int length)
 {
     Selection s;
     s.bad = false;
@@ -112,14 +119,14 @@ __device__ __forceinline__ Selection load_selection(const DecodeParams &p, int b
     s.keep = index_load_policy();
     if (p.sel_idx != nullptr) {
         s.list = p.sel_idx + (size_t)b * p.max_sel;
-        s.n = __ldg(p.sel_len + b);
+        s.n = length;
         if (s.n < 0 || s.n > p.max_sel) {
             s.bad = true;
             s.n = 0;
         }
     } else {
         s.list = nullptr;
-        int m = __ldg(p.ctx_len + b);
+        int m = length;
         // a rolling cache holds contexts of any length in its few pages
         if (m < 0 || (p.ring_pages == 0 && (int64_t)m > (int64_t)p.max_pages * kPage)) {
             s.bad = true;
@@ -133,6 +140,11 @@ __device__ __forceinline__ Selection load_selection(const DecodeParams &p, int b
         s.n = s.vstart + (m - s.rs);
     }
     return s;
+}
+
+__device__ __forceinline__ Selection load_selection(const DecodeParams &p, int b)
+{
+    return make_selection(p, b, load_length(p, b));
 }
 
 // Whether entry value t is range padding ("no token") rather than a position the caller wrote:

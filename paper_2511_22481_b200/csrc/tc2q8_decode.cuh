@@ -265,7 +265,13 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (!kClusterMerge) {
         bool cut = true;
-        const int request = p.longest_first ? c2_request_by_length_rank(p, reinterpret_cast<int *>(smem), &ctl->merge_flag, unit.b, cut) : unit.b;
+        int request = unit.b;
+        if (p.longest_first) {
+            uint8_t *order = smem + 4096;                 // (behind the sizes; shared memory nobody uses yet)
+            cut = c2_rank_requests(p, reinterpret_cast<int *>(smem), order);
+            request = order[unit.b];
+            __syncthreads();
+        }
         c2_name_request(p, unit, request, cut, rank == 0 && threadIdx.x == 0);
     }
     const int b = unit.b, s = unit.s;
@@ -279,7 +285,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
 
     const bool active = units > 0;
     if (!active && bad_len && threadIdx.x == 0 && crank == 0) flag_status(p.status, OMNI_DEV_BAD_INDEX);
-    if (!kClusterMerge && !active) c2_store_empty(p, unit, h0, head_rows, warp, lane);
+    if (!kClusterMerge && !active) c2_store_empty(p, unit, h0, head_rows, warp, kC2Threads / 32, lane);
 
     const uint32_t tmem = ctl->tmem_base;
     volatile uint32_t *abort_flag = &ctl->abort;
@@ -845,7 +851,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             tc_fence_after();
             const float lt = (ctl->xchg[tiles & 1][0][row] + ctl->xchg[tiles & 1][1][row]) +
                              (ctl->xchg[tiles & 1][2][row] + ctl->xchg[tiles & 1][3][row]);
-            c2_store_result(p, smem, tmem, warp, lane, unit, h0, head_rows, lt, m_ref);
+            c2_store_result<128>(p, smem, tmem, warp, lane, unit, h0, head_rows, lt, m_ref);
             if (unit.splits != 1 && p.counters != nullptr) __threadfence();
         }
         if (!ok && lane == 0) {
