@@ -1,7 +1,7 @@
 // Paired-CTA tensor-core decode kernel for sm_100a (every problem but the smallest with few heads).
 //
-// A cluster of two CTAs owns all heads of one (request, split): CTA r serves heads
-// [64r, 64r+64).  The pair issues cta_group::2 MMAs with M = 128 (64 rows per CTA), which run
+// A cluster of two CTAs owns all heads of one (request, split), each CTA half of them, up to 64
+// rows.  The pair issues cta_group::2 MMAs with M = 128 (64 rows per CTA), which run
 // the tensor pipe of each SM at full rate where a lone M = 64 MMA runs it at half rate, and it
 // halves the operand bytes each SM must hold.  Per tile of 128 tokens, two units of 64:
 //   S = Q K^T   M=128, N=128 tokens, K=576: every CTA supplies its 64 Q rows and the K rows of
@@ -96,6 +96,9 @@ __device__ __forceinline__ void nap_after_abort()
     for (int i = 0; i < 200; ++i) __nanosleep(1000);
 }
 
+// Head rows per CTA of a pair.
+__host__ __device__ __forceinline__ int c2_rows(int heads) { return (heads + 1) >> 1; }
+
 // What a pair works on: split s of `splits` of request b (splits = 0: nothing), whose partial results are those
 // of request `slot`.
 struct C2Unit {
@@ -180,6 +183,17 @@ __device__ __forceinline__ void tma_box3d_pair(uint32_t dst, const CUtensorMap *
         "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
         " [%0], [%1, {%2, %3, %4}], [%5];"
         ::"r"(dst), "l"(map), "r"(0), "r"(row), "r"(panel), "r"(bar_cluster_addr)
+        : "memory");
+}
+
+// The same of q: box {64 columns, 64 rows, 3 panels} of one CTA's heads of one request (see encode_q_map).
+__device__ __forceinline__ void tma_box5d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar_cluster_addr, int row, int panel,
+                                               int side, int request)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+        ::"r"(dst), "l"(map), "r"(0), "r"(row), "r"(panel), "r"(side), "r"(request), "r"(bar_cluster_addr)
         : "memory");
 }
 
@@ -318,11 +332,11 @@ __device__ __forceinline__ void tc_commit_pair_elect(uint64_t *bar, uint16_t bot
 // The copy lands in shared memory that held the partner's operand tiles, so it is not sent
 // before the partner has said that its main loop is over (`ready_bar`, a remote arrive that the
 // partner fires as soon as its last P V has retired, while this CTA is still staging).
-// Called by every thread of the CTA after the main loop.
+// Called by every thread of the CTA after the main loop.  rows: head rows per CTA; only these are sent.
 template <class Control>
 __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Control *ctl, uint8_t *smem,
                                                        uint32_t tmem, int b, int s, uint32_t crank, int h0,
-                                                       int head_rows, bool active, bool main_ok, float cm_lse, float cm_inv)
+                                                       int rows, int head_rows, bool active, bool main_ok, float cm_lse, float cm_inv)
 {
     // The block travels as four chunks, so that the copy of one overlaps the staging of the next and the mixing
     // of the one before: chunk q holds, for every head row, the q-th 32 columns of both 128-column runs
@@ -362,7 +376,7 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
         auto send_chunks = [&](int upto) {
 #pragma unroll 1
             for (; sent <= upto; ++sent) {
-                const uint32_t from = sent == 0 ? 0u : kLseBytes + sent * kChunkBytes, bytes = kChunkBytes + (sent == 0 ? kLseBytes : 0u);
+                const uint32_t from = sent == 0 ? 0u : kLseBytes + sent * kChunkBytes, bytes = rows * kChunkPitch + (sent == 0 ? kLseBytes : 0u);
                 const uint32_t dst = map_to_rank(smem_u32(recv + from), partner);
                 const uint32_t bar = map_to_rank(smem_u32(&ctl->recv_bar[sent]), partner);
                 if (lane == 0)
@@ -404,7 +418,7 @@ __device__ __forceinline__ void cluster_merge_exchange(const DecodeParams &p, Co
             }
         }
     } else if (quarter == 0 && lane == 0) {
-        for (int q = 0; q < 4; ++q) mbar_expect_tx(&ctl->recv_bar[q], kChunkBytes + (q == 0 ? kLseBytes : 0u));
+        for (int q = 0; q < 4; ++q) mbar_expect_tx(&ctl->recv_bar[q], rows * kChunkPitch + (q == 0 ? kLseBytes : 0u));
     }
 
     // ---- finish: the columns kept here (those of the warps with sub == s) never left tensor
@@ -604,7 +618,7 @@ __device__ __forceinline__ void c2_store_result(const DecodeParams &p, uint8_t *
     uint8_t *gbase = (final_out ? reinterpret_cast<uint8_t *>(p.out + u0 * kDv)
                                 : reinterpret_cast<uint8_t *>(p.part_out + u0 * kDv)) + part * (row_bytes / 4);
     const int rows_here = max(0, min(32, head_rows - row0));              // rows of this warp that exist
-    const int rounds = (int)(row_bytes / 4) / kRow;
+    const int rounds = rows_here > 0 ? (int)(row_bytes / 4) / kRow : 0;
     constexpr int kCols16 = kRow / 2, kCols32 = kRow / 4;                 // columns of a round, bf16 and fp32
 #pragma unroll 1
     for (int q = 0; q < rounds; ++q) {
@@ -650,7 +664,7 @@ __device__ __forceinline__ void c2_store_result(const DecodeParams &p, uint8_t *
             if (r < rows_here) *reinterpret_cast<uint4 *>(gq + (size_t)r * row_bytes + (lane % kChunks) * 16) = v[k];
         }
     }
-    if (h < p.heads && part == 0) {
+    if (row < head_rows && part == 0) {
         const float lse = row_lse(lt, m_ref, !final_out);
         if (final_out)
             p.lse[u] = lse;
@@ -703,8 +717,11 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     const int pair = blockIdx.x >> 1;
     C2Unit unit = kClusterMerge ? C2Unit{(int)(blockIdx.x >> 2), (int)(crank >> 1), 2, 0} : c2_unit(p, pair);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform
-    const int h0 = (int)rank * kTcHeads;
-    const int head_rows = min(kTcHeads, p.heads - h0);
+    // The heads are dealt out evenly, so that neither CTA has more rows than it must to exchange and store.  The rows of q behind
+    // them are zeros, see encode_q_map.
+    const int rows = c2_rows(p.heads);
+    const int h0 = (int)rank * rows;
+    const int head_rows = min(rows, p.heads - h0);
 
     // ---- set-up: barriers and tensor memory (nothing here touches global memory, so with a
     // programmatic dependent launch it overlaps the tail of the kernel before this one) --------
@@ -898,11 +915,11 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         // This CTA's K rows are unit 2 t + rank of every tile t, refilled in three groups of three panels as the
         // score MMAs of the tile before retire.
         const uint32_t k_full_leader = map_to_rank(smem_u32(&ctl->k_full[0]), leader);
-        // the columns of q that group g is scored against; a CTA without heads (64 or fewer in all) takes zeros: the
-        // box starts past the last row
+        // the columns of q that group g is scored against
         auto load_q = [&](int g) {
-            tma_box3d_pair(smem_base + kC2SmemQ + g * kC2GroupBytes, &q_map, k_full_leader + 8 * g,
-                           head_rows > 0 ? unit.b * p.heads + h0 : p.batch * p.heads, g * kC2GroupPanels);
+            const bool odd = p.heads & 1;
+            tma_box5d_pair(smem_base + kC2SmemQ + g * kC2GroupBytes, &q_map, k_full_leader + 8 * g, odd ? h0 : 0,
+                           g * kC2GroupPanels, odd ? 0 : (int)rank, unit.b);
         };
         bool any_bad = false, ok = true;
         int round = 0, tile0 = 0;            // tile0: tiles of the units before this one
@@ -1449,7 +1466,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
 
     // ---- tear-down: nobody leaves while the other CTA may still touch this one's memory --
     if (*abort_flag) nap_after_abort();
-    if (kClusterMerge) cluster_merge_exchange(p, ctl, smem, tmem, unit.b, unit.s, crank, h0, head_rows, active, softmax_ok, cm_lse, cm_inv);
+    if (kClusterMerge) cluster_merge_exchange(p, ctl, smem, tmem, unit.b, unit.s, crank, h0, rows, head_rows, active, softmax_ok, cm_lse, cm_inv);
     tc_fence_before();
     __syncthreads();
     // Tensor memory was allocated for the pair, so it is released only when both CTAs are done
@@ -1562,14 +1579,35 @@ inline bool tc2_prepare_device()
     return true;
 }
 
+// q [requests * heads, 576] as the pair kernel loads it: {64 columns, head rows, 9 panels, CTA of the pair, request}.  A CTA's rows
+// end where its half of the heads does, so that a box of 64 rows brings zeros for the others: rows that hold other
+// heads' values would be multiplied for nothing, and long launches are held back by power (64 requests x 33 units of
+// 64 heads 46.1 us with zeros, 48.7 with the neighbours' rows).  An odd number of heads does not halve: there the rows
+// are all heads of the request, and the first CTA's box brings some that are the second's.
+inline bool encode_q_map(CUtensorMap *map, const void *base, uint64_t qrows, uint32_t heads, uint32_t panels)
+{
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const bool odd = heads & 1;
+    const cuuint64_t row = (cuuint64_t)kDqk * 2, rows = odd ? heads : heads / 2;
+    const cuuint64_t dims[5] = {64, rows, (cuuint64_t)kPanels, odd ? 1u : 2u, qrows / heads};
+    const cuuint64_t strides[4] = {row, 128, rows * row, heads * row};
+    const cuuint32_t box[5] = {64, kTcHeads, panels, 1, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // maps[0] = q, maps[1] = K role boxes, maps[2] = V role boxes, maps[3] = whole pages
 inline bool tc2_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cached)
 {
     const uint64_t rows = (uint64_t)p.num_pages * kPage, qrows = (uint64_t)p.batch * p.heads;
     if (cached)
-        return make_panel_map(&maps[0], p.q, qrows, kTcHeads, kC2GroupPanels) && make_panel_map(&maps[1], p.kv, rows, kTile, kC2GroupPanels) &&
-               make_panel_map(&maps[2], p.kv, rows, kTile, 4) && make_panel_map(&maps[3], p.kv, rows, kTile, kPanels);
-    return encode_panel_map(&maps[0], p.q, qrows, kTcHeads, kC2GroupPanels) && encode_panel_map(&maps[1], p.kv, rows, kTile, kC2GroupPanels) &&
+        return cached_map(&maps[0], p.q, qrows, p.heads, kC2GroupPanels, 2, encode_q_map) &&
+               make_panel_map(&maps[1], p.kv, rows, kTile, kC2GroupPanels) && make_panel_map(&maps[2], p.kv, rows, kTile, 4) &&
+               make_panel_map(&maps[3], p.kv, rows, kTile, kPanels);
+    return encode_q_map(&maps[0], p.q, qrows, p.heads, kC2GroupPanels) && encode_panel_map(&maps[1], p.kv, rows, kTile, kC2GroupPanels) &&
            encode_panel_map(&maps[2], p.kv, rows, kTile, 4) && encode_panel_map(&maps[3], p.kv, rows, kTile, kPanels);
 }
 

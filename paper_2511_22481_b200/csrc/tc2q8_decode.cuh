@@ -219,8 +219,9 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
     const int pair = blockIdx.x >> 1;
     C2Unit unit = kClusterMerge ? C2Unit{(int)(blockIdx.x >> 2), (int)(crank >> 1), 2, 0} : c2_unit(p, pair);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform
-    const int h0 = (int)rank * kTcHeads;
-    const int head_rows = min(kTcHeads, p.heads - h0);
+    const int rows = c2_rows(p.heads);
+    const int h0 = (int)rank * rows;                          // (dealt out evenly, as in tc2_decode_kernel)
+    const int head_rows = min(rows, p.heads - h0);
 
     // ---- set-up (no global memory access before the dependent-launch wait) -------------------
     if (threadIdx.x == 0) {
@@ -863,7 +864,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
 
     // ---- tear-down (as in tc2_decode_kernel) ---------------------------------------------------
     if (*abort_flag) nap_after_abort();
-    if (kClusterMerge) cluster_merge_exchange(p, ctl, smem, tmem, b, s, crank, h0, head_rows, active, softmax_ok, cm_lse, cm_inv);
+    if (kClusterMerge) cluster_merge_exchange(p, ctl, smem, tmem, b, s, crank, h0, rows, head_rows, active, softmax_ok, cm_lse, cm_inv);
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
