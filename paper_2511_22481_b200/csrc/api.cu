@@ -69,19 +69,20 @@ int64_t rolling_ring_pages(int32_t n_recent) { return ((int64_t)n_recent + kPage
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
 // Which tensor-core kernel serves a problem: the paired-CTA one (a cluster of two CTAs per work unit)
-// unless there are few heads and little to read.  Up to 64 heads fill only one CTA of a pair, but the
-// other still carries half of every tile's loads and holds half of its operands, and an M = 128 pair runs the
-// tensor pipe at full rate where the single CTA's M = 64 runs it at half rate, with 2 tiles of
-// buffers to the pair's 4: 64 requests x 33 tiles 42 us against 64 with 64 heads, 41 against 58
-// with 16; one request of 128 tiles 17 against 24 and 15.6 against 18.7.  What the single-CTA kernel has is the
-// shorter start and end and twice as many work units, which shows up to 32 heads while two tiles per
-// unit spread over all SMs in one wave (4 requests x 33 tiles of 16 heads: 13.0 against 15.1 us).
-constexpr int kSingleCtaHeads = 32, kSingleCtaUnits = 148;     // (units: the SMs of the device this library is for)
+// unless there are few heads and little to read.  Up to 64 heads leave half of a pair's rows empty, but an M = 128 pair
+// runs the tensor pipe at full rate where the single CTA's M = 64 runs it at half rate, with 2 tiles of
+// buffers to the pair's 4.  What the single-CTA kernel has is the shorter start and twice as many work units, which
+// shows up to 32 heads while two tiles per unit spread over all SMs in one wave (one request of 13 tiles of 16 heads 9.3
+// against 9.7 us on pairs, 4 x 33 11.2 against 12.0, 8 x 33 12.8 against 14.8).
+// More than 40 tiles a request (of at most 32 splits) are two and more tiles a split, at half the pair's rate: one request of 48
+// tiles 11.1 us against 10.8 on pairs, of 96 13.3 against 12.3, of 192 18.9 against 14.3; two requests of 64 tiles 11.8
+// against 13.2, of 96 13.4 against 12.7; four of 64 13.2 against 13.5.
+constexpr int kSingleCtaHeads = 32, kSingleCtaUnits = 148, kSingleCtaTiles = 40;     // (units: the SMs of the device this library is for)
 bool use_pair_kernel(const omni_mla_desc_t *d)
 {
     if (d->flags & OMNI_FLAG_SIMT) return false;
     const int tiles = (d->max_sel + kTile - 1) / kTile;
-    return d->num_heads > kSingleCtaHeads || (long)d->batch * ((tiles + 1) / 2) > kSingleCtaUnits;
+    return d->num_heads > kSingleCtaHeads || (long)d->batch * ((tiles + 1) / 2) > kSingleCtaUnits || tiles > (long)kSingleCtaTiles * d->batch;
 }
 
 // The 8-bit kernel takes more than 64 heads (both CTAs of its pairs have some).

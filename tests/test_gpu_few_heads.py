@@ -19,3 +19,14 @@ def test_head_rows_and_tiles(heads, splits):
     w = W._pack("few heads", 9, heads, pages, W._shuffled_tables(rng, pages, True),
                 [np.asarray(x, dtype=np.int32) for x in lists], "cuda", dict(kind="custom"))
     check_workload(w, 0, num_splits=splits, what="H=%d S=%d" % (heads, splits))
+
+
+@pytest.mark.parametrize("batch,tiles", [(1, 40), (1, 41), (2, 81), (1, 192)])
+def test_either_side_of_forty_tiles_a_request(batch, tiles):
+    """The longest selection that few requests of few heads take to this kernel, and the first that pairs serve."""
+    rng = np.random.default_rng(tiles)
+    lists = [rng.permutation(tiles * 64), np.arange(tiles * 64 - 63)][:batch]
+    pages = [tiles] * batch
+    w = W._pack("forty", 10, 16, pages, W._shuffled_tables(rng, pages, True),
+                [np.asarray(x, dtype=np.int32) for x in lists], "cuda", dict(kind="custom"))
+    check_workload(w, 0, what="B=%d tiles=%d" % (batch, tiles))
