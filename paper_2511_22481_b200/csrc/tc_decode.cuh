@@ -696,6 +696,7 @@ tc_decode_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constan
 #pragma unroll 1
                     for (int c = 0; c < kDv; c += 64) {
                         uint32_t ov[32];
+                        __syncwarp();                       // (the lanes part in the stores below where eight rows are not all heads)
                         tc_ld16x256x8(tmem + lane_base + kColO + (c & 255) + (c >= 256 ? kLane16 : 0u), ov);
                         tc_wait_ld();
 #pragma unroll
