@@ -678,10 +678,11 @@ __device__ __forceinline__ void c2_store_result(const DecodeParams &p, uint8_t *
     }
 }
 
-// Zeroes 128 columns of the warp's tensor-memory lanes.
+// Zeroes 128 columns of the warp's tensor-memory lanes.  (The lanes come here from stores that not all of them took part in.)
 __device__ __forceinline__ void c2_clear(uint32_t at)
 {
     const uint32_t zero[32] = {};
+    __syncwarp();
 #pragma unroll
     for (int c = 0; c < 128; c += 32) tc_st32(at + c, zero);
     tc_wait_st();
