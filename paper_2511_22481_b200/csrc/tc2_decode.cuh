@@ -67,10 +67,12 @@ constexpr int kC2Threads = 384;
 // an earlier tile delays them (requested one tile earlier 25.8 us per step of 32 requests x 33 units, just
 // before those loads 25.5, just after them 24.5).
 constexpr int kScatterAhead = 1;
-// Long work units take the prefetch for their first tiles only.  In a short launch it hides a memory latency per tile; in a
+// Long work units prefetch whole pages for their first tiles only.  In a short launch the prefetch hides a memory latency per tile; in a
 // long one HBM has the requests of many pairs at once anyway, and a prefetch is a third pass through L2 and the copy
 // engine on launches that are held back by power: 32 x 1024 units 703 -> 680 us, 74 x 128 200 -> 186, 128 requests of 8 to
-// 128 units 185.5 -> 182.  Cut there as well, 32 x 33 units (17 a pair) would go from 27.2 to 27.9.
+// 128 units 185.5 -> 182.  Cut there as well, 32 x 33 units (17 a pair) would go from 27.2 to 27.9.  Scattered rows are prefetched
+// throughout: a gathered group waits a latency of its own, however long the unit (without: 37 x 96 units of scattered tokens 99 ->
+// 103 us, 74 x 96 181 -> 184, 32 x 128 183 -> 195, 4 x 256 on a pair each 349 -> 381).
 constexpr int kPrefetchAllUnits = 48, kPrefetchFirstUnits = 8;
 constexpr int kC2GroupPanels = 3;                        // K role: refilled in three groups of three panels
 constexpr int kC2Groups = kPanels / kC2GroupPanels;
@@ -1126,8 +1128,8 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         bool ok = true;
         int round = 0, tile0 = 0;
         do {
-            const int most = kClusterMerge || units < kPrefetchAllUnits ? units : kPrefetchFirstUnits;
-            for (int t0 = (int)rank; ok && t0 < most; t0 += 64) {
+            const int pages_upto = kClusterMerge || units < kPrefetchAllUnits ? units : kPrefetchFirstUnits;
+            for (int t0 = (int)rank; ok && t0 < units; t0 += 64) {
                 const int t = t0 + 2 * lane;
                 const int j0 = begin + t * kC2Tile;
                 int row = -1;
@@ -1140,9 +1142,10 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 }
                 __syncwarp();
                 TileIdx x = {-1, -1, -1, -1};    // of a unit that is not a whole page
-                for (int k = 0; ok && k < 32 && t0 + 2 * k < most; ++k) {
+                for (int k = 0; ok && k < 32 && t0 + 2 * k < units; ++k) {
                     const int i = t0 + 2 * k, running = tile0 + (i >> 1);
                     const bool page = __shfl_sync(0xffffffffu, row, k) >= 0;
+                    if (page && i >= pages_upto) continue;
                     if (!page) {
                         stage_tokens(i, x);
                         stage_pages(x);
