@@ -73,7 +73,10 @@ constexpr int kScatterAhead = 1;
 // 128 units 185.5 -> 182.  Cut there as well, 32 x 33 units (17 a pair) would go from 27.2 to 27.9.  Scattered rows are prefetched
 // throughout: a gathered group waits a latency of its own, however long the unit (without: 37 x 96 units of scattered tokens 99 ->
 // 103 us, 74 x 96 181 -> 184, 32 x 128 183 -> 195, 4 x 256 on a pair each 349 -> 381).
-constexpr int kPrefetchAllUnits = 48, kPrefetchFirstUnits = 8;
+// Where few pairs run, HBM is not busy and the prefetch pays up to longer units (never cut -> always, one unit to a pair): 16 and 32 pairs of
+// 48 units 41.7 -> 42.6 and 44.9 -> 46.2, 32 of 64 58.5 -> 59.4, of 96 86.3 -> 85.8; 40 pairs of 48 53.9 -> 53.8, 56 of them 63.4 -> 61.3, 74 of 64
+// 98.3 -> 95.9, 8 of 96 79.7 -> 76.7.
+constexpr int kPrefetchAllUnits = 48, kPrefetchManyPairs = 40, kPrefetchLongUnits = 96, kPrefetchFirstUnits = 8;
 constexpr int kC2GroupPanels = 3;                        // K role: refilled in three groups of three panels
 constexpr int kC2Groups = kPanels / kC2GroupPanels;
 constexpr int kC2GroupBytes = kC2GroupPanels * kPanelBytes;   // [64 tokens x 128 B] x 3
@@ -1128,7 +1131,8 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         bool ok = true;
         int round = 0, tile0 = 0;
         do {
-            const int pages_upto = kClusterMerge || units < kPrefetchAllUnits ? units : kPrefetchFirstUnits;
+            const int all_upto = (int)(gridDim.x >> 1) < kPrefetchManyPairs ? kPrefetchLongUnits : kPrefetchAllUnits;
+            const int pages_upto = kClusterMerge || units < all_upto ? units : kPrefetchFirstUnits;
             for (int t0 = (int)rank; ok && t0 < units; t0 += 64) {
                 const int t = t0 + 2 * lane;
                 const int j0 = begin + t * kC2Tile;
