@@ -213,6 +213,20 @@ bool merge_in_kernel(const omni_mla_desc_t *d)
     return use_pair_kernel(d) && (d->flags & OMNI_FLAG_FUSED_MERGE);
 }
 
+// The form of the paired-CTA kernel that serves a problem (see tc2_kernel_for): two splits merged inside a cluster, several work units per
+// pair, or one.  Several where there are more units than pairs and they are taken by size (not more than 256 requests), short, and
+// neither cut at the end only nor merged by the last CTA of a request; the units are dealt out as pairs become free.  What is saved is part of the start and the end of every
+// unit but a pair's first: 128 requests x 18 units of a rolling cache 64.7 -> 62.7 us, 128 x 18 of a list 58.4 -> 57.7, 148 x 17
+// 62.2 -> 61.2.  Where the main loop is most of a unit, its inner loop, which has to look for gaps, weighs more: 128 x 64 172 ->
+// 178, 288 units of 114 674 -> 740.
+constexpr int kMultiUnits = 32;
+int pair_form(const omni_mla_desc_t *d, int splits, int whole, bool cluster_merge, bool fused_merge, int pairs)
+{
+    if (cluster_merge) return 1;
+    const int longest = ((d->max_sel + kC2Tile - 1) / kC2Tile + splits - 1) / splits;
+    return whole == 0 && !fused_merge && d->batch <= 256 && (long)d->batch * splits > pairs && longest <= kMultiUnits ? 2 : 0;
+}
+
 // Launch whose blocks may become resident while the kernel in front of it in the stream still runs
 // (programmatic dependent launch); the kernel itself waits (griddepcontrol.wait) before it touches
 // global memory, so only the launch gap between the two kernels goes away.
@@ -350,6 +364,15 @@ int32_t omni_sparse_mla_plan_query(const omni_mla_desc_t *desc, int32_t sm_count
     return s;
 }
 
+// Part of the tests of the dispatch: the form of the paired-CTA kernel that a call with a workspace takes, or -1 where another kernel serves it.
+int32_t omni_internal_pair_form(const omni_mla_desc_t *desc, int32_t sm_count, int32_t resident_merge_clusters)
+{
+    if (!desc_ok(desc) || sm_count < 1 || resident_merge_clusters < 0 || !use_pair_kernel(desc)) return -1;
+    const SplitPlan plan = split_plan(desc, sm_count, resident_merge_clusters);
+    return pair_form(desc, plan.splits, plan.whole, plan.whole == 0 && merge_in_cluster(desc, plan.splits, resident_merge_clusters),
+                     plan.splits > 1 && merge_in_kernel(desc), sm_count / 2);
+}
+
 size_t omni_sparse_mla_workspace_bytes(const omni_mla_desc_t *desc)
 {
     if (!desc_ok(desc)) return 0;
@@ -365,7 +388,7 @@ struct LaunchPlan {
     uint32_t magic;
     int32_t kernel;            // 0 plain-FMA, 1 single-CTA tensor-core, 2 paired-CTA tensor-core, 3 the same over the 8-bit cache
     int32_t splits, whole;     // the first `whole` requests are not split
-    int32_t cluster_merge, longest_first, fused_merge, resident_pairs;
+    int32_t cluster_merge, longest_first, fused_merge, pairs;   // pairs: that the device holds
     int32_t device;
     size_t need, part_out, part_lse, counters;
     omni_mla_desc_t desc;
@@ -410,7 +433,7 @@ static omni_status_t build_plan(const omni_mla_desc_t *desc, const void *q, cons
                            (long)desc->batch * splits > dev.sm_count / 2)
                               ? 1
                               : 0;
-    plan->resident_pairs = plan->kernel == 2 ? tc2_resident().pairs : 0;
+    plan->pairs = dev.sm_count / 2;
     DecodeParams shape = {};
     shape.q = static_cast<const __nv_bfloat16 *>(q);
     shape.kv = static_cast<const __nv_bfloat16 *>(kv_cache);
@@ -501,8 +524,8 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
     p.whole = whole ? 0 : plan.whole;
     p.tail_request = p.whole > 0 ? reinterpret_cast<int32_t *>(static_cast<char *>(workspace) + plan.part_out + plan.part_lse) : nullptr;
     p.cluster_merge = cluster_merge ? 1 : 0;
-    p.longest_first = plan.longest_first;
-    p.resident_pairs = plan.resident_pairs;
+    const int form = pair_form(desc, splits, p.whole, cluster_merge, fused_merge, plan.pairs);
+    p.longest_first = plan.longest_first || (plan.kernel == 2 && form == 2);
     if (fused_merge) {
         p.counters = reinterpret_cast<int32_t *>(static_cast<char *>(workspace) + plan.part_out + plan.part_lse);
         if (cudaMemsetAsync(p.counters, 0, plan.counters, stream) != cudaSuccess) return OMNI_ERR_CUDA;
@@ -524,7 +547,7 @@ static omni_status_t run_plan(const LaunchPlan &plan, const int32_t *page_table,
         if (cudaPeekAtLastError() != cudaSuccess) st = OMNI_ERR_CUDA;
     } else {
         st = plan.kernel == 3   ? tc2q8_launch(plan.maps, p, stream)
-             : plan.kernel == 2 ? tc2_launch(plan.maps, p, stream)
+             : plan.kernel == 2 ? tc2_launch(plan.maps, p, form, stream)
                                 : tc_launch(plan.maps, p, stream);
     }
     if (st != OMNI_OK) return st;

@@ -40,7 +40,6 @@ struct DecodeParams {
     int32_t whole;                 // the first `whole` requests (in the order they are taken) are not split, only the rest
     int32_t *tail_request;         // whole > 0: which request the k-th of the rest is, for the merge kernel
     int32_t longest_first;         // 1: work units take the requests in order of decreasing selection size
-    int32_t resident_pairs;        // CTA pairs that the device holds at once
     float scale_log2;              // softmax_scale * log2(e)
 };
 

@@ -52,7 +52,6 @@
 // head half) in the workspace).
 #pragma once
 
-#include <algorithm>
 #include <type_traits>
 
 #include "merge.cuh"
@@ -115,14 +114,13 @@ struct C2Unit {
     int b, s, splits, slot;
 };
 
-// The same with what every role needs of it: the length the caller gave and the entries [begin, end) of the selection.
+// A further unit of a pair, as it is dealt out: request and split (negative: there is none), the length the caller gave and the entries
+// [begin, end) of the selection.
 struct alignas(16) C2Work {
-    C2Unit unit;
-    int length, begin, end, pad;
+    int request_split, length, begin, end;
 };
-// A pair takes at most this many work units one after the other; with more there are more pairs.  See tc2_launch.
+// A pair takes at most this many work units one after the other.
 constexpr int kC2Rounds = 16;
-constexpr int kC2MultiUnits = 32;                        // longest unit that is taken this way
 
 struct C2Control {
     uint64_t k_full[kC2Groups];          // per tile; those of the first tile wait for q's panels too
@@ -141,11 +139,14 @@ struct C2Control {
     uint32_t merge_flag;
     uint32_t xfail;                      // cluster merge: some wait of this CTA ran out (decided CTA-wide)
     int32_t k_progress;                  // tiles whose K loads have been requested (L2 prefetch pacing)
-    int32_t rounds;                      // work units of this pair
     uint64_t recv_bar[4];                // cluster merge: the partner's chunks have arrived
     uint64_t ready_bar;                  // cluster merge: the partner's main loop is over
     uint64_t taken_bar;                  // cluster merge: the partner's softmax warps have received this CTA's block
     uint64_t xg_bar;                     // row-maximum exchange of a tile
+    // several units per pair: the next cluster that has not begun (grant, asked for by CTA 0) and the unit it is, written to both CTAs
+    uint64_t grant_bar;
+    uint64_t work_full[kC2Rounds];
+    alignas(16) uint4 grant;
     C2Work work[kC2Rounds];
 };
 static_assert(sizeof(C2Control) <= kC2SmemCtlBytes, "control block too large");
@@ -317,6 +318,37 @@ __device__ __forceinline__ void tc_commit_pair_elect(uint64_t *bar, uint16_t bot
         "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
         ::"r"(smem_u32(bar)), "h"(both)
         : "memory");
+}
+
+// Asks for the next cluster of this grid that has not begun, which then never will: 16 bytes that say which one it is, or that there was none
+// to be had, arrive at `response`.  One thread.
+__device__ __forceinline__ void try_cancel_cluster(uint4 *response, uint64_t *bar)
+{
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(smem_u32(response)),
+                 "r"(smem_u32(bar))
+                 : "memory");
+}
+// The first CTA of the cluster that such an answer names, or -1.
+__device__ __forceinline__ int cancelled_cluster(const uint4 *response)
+{
+    int first;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 answer;\n\t"
+        "ld.shared.b128 answer, [%1];\n\t"
+        "mov.b32 %0, -1;\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, answer;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, answer;\n\t}"
+        : "=&r"(first)
+        : "r"(smem_u32(response))
+        : "memory");
+    return first;
+}
+// 16 bytes to a CTA of the cluster, credited to a barrier there.
+__device__ __forceinline__ void st_async16(uint32_t dst_cluster_addr, uint32_t bar_cluster_addr, const int4 &v)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst_cluster_addr), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar_cluster_addr)
+                 : "memory");
 }
 
 // Split-KV merge inside a cluster of two pairs, i.e. the two splits of one request (cluster
@@ -568,7 +600,7 @@ __device__ __forceinline__ void c2_store_empty(const DecodeParams &p, const C2Un
     if (w.splits > 1 && p.counters != nullptr) __threadfence();
 }
 
-// Where a pair takes several work units, the requests are taken longest first (ties by index).  Every CTA ranks
+// Where there are more work units than pairs, the requests are taken longest first (ties by index).  Every CTA ranks
 // the (at most 256) selection sizes itself: request j has rank #{i : n_i > n_j, or n_i = n_j and i < j}.
 // lens: shared memory nobody uses yet (batch + 3 ints).  Called by all threads.  Returns, where only the
 // requests behind the first wave are split (p.whole > 0), whether that pays.  Whole, the longest of them would
@@ -698,10 +730,18 @@ __device__ __forceinline__ void c2_clear(uint32_t at)
 // kernel, fused merge).  kRanges = false: the selection is the caller's index list; true: Eq. 2's two ranges (with or
 // without a rolling cache).  Each instance carries only its own merge, epilogue and index code.
 //
-// Several units per pair (kMulti).  Every role goes through the units on its own; the barriers' phases, the score buffers and the
+// Several units per pair (kMulti).  As many clusters as units are launched, and a pair that is nearly through with its unit takes
+// the place of the next one that has not begun (cluster launch control), so that the units go out longest first to whichever pair
+// becomes free, as they do where the hardware starts a cluster for each.  Dealt out in a fixed pattern instead, a pair with long units waits for nobody
+// and is waited for.  One unit per pair / fixed pattern / this, us: 10 requests of 32 units and 246 of 4 60.1 / 55.6 / 45.3, 30 of 18 and 98 of 4
+// 36.2 / 34.6 / 29.9, 256 sizes spread evenly in the logarithm over 1 to 32 72.9 / 64.1 / 60.7, 128 of them 37.4 / 40.2 / 38.5, 40 of 32 and 100 of 2
+// 42.6 / 46.3 / 43.6, 128 of 18 57.9 / 56.7 / 56.1.  (The two that one unit per pair would do faster have few long
+// units; this form has a longer start and end, and where few pairs run its main loop takes up to 2 % longer.)
+// Every role goes through the units on its own; the barriers' phases, the score buffers and the
 // mask ring go on by a running tile number.  So the loads and the first scores of a unit overlap the end of the one
 // before: q and K follow as its last scores retire, V as its last P V does, and what remains between two units is
 // the epilogue of one and the first softmax of the next.  An odd last tile's second unit is a gap that the barriers count.
+// Launched only with the requests ranked, none cut at the end only (p.whole = 0) and no merge by the last CTA (p.counters null).
 // (`unit` is set where the kernel begins although some instances set it anew: with that line further down the compiler makes
 // 10 % more code of every instance and the merging ones run 1.4 times slower.)
 template <bool kClusterMerge, bool kRanges, bool kMulti>
@@ -755,6 +795,13 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         mbar_init(&ctl->xg_bar, 256);
         mbar_init(&ctl->x_bar, 256);
         mbar_init(&ctl->exit_bar, 2);
+        if (kMulti) {
+            mbar_init(&ctl->grant_bar, 1);
+            for (int i = 1; i < kC2Rounds; ++i) {
+                mbar_init(&ctl->work_full[i], 1);
+                mbar_expect_tx(&ctl->work_full[i], sizeof(C2Work));
+            }
+        }
         for (int i = 0; i < 4; ++i) mbar_init(&ctl->recv_bar[i], 1);
         mbar_init(&ctl->ready_bar, 1);
         mbar_init(&ctl->taken_bar, 8);
@@ -779,62 +826,56 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     // may be scheduled as soon as resources allow; it waits in the same way before it reads.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // The work units of this pair: one, or (fewer pairs than units) one of every round, the order of the pairs turning
-    // round from one to the next so that the sums of sizes that fall from unit to unit come out alike.
-    if (!kClusterMerge && !kMulti) {
+    uint2 order_here = {0, 0};           // kMulti: the requests of ranks 8 lane, ... + 7, a byte each
+    if (!kClusterMerge) {
         bool cut = true;
         int request = unit.b;
         if (p.longest_first) {
             uint8_t *order = smem + 4096;                     // (behind the sizes; shared memory nobody uses yet)
             cut = c2_rank_requests(p, reinterpret_cast<int *>(smem), order);
             request = order[unit.b];
+            if (kMulti) order_here = reinterpret_cast<const uint2 *>(order)[lane];
             __syncthreads();
         }
         c2_name_request(p, unit, request, cut, rank == 0 && threadIdx.x == 0);
     }
-    if (kMulti) {
-        bool cut = true;
-        uint8_t *order = smem + 4096;                         // (behind the sizes; shared memory nobody uses yet)
-        if (p.longest_first) cut = c2_rank_requests(p, reinterpret_cast<int *>(smem), order);
-        const int pairs = (int)(gridDim.x >> 1), all_units = p.whole + (p.batch - p.whole) * p.splits;
-        if (threadIdx.x < kC2Rounds) {
-            const int k = (int)threadIdx.x, at = k * pairs + ((k & 1) ? pairs - 1 - pair : pair);
-            const bool some = k * pairs < all_units && at < all_units;       // (the first k of them)
-            if (some) {
-                C2Work w;
-                w.unit = c2_unit(p, at);
-                c2_name_request(p, w.unit, p.longest_first ? (int)order[w.unit.b] : w.unit.b, cut, rank == 0);
-                w.length = load_length(p, w.unit.b);
-                split_range(w.unit.splits == 0 ? 0 : make_selection(p, w.unit.b, w.length).n, max(w.unit.splits, 1), w.unit.s, w.begin,
-                            w.end, kC2Tile);
-                ctl->work[k] = w;
-            }
-            const uint32_t have = __ballot_sync((1u << kC2Rounds) - 1u, some);
-            if (k == 0) ctl->rounds = __popc(have);
-        }
-        __syncthreads();
-    }
-    // The unit that a warp has in hand; take() moves on to the next.
+    volatile uint32_t *abort_flag = &ctl->abort;
+    // The work unit that a warp has in hand; take() moves on to the next.  Its tiles are numbered on from those of the one before,
+    // [tile0, tile_end), and so are its 64-token units, two a tile, [2 tile0, unit_end); `begin` is the entry where unit 0 would begin.
     Selection selection;
     bool bad_len;
-    int begin, end, units, tiles;
+    int begin, end, units, tile0 = 0, tile_end = 0, unit_end;
     const int32_t *pt;
     auto take = [&](int round) {
-        if (round > 0 && (!kMulti || round >= ctl->rounds)) return false;
-        if (!kMulti) {
+        if (round == 0) {
             selection = load_selection(p, unit.b);
             split_range(!kClusterMerge && unit.splits == 0 ? 0 : selection.n, max(unit.splits, 1), unit.s, begin, end, kC2Tile);
         } else {
-            const C2Work &w = ctl->work[round];
-            unit = w.unit;
-            begin = w.begin;
-            end = w.end;
-            selection = make_selection(p, unit.b, w.length);
+            if (!kMulti || round >= kC2Rounds) return false;
+            if (!__all_sync(0xffffffffu, mbar_wait(&ctl->work_full[round], 0))) {
+                if (lane == 0) {
+                    flag_status(p.status, OMNI_DEV_TIMEOUT);
+                    *abort_flag = 1;
+                }
+                return false;
+            }
+            const int4 w = *reinterpret_cast<const int4 *>(&ctl->work[round]);
+            if (w.x < 0) return false;
+            unit.b = unit.slot = w.x & 0xff;
+            unit.s = w.x >> 8;
+            begin = w.z;
+            end = w.w;
+            selection = make_selection(p, unit.b, w.y);
         }
         __builtin_assume(kRanges ? selection.list == nullptr : selection.list != nullptr);
         bad_len = selection.bad;
         units = (end - begin + kC2Tile - 1) / kC2Tile;
-        tiles = (units + 1) / 2;
+        if (kMulti) {
+            tile0 = tile_end;
+            begin -= 2 * tile0 * kC2Tile;
+        }
+        tile_end = tile0 + (units + 1) / 2;
+        unit_end = 2 * tile0 + units;
         pt = p.page_table + (size_t)unit.b * p.max_pages;
         return true;
     };
@@ -845,7 +886,6 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
     if (!kClusterMerge && !active) c2_store_empty(p, unit, h0, head_rows, warp, kC2Threads / 32, lane);
 
     const uint32_t tmem = ctl->tmem_base;
-    volatile uint32_t *abort_flag = &ctl->abort;
 
     // Index pipeline of the producers.  Lane l serves tokens l and l+32 of a unit.  The three
     // dependent steps (token position -> page id -> pool row) run in different loop iterations, so no
@@ -933,10 +973,10 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                            g * kC2GroupPanels, odd ? 0 : (int)rank, unit.b);
         };
         bool any_bad = false, ok = true;
-        int round = 0, tile0 = 0;            // tile0: tiles of the units before this one
+        int round = 0;
         do {
             any_bad |= bad_len;
-            if (kMulti && tiles == 0) continue;
+            if (kMulti && units == 0) continue;
             if (tile0 == 0 && lane == 0) {
 #pragma unroll
                 for (int g = 0; g < kC2Groups; ++g) load_q(g);
@@ -955,7 +995,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                     uint64_t mask;
                     bool whole;
                     stage_rows(2 * tile + h, x[h], lo, hi, mask, whole, first, any_bad);
-                    if (lane == 0) ctl->valid_mask[(2 * (tile0 + tile) + h) % kMaskRing] = mask;
+                    if (lane == 0) ctl->valid_mask[(2 * tile + h) % kMaskRing] = mask;
                     if (h == (int)rank) {
                         row_lo = lo;
                         row_hi = hi;
@@ -973,16 +1013,16 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 TileIdx x0[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    stage_tokens(h, x0[h]);
-                    stage_tokens(2 + h, x1[h]);
-                    stage_tokens(4 + h, x2[h]);
+                    stage_tokens(2 * tile0 + h, x0[h]);
+                    stage_tokens(2 * tile0 + 2 + h, x1[h]);
+                    stage_tokens(2 * tile0 + 4 + h, x2[h]);
                 }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     stage_pages(x0[h]);
                     stage_pages(x1[h]);
                 }
-                resolve_tile(0, x0);
+                resolve_tile(tile0, x0);
             }
             // gathered groups whose bytes are not credited yet, first in first out: a single scattered group takes
             // about a memory latency, so all three are requested before the first is waited for
@@ -992,25 +1032,24 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 oldest = oldest == kC2Groups - 1 ? 0 : oldest + 1;
             };
             const char *kv_bytes = reinterpret_cast<const char *>(p.kv);
-            for (int tile = 0; ok && tile < tiles; ++tile) {
+            for (int tile = tile0; ok && tile < tile_end; ++tile) {
                 // The last tile has a single unit when their number is odd: CTA 1 then leaves its half of the K
                 // rows as it is (the scores of those tokens are masked) and credits the bytes all the same.  Every
                 // tile's scores thus wait for this warp of either CTA: for the masks it has written by then, and
                 // because k_empty must not get two phases ahead of a wait below, whose parity would then match again and
                 // the wait run out.
-                const bool mine = 2 * tile + (int)rank < units;
-                const uint32_t bytes = (tile == 0 ? 4 : 2) * kC2GroupBytes;
-                const int running = tile0 + tile;
+                const bool mine = 2 * tile + (int)rank < unit_end;
+                const uint32_t bytes = (tile == tile0 ? 4 : 2) * kC2GroupBytes;
 #pragma unroll 1
                 for (int g = 0; g < kC2Groups; ++g) {
-                    if (running > 0) {
+                    if (tile > 0) {
                         // nothing to do until the group is free: credit what has landed meanwhile
-                        while (waiting > 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->k_empty[g], (running - 1) & 1))) credit_oldest();
-                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->k_empty[g], (running - 1) & 1));
+                        while (waiting > 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->k_empty[g], (tile - 1) & 1))) credit_oldest();
+                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->k_empty[g], (tile - 1) & 1));
                         if (!ok) break;
                     }
                     if (lane == 0 && rank == 0) mbar_expect_tx(&ctl->k_full[g], bytes);
-                    if (kMulti && tile == 0 && tile0 > 0 && lane == 0) load_q(g);      // (the scores that read the q before have retired)
+                    if (kMulti && tile == tile0 && tile0 > 0 && lane == 0) load_q(g);  // (the scores that read the q before have retired)
                     if (!mine) {
                         if (lane == 0) credit_bytes(k_full_leader + 8 * g, kC2GroupBytes);
                         continue;
@@ -1023,14 +1062,14 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                         if (waiting++ == 0) oldest = g;
                     }
                 }
-                if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = running + 1;
+                if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = tile + 1;
                 // (before the index work: that fits into the time the score MMAs then take)
                 while (waiting > 0) credit_oldest();
                 ok = ok && (*abort_flag == 0);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 // advance the index pipeline: rows of the next tile, page ids of the one after, positions of the third
-                if (tile + 1 < tiles) resolve_tile(tile + 1, x1);
+                if (tile + 1 < tile_end) resolve_tile(tile + 1, x1);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     x1[h] = x2[h];
@@ -1038,7 +1077,6 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                     stage_tokens(2 * tile + 6 + h, x2[h]);
                 }
             }
-            tile0 += tiles;
         } while (ok && take(++round));
         if (lane == 0) *const_cast<volatile int32_t *>(&ctl->k_progress) = 0x7fffffff;
         if (!ok && lane == 0) {
@@ -1050,7 +1088,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         // =========================== V-role producer =====================================
         // This CTA's V columns are [256*rank, 256*rank+256) = panels [4*rank, 4*rank+4) of all 64 tokens.
         bool any_bad = false, ok = true;
-        int round = 0, step0 = 0;            // step0: V loads of the units before this one, two a tile
+        int round = 0;
         int pending = -1;                    // stage of a gathered unit whose bytes are not credited yet
         const char *kv_bytes = reinterpret_cast<const char *>(p.kv);
         do {
@@ -1062,25 +1100,26 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 // the position loads of the first three units go out together, then the two page-id
                 // loads that depend on them: two cache misses in a row before the first copy, not four
                 TileIdx x0;
-                stage_tokens(0, x0);
-                stage_tokens(1, x1);
-                stage_tokens(2, x2);
+                const int first = 2 * tile0;
+                stage_tokens(first, x0);
+                stage_tokens(first + 1, x1);
+                stage_tokens(first + 2, x2);
                 stage_pages(x0);
                 stage_pages(x1);
-                stage_rows(0, x0, row_lo, row_hi, mask_unused, contig, box_unused, any_bad);
+                stage_rows(first, x0, row_lo, row_hi, mask_unused, contig, box_unused, any_bad);
             }
-            for (int i = 0; ok && i < (kMulti ? 2 * tiles : units); ++i) {
-                const int st = i & 1, running = step0 + i;
-                if (running >= 2) {
-                    if (pending >= 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->pv_done[st], ((running >> 1) - 1) & 1))) {
+            for (int i = 2 * tile0; ok && i < (kMulti ? 2 * tile_end : unit_end); ++i) {
+                const int st = i & 1;
+                if (i >= 2) {
+                    if (pending >= 0 && !__all_sync(0xffffffffu, mbar_test(&ctl->pv_done[st], ((i >> 1) - 1) & 1))) {
                         retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, 0, lane);
                         pending = -1;
                     }
-                    ok = mbar_wait(&ctl->pv_done[st], ((running >> 1) - 1) & 1);
+                    ok = mbar_wait(&ctl->pv_done[st], ((i >> 1) - 1) & 1);
                 }
                 ok = __all_sync(0xffffffffu, ok) && (*abort_flag == 0);
                 if (!ok) break;
-                if (kMulti && i >= units) {
+                if (kMulti && i >= unit_end) {
                     // an odd last tile has no second unit: only the phases of its barriers go on
                     if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, 0, lane);
                     pending = -1;
@@ -1106,17 +1145,16 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 if (gathered) {
                     pending = st;
                     // the next stage is still in use: credit this one before the index work
-                    if (running >= 1 && !__all_sync(0xffffffffu, mbar_test(&ctl->pv_done[st ^ 1], (((running + 1) >> 1) - 1) & 1))) {
+                    if (i >= 1 && !__all_sync(0xffffffffu, mbar_test(&ctl->pv_done[st ^ 1], (((i + 1) >> 1) - 1) & 1))) {
                         retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, 0, lane);
                         pending = -1;
                     }
                 }
-                if (i + 1 < units) stage_rows(i + 1, x1, row_lo, row_hi, mask_unused, contig, box_unused, any_bad);
+                if (i + 1 < unit_end) stage_rows(i + 1, x1, row_lo, row_hi, mask_unused, contig, box_unused, any_bad);
                 x1 = x2;
                 stage_pages(x1);
                 stage_tokens(i + 3, x2);
             }
-            step0 += 2 * tiles;
         } while (ok && take(++round));
         if (pending >= 0) retire_gathered_stage(map_to_rank(smem_u32(&ctl->v_full[pending]), leader), kC2VBytes, 0, lane);
         if (!ok && lane == 0) {
@@ -1129,15 +1167,45 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         // order (first position page-aligned, last position 63 further) by one tensor prefetch, anything
         // else row by row.  Lane l looks at the ends of unit r + 2 l, ... of a batch of 32 in parallel.
         bool ok = true;
-        int round = 0, tile0 = 0;
+        int round = 0;
+        // Several units per pair: CTA 0 asks for the next one and hands it to both CTAs, some 3 us before the pair is free; the answer takes
+        // 0.3 us.  Where the unit in hand ends in a whole page it asks once the K loads of the last tile have been requested (the earlier, the less
+        // is known of who is free first: a tile earlier 75 x 32 and one of 16 units take 60.9 us, not 58.2), behind scattered rows at once, two
+        // tiles earlier, since the next unit's are late without a prefetch (100 x 11 after a selection 57.1 -> 55.7).
+        auto deal = [&](int round) {
+            if (lane == 0) {
+                mbar_expect_tx(&ctl->grant_bar, sizeof(ctl->grant));
+                try_cancel_cluster(&ctl->grant, &ctl->grant_bar);
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait(&ctl->grant_bar, (round - 1) & 1))) {
+                if (lane == 0) {
+                    flag_status(p.status, OMNI_DEV_TIMEOUT);
+                    *abort_flag = 1;
+                }
+                return;
+            }
+            const int first = __shfl_sync(0xffffffffu, cancelled_cluster(&ctl->grant), 0);
+            fence_async_smem();                               // (the next answer is written by the asynchronous proxy)
+            int4 w = {-1, 0, 0, 0};
+            if (first >= 0) {
+                const C2Unit next = c2_unit(p, first >> 1);
+                const uint32_t word = __shfl_sync(0xffffffffu, (next.b & 4) ? order_here.y : order_here.x, next.b >> 3);
+                const int b = (int)(word >> (8 * (next.b & 3))) & 0xff;
+                w.x = b | (next.s << 8);
+                w.y = load_length(p, b);
+                split_range(make_selection(p, b, w.y).n, p.splits, next.s, w.z, w.w, kC2Tile);
+            }
+            if (lane < 2) st_async16(map_to_rank(smem_u32(&ctl->work[round]), lane), map_to_rank(smem_u32(&ctl->work_full[round]), lane), w);
+        };
         do {
             const int all_upto = (int)(gridDim.x >> 1) < kPrefetchManyPairs ? kPrefetchLongUnits : kPrefetchAllUnits;
-            const int pages_upto = kClusterMerge || units < all_upto ? units : kPrefetchFirstUnits;
-            for (int t0 = (int)rank; ok && t0 < units; t0 += 64) {
+            bool paged = false;                               // the last of these units is a whole page
+            const int pages_upto = kClusterMerge || units < all_upto ? unit_end : kPrefetchFirstUnits;
+            for (int t0 = 2 * tile0 + (int)rank; ok && t0 < unit_end; t0 += 64) {
                 const int t = t0 + 2 * lane;
                 const int j0 = begin + t * kC2Tile;
                 int row = -1;
-                if (t < units && j0 + kC2Tile <= end) {
+                if (t < unit_end && j0 + kC2Tile <= end) {
                     const int first = selection_at(selection, j0), last = selection_at(selection, j0 + kC2Tile - 1);
                     if (first >= 0 && first % kPage == 0 && last == first + kC2Tile - 1 && first / kPage < p.max_pages) {
                         const int pg = ldg_index(pt + first / kPage, selection.keep);
@@ -1146,9 +1214,10 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 }
                 __syncwarp();
                 TileIdx x = {-1, -1, -1, -1};    // of a unit that is not a whole page
-                for (int k = 0; ok && k < 32 && t0 + 2 * k < units; ++k) {
-                    const int i = t0 + 2 * k, running = tile0 + (i >> 1);
+                for (int k = 0; ok && k < 32 && t0 + 2 * k < unit_end; ++k) {
+                    const int i = t0 + 2 * k, tile = i >> 1;
                     const bool page = __shfl_sync(0xffffffffu, row, k) >= 0;
+                    if (kMulti) paged = page;
                     if (page && i >= pages_upto) continue;
                     if (!page) {
                         stage_tokens(i, x);
@@ -1157,7 +1226,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                     // a page is prefetched once the K loads of the tile before have been requested (a monotonic
                     // counter, polled with a bounded number of naps)
                     const volatile int32_t *progress = &ctl->k_progress;
-                    for (int naps = 0; *progress < running - (page ? 0 : kScatterAhead) && *abort_flag == 0; ++naps) {
+                    for (int naps = 0; *progress < tile - (page ? 0 : kScatterAhead) && *abort_flag == 0; ++naps) {
                         if (naps > (1 << 22)) {
                             ok = false;
                             break;
@@ -1170,14 +1239,19 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                         asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(&kv_tile_map),
                                      "r"(0), "r"(row), "r"(0)
                                      : "memory");
-                    if (ok && !page && *progress <= running) {      // (not once the unit's own loads are out)
+                    if (ok && !page && *progress <= tile) {      // (not once the unit's own loads are out)
                         if ((uint32_t)x.pg0 < page_limit) prefetch_row(p.kv, x.pg0 * kPage + (x.t0 & (kPage - 1)));
                         if ((uint32_t)x.pg1 < page_limit) prefetch_row(p.kv, x.pg1 * kPage + (x.t1 & (kPage - 1)));
                     }
                     __syncwarp();
                 }
             }
-            tile0 += tiles;
+            if (kMulti && rank == 0 && ok && round + 1 < kC2Rounds) {
+                const volatile int32_t *progress = &ctl->k_progress;
+                for (int naps = 0; paged && *progress < tile_end && *abort_flag == 0 && naps < (1 << 22); ++naps) __nanosleep(100);
+                __syncwarp();
+                deal(round + 1);
+            }
         } while (ok && take(++round));
     } else if (warp == 1) {
         // =========================== MMA issuer (CTA 0 only) =============================
@@ -1193,25 +1267,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             // Values that steer the loop are broadcast from lane 0 so that the compiler can see
             // they are warp-uniform and keep the descriptor arithmetic on the uniform datapath;
             // with thread-dependent control flow every MMA costs ~70 clocks to issue instead of ~25.
-            // sizes of this pair's work units, a round to a lane, and the tiles of all of them
-            int sizes = 0, gap_here = 0, tiles_u, steps_u;
-            if (kMulti) {
-                const C2Work &w = ctl->work[lane & (kC2Rounds - 1)];
-                if (lane < ctl->rounds) sizes = (w.end - w.begin + kC2Tile - 1) / kC2Tile;
-                tiles_u = __shfl_sync(0xffffffffu, (int)__reduce_add_sync(0xffffffffu, (uint32_t)(sizes + 1) / 2), 0);
-                steps_u = 2 * tiles_u;
-                // the last step of this lane's work unit
-                int upto = (sizes + 1) / 2;
-#pragma unroll
-                for (int d = 1; d < kC2Rounds; d <<= 1) {
-                    const int o = __shfl_up_sync(0xffffffffu, upto, d);
-                    if (lane >= d) upto += o;
-                }
-                gap_here = 2 * upto - 1;
-            } else {
-                tiles_u = __shfl_sync(0xffffffffu, tiles, 0);
-                steps_u = __shfl_sync(0xffffffffu, units, 0);
-            }
+            const int tiles_u = __shfl_sync(0xffffffffu, tile_end, 0), units_u = __shfl_sync(0xffffffffu, units, 0);
             const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
             // One copy of each issue routine: group, stage and buffer enter as warp-uniform run-time values
             // (every operand of an MMA is then a uniform base plus a compile-time offset), which
@@ -1244,56 +1300,60 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             // Whatever is ready goes next, scores first (P V first was 1 to 5 % slower): group g of tile t once its
             // K panels have landed and (first group) the score buffer t % 3 is free; P V of unit u once the
             // weights of its tile are written and its V rows have landed.
-            // Scores run ahead of P V across the work units.  u: steps of P V, two a tile; the second of an odd last tile (a
-            // gap) multiplies nothing.  Every step but the first adds to O, which the softmax warps clear between two units.
-            auto next_gap = [&](int after) {
-                const uint32_t mine = kMulti && (sizes & 1) && gap_here > after ? (uint32_t)gap_here : 0x7fffffffu;
-                return __shfl_sync(0xffffffffu, (int)__reduce_min_sync(0xffffffffu, mine), 0);
-            };
+            // u counts steps of P V, two a tile.  Several units per pair: scores run ahead of P V across the units, and every step but the
+            // first adds to O, which the softmax warps clear between two units.
             bool ok = true;
             int t = 0, g = 0, u = 0, sbuf = 0, sph = 1;     // sph: parity of the wait on s_empty (the first use passes at once)
-            int gap = kMulti ? next_gap(-1) : 0;
+            int round = 0, stop = units_u;                  // stop: the step behind the unit that P V is at, a gap if that is odd
             long long start = 0;
             uint32_t idle = 0;
-            while (ok && u < steps_u) {
-                const bool qk = t < tiles_u && mbar_test(&ctl->k_full[g], t & 1) && (g > 0 || mbar_test(&ctl->s_empty[sbuf], sph));
-                if (__all_sync(0xffffffffu, qk)) {
-                    tc_fence_after();
-                    issue_qk(g, sbuf);
-                    if (++g == kC2Groups) {
-                        g = 0;
-                        ++t;
-                        if (++sbuf == 3) {
-                            sbuf = 0;
-                            sph ^= 1;
+            do {
+                while (ok && u < stop) {
+                    const bool qk = (kMulti || t < tiles_u) && mbar_test(&ctl->k_full[g], t & 1) && (g > 0 || mbar_test(&ctl->s_empty[sbuf], sph));
+                    if (__all_sync(0xffffffffu, qk)) {
+                        tc_fence_after();
+                        issue_qk(g, sbuf);
+                        if (++g == kC2Groups) {
+                            g = 0;
+                            ++t;
+                            if (++sbuf == 3) {
+                                sbuf = 0;
+                                sph ^= 1;
+                            }
                         }
+                        idle = 0;
+                        continue;
                     }
-                    idle = 0;
-                    continue;
-                }
-                const bool pv = mbar_test(&ctl->p_full, (u >> 1) & 1) && mbar_test(&ctl->v_full[u & 1], (u >> 1) & 1);
-                if (__all_sync(0xffffffffu, pv)) {
-                    tc_fence_after();
-                    if (!kMulti || u != gap) {
+                    const bool pv = mbar_test(&ctl->p_full, (u >> 1) & 1) && mbar_test(&ctl->v_full[u & 1], (u >> 1) & 1);
+                    if (__all_sync(0xffffffffu, pv)) {
+                        tc_fence_after();
                         issue_pv(u & 1, u == 0);
-                    } else {
-                        gap = next_gap(u);
+                        tc_commit_pair_elect(&ctl->pv_done[u & 1], pair_mask);
+                        ++u;
+                        idle = 0;
+                        continue;
                     }
-                    tc_commit_pair_elect(&ctl->pv_done[u & 1], pair_mask);
+                    // bounded: the clock is read now and then while nothing is ready
+                    if ((++idle & 63u) == 0u) {
+                        const long long now = __shfl_sync(0xffffffffu, clock64(), 0);
+                        if (idle == 64u)
+                            start = now;
+                        else
+                            ok = now - start <= kWaitCycles;
+                        ok = ok && __shfl_sync(0xffffffffu, *abort_flag, 0) == 0u;
+                    }
+                }
+                if (!kMulti || !ok) break;
+                if (u & 1) {
+                    // the gap: its barriers' phases only
+                    ok = __all_sync(0xffffffffu, mbar_wait(&ctl->v_full[1], (u >> 1) & 1));
+                    if (!ok) break;
+                    tc_commit_pair_elect(&ctl->pv_done[1], pair_mask);
                     ++u;
-                    idle = 0;
-                    continue;
                 }
-                // bounded: the clock is read now and then while nothing is ready
-                if ((++idle & 63u) == 0u) {
-                    const long long now = __shfl_sync(0xffffffffu, clock64(), 0);
-                    if (idle == 64u)
-                        start = now;
-                    else
-                        ok = now - start <= kWaitCycles;
-                    ok = ok && __shfl_sync(0xffffffffu, *abort_flag, 0) == 0u;
-                }
-            }
+                if (!take(++round)) break;
+                stop = u + __shfl_sync(0xffffffffu, units, 0);
+            } while (true);
             if (!ok && lane == 0) {
                 flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_MMA);
                 *abort_flag = 1;
@@ -1314,7 +1374,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         const uint32_t s_empty_leader = map_to_rank(smem_u32(&ctl->s_empty[0]), leader);   // [1], [2] follow at +8, +16
         const uint32_t p_full_leader = map_to_rank(smem_u32(&ctl->p_full), leader);
         bool ok = true;
-        int round = 0, tile0 = 0, sbuf = 0, sph = 0;        // sph: parity of the wait on s_full
+        int round = 0, sbuf = 0, sph = 0;        // sph: parity of the wait on s_full
         // Every tile is worked on by all eight warps: a thread serves head row `row` and 32 of the 128 tokens,
         // [64 half + 32 sub, + 32), and the four threads of a row meet over its maximum through shared
         // memory.  (Two groups of four warps that take the tiles in turn, 64 tokens a thread, overlap one
@@ -1323,14 +1383,13 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         // units 16.8 us that way, 16.2 this way.)
         const int tq = half * 2 + sub;                     // quarter of the tile's tokens
         do {
-            if (kMulti && tiles == 0) {
+            if (kMulti && units == 0) {
                 // an empty split (the same decision in both CTAs of the pair): zeros and -inf, no pipeline
                 c2_store_empty(p, unit, h0, head_rows, warp < 8 ? warp - 2 : warp - 4, 8, lane);
                 continue;
             }
             float m_ref = -INFINITY, l = 0.f;
-            for (int i = 0; i < tiles; ++i) {
-                const int running = tile0 + i;
+            for (int i = tile0; i < tile_end; ++i) {
                 ok = mbar_wait(&ctl->s_full[sbuf], sph);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
@@ -1347,7 +1406,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                     sbuf = 0;
                     sph ^= 1;
                 }
-                const uint32_t valid = (uint32_t)(ctl->valid_mask[(2 * running + half) % kMaskRing] >> (32 * sub));
+                const uint32_t valid = (uint32_t)(ctl->valid_mask[(2 * i + half) % kMaskRing] >> (32 * sub));
                 // x * xs is the scaled score of a token.  Under a positive scale x is the raw score: the
                 // maximum is taken on them and the scale rides on the fused multiply-add in front of the
                 // exponential, one instruction less per token.
@@ -1363,12 +1422,12 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                         if (!((valid >> j) & 1u)) sv[j] = __float_as_uint(-INFINITY);
                 }
                 float mt = fmaxf(max32([&](int j) { return __uint_as_float(sv[j]); }), -INFINITY) * xs;
-                float *xg = &ctl->xchg[running & 1][0][row];
+                float *xg = &ctl->xchg[i & 1][0][row];
                 // (the row sums of the unit before went through the same slots: everybody has read them)
-                if (kMulti && i == 0 && tile0 > 0) ok = mbar_wait(&ctl->x_bar, 1);
+                if (kMulti && i == tile0 && tile0 > 0) ok = mbar_wait(&ctl->x_bar, 1);
                 xg[tq * 64] = mt;
                 mbar_arrive(&ctl->xg_bar);
-                ok = mbar_wait(&ctl->xg_bar, running & 1) && ok;
+                ok = mbar_wait(&ctl->xg_bar, i & 1) && ok;
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
                     break;
@@ -1397,8 +1456,8 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 l = l * factor + (sum.x + sum.y);
                 // P and O are free once P V of the tile before (its second unit: only the last tile can have a
                 // single one) retired
-                if (i >= 1) {
-                    ok = mbar_wait(&ctl->pv_done[1], (running - 1) & 1);
+                if (i > tile0) {
+                    ok = mbar_wait(&ctl->pv_done[1], (i - 1) & 1);
                     if (!__all_sync(0xffffffffu, ok)) {
                         ok = false;
                         break;
@@ -1434,7 +1493,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             // that tile, which it reached only after reading the slots of the tile before.
             float lt = 0.f;
             if (ok) {
-                float *sums = &ctl->xchg[(tile0 + tiles) & 1][0][row];
+                float *sums = &ctl->xchg[tile_end & 1][0][row];
                 sums[tq * 64] = l;
                 mbar_arrive(&ctl->x_bar);
                 ok = mbar_wait(&ctl->x_bar, 0);
@@ -1446,7 +1505,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 cm_inv = lt > 0.f ? 1.f / lt : 0.f;
                 cm_lse = row_lse(lt, m_ref, true);
                 // now the last P V
-                const int last = kMulti ? 2 * (tile0 + tiles) - 1 : units - 1;
+                const int last = kMulti ? 2 * tile_end - 1 : units - 1;
                 ok = mbar_wait(&ctl->pv_done[last & 1], (last >> 1) & 1);
                 ok = __all_sync(0xffffffffu, ok);
             }
@@ -1460,16 +1519,16 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
                 tc_fence_after();
                 // With more units to come only the P buffer is free to stage in: the next tile's weights are written once all eight warps
                 // are through.
-                if (kMulti)
+                if (kMulti) {
                     c2_store_result<64>(p, smem + kC2SmemP, tmem, warp, lane, unit, h0, head_rows, lt, m_ref);
-                else
+                    c2_clear(tmem + lane_base + kColO + 128 * sub);
+                } else {
                     c2_store_result<128>(p, smem, tmem, warp, lane, unit, h0, head_rows, lt, m_ref);
-                if (kMulti) c2_clear(tmem + lane_base + kColO + 128 * sub);
+                }
                 tc_fence_before();
                 // with the in-kernel merge the partial results must be visible before this CTA is counted
-                if (unit.splits != 1 && p.counters != nullptr) __threadfence();
+                if (!kMulti && unit.splits != 1 && p.counters != nullptr) __threadfence();
             }
-            tile0 += tiles;
         } while (ok && take(++round));
         if (!ok && lane == 0) {
             flag_status(p.status, OMNI_DEV_TIMEOUT | OMNI_DEV_ROLE_SOFTMAX);
@@ -1504,7 +1563,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
     // ---- split merge by whichever CTA finishes a (request, head half) last ---------------
-    if (!kClusterMerge && p.splits > 1 && p.counters != nullptr)
+    if (!kClusterMerge && !kMulti && p.splits > 1 && p.counters != nullptr)
         merge_if_last(p, unit.b, (int)rank, 2, h0, head_rows, reinterpret_cast<float *>(smem), &ctl->merge_flag);
 }
 
@@ -1533,48 +1592,39 @@ inline C2KernelFn tc2_kernel_for(int form, bool ranges)
     return table[form][ranges ? 1 : 0];
 }
 
-// Clusters of `ctas` CTAs of a kernel that can be resident at once on the current device, or 0.
-inline int tc2_resident_clusters(C2KernelFn kernel, unsigned ctas)
+// Clusters of two pairs (cluster merge) that can be resident at once on the current device, or 0.
+inline int tc2_max_merge_clusters()
 {
-    int n = 0;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kC2SmemBytes) != cudaSuccess) return 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas * 64);
-    cfg.blockDim = dim3(kC2Threads);
-    cfg.dynamicSmemBytes = kC2SmemBytes;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        n = 0;
-    }
-    return n;
-}
-
-// Clusters of two pairs (cluster merge) and of one (several work units per pair); asked once per device.
-struct C2Resident {
-    int merge_clusters, pairs;
-};
-inline C2Resident tc2_resident()
-{
-    static C2Resident cached[64];
+    static int cached[64];
     static bool known[64] = {};
     static std::mutex mu;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return {0, 0};
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     std::lock_guard<std::mutex> lock(mu);
     if (!known[dev]) {
-        cached[dev] = {tc2_resident_clusters(tc2_decode_cm_kernel, 4), tc2_resident_clusters(tc2_decode_multi_kernel, 2)};
+        int n = 0;
+        if (cudaFuncSetAttribute(tc2_decode_cm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kC2SmemBytes) == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(4 * 64);
+            cfg.blockDim = dim3(kC2Threads);
+            cfg.dynamicSmemBytes = kC2SmemBytes;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 4;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&n, tc2_decode_cm_kernel, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+        }
+        cached[dev] = n;
         known[dev] = true;
     }
     return cached[dev];
 }
-inline int tc2_max_merge_clusters() { return tc2_resident().merge_clusters; }
 
 inline bool tc2_prepare_device()
 {
@@ -1625,21 +1675,11 @@ inline bool tc2_make_maps(const DecodeParams &p, CUtensorMap *maps, bool cached)
            encode_panel_map(&maps[2], p.kv, rows, kTile, 4) && encode_panel_map(&maps[3], p.kv, rows, kTile, kPanels);
 }
 
-inline omni_status_t tc2_launch(const CUtensorMap *maps, const DecodeParams &p, cudaStream_t stream)
+// form: see tc2_kernel_for
+inline omni_status_t tc2_launch(const CUtensorMap *maps, const DecodeParams &p, int form, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
-    // Several work units per pair, one after the other, where they are taken by size (sizes that nobody ranks are better dealt
-    // out by the hardware as pairs become free), are short, and are not merged by the last CTA of a request.  What is saved is
-    // part of the start and the end of every unit but a pair's first: 128 requests x 18 units of a rolling cache 64.7 ->
-    // 62.7 us, 128 x 18 of a list 58.4 -> 57.7, 148 x 17 62.2 -> 61.2.  Where the main loop is most of a unit, its inner loop,
-    // which has to look for gaps, weighs more: 128 x 64 172 -> 178, 288 units of 114 674 -> 740.
-    const int all = p.whole + (p.batch - p.whole) * p.splits;
-    const int longest = ((p.max_sel + kC2Tile - 1) / kC2Tile + p.splits - 1) / p.splits;
-    int pairs = all;
-    if (!p.cluster_merge && p.longest_first && p.whole == 0 && p.counters == nullptr && longest <= kC2MultiUnits && p.resident_pairs > 0)
-        pairs = std::max(std::min(all, p.resident_pairs), (all + kC2Rounds - 1) / kC2Rounds);
-    const int form = p.cluster_merge ? 1 : pairs < all ? 2 : 0;
-    cfg.gridDim = dim3((unsigned)(pairs * 2));
+    cfg.gridDim = dim3((unsigned)((p.whole + (p.batch - p.whole) * p.splits) * 2));
     cfg.blockDim = dim3(kC2Threads);
     cfg.dynamicSmemBytes = kC2SmemBytes;
     cfg.stream = stream;

@@ -1,6 +1,7 @@
 """The split plan where it weighs a merge in a cluster, the merge kernel and the number of partial results
 against each other (148 SMs, 33 resident merging clusters).  The counts are the fastest, or within 4 % of
 it, of all those measured at the shape."""
+import ctypes
 import math
 
 import pytest
@@ -25,6 +26,20 @@ def test_split_choice(batch, heads, units, want):
     builder.build()
     d = B.make_desc(batch, heads, batch * units, units, units * 64, 1.0 / math.sqrt(192.0))
     assert B.omni_sparse_mla_plan_query(d, 148, 33) == want
+
+
+@pytest.mark.parametrize("batch,heads,units,splits,flags,want", [
+    (75, 128, 32, 1, 0, 2), (75, 128, 33, 1, 0, 0), (74, 128, 32, 1, 0, 0),       # more units than pairs, none longer than 32
+    (256, 128, 18, 1, 0, 2), (257, 128, 18, 1, 0, 0),                             # as many as the kernel ranks
+    (40, 128, 64, 2, 0, 2), (33, 128, 64, 2, 0, 1), (100, 40, 12, 13, 0, 2),      # splits; a merge in a cluster
+    (100, 128, 12, 3, B.OMNI_FLAG_FUSED_MERGE, 0),                                # a merge by the last CTA
+    (76, 128, 64, 0, 0, 0),                                                       # only the last two requests are cut
+    (4, 16, 4, 0, 0, -1),                                                         # single-CTA kernel
+])
+def test_units_per_pair(batch, heads, units, splits, flags, want):
+    builder.build()
+    d = B.make_desc(batch, heads, batch * units, units, units * 64, 1.0 / math.sqrt(192.0), num_splits=splits, flags=flags)
+    assert B.load().omni_internal_pair_form(ctypes.byref(d), 148, 33) == want
 
 
 @pytest.mark.gpu
