@@ -602,7 +602,8 @@ __device__ __forceinline__ void c2_store_empty(const DecodeParams &p, const C2Un
 
 // Where there are more work units than pairs, the requests are taken longest first (ties by index).  Every CTA ranks
 // the (at most 256) selection sizes itself: request j has rank #{i : n_i > n_j, or n_i = n_j and i < j}.
-// lens: shared memory nobody uses yet (batch + 3 ints).  Called by all threads.  Returns, where only the
+// lens: shared memory nobody uses yet (batch + 3 ints); order: the same, the request of every rank.  Called by all threads; the caller hands
+// the memory to the producers' copies with c2_release_scratch once it has read `order`.  Returns, where only the
 // requests behind the first wave are split (p.whole > 0), whether that pays.  Whole, the longest of them would
 // start when the shortest of the first wave ends; only if it then ends after the longest of all, by more than
 // a merge costs (12 units), do pieces help.
@@ -622,9 +623,14 @@ __device__ __forceinline__ bool c2_rank_requests(const DecodeParams &p, int *len
         if (before == p.whole) mark[2] = nj;
     }
     __syncthreads();
-    const bool cut = p.whole == 0 || (int64_t)mark[1] + mark[2] > (int64_t)mark[0] + kCutGain;
-    __syncthreads();                                          // the shared memory is handed to the producers next
-    return cut;
+    return p.whole == 0 || (int64_t)mark[1] + mark[2] > (int64_t)mark[0] + kCutGain;
+}
+
+// Shared memory that threads have written and read goes to the asynchronous copies: their writes must not pass the threads' accesses.
+__device__ __forceinline__ void c2_release_scratch()
+{
+    fence_async_smem();
+    __syncthreads();
 }
 
 // Epilogue of a work unit whose result leaves through global memory (final bf16 rows, or fp32
@@ -835,7 +841,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
             cut = c2_rank_requests(p, reinterpret_cast<int *>(smem), order);
             request = order[unit.b];
             if (kMulti) order_here = reinterpret_cast<const uint2 *>(order)[lane];
-            __syncthreads();
+            c2_release_scratch();
         }
         c2_name_request(p, unit, request, cut, rank == 0 && threadIdx.x == 0);
     }

@@ -271,7 +271,7 @@ __device__ __forceinline__ void tc2q8_decode_body(const CUtensorMap &q_nope_map,
             uint8_t *order = smem + 4096;                 // (behind the sizes; shared memory nobody uses yet)
             cut = c2_rank_requests(p, reinterpret_cast<int *>(smem), order);
             request = order[unit.b];
-            __syncthreads();
+            c2_release_scratch();
         }
         c2_name_request(p, unit, request, cut, rank == 0 && threadIdx.x == 0);
     }
