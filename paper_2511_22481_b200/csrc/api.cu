@@ -74,9 +74,9 @@ bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) &
 // buffers to the pair's 4.  What the single-CTA kernel has is the shorter start and twice as many work units, which
 // shows up to 32 heads while two tiles per unit spread over all SMs in one wave (one request of 13 tiles of 16 heads 9.3
 // against 9.7 us on pairs, 4 x 33 11.2 against 12.0, 8 x 33 12.8 against 14.8).
-// More than 40 tiles a request (of at most 32 splits) are two and more tiles a split, at half the pair's rate: one request of 48
-// tiles 11.1 us against 10.8 on pairs, of 96 13.3 against 12.3, of 192 18.9 against 14.3; two requests of 64 tiles 11.8
-// against 13.2, of 96 13.4 against 12.7; four of 64 13.2 against 13.5.
+// From 40 tiles for one request and 80 for each of two on, pairs are faster all the same: a split (32 at most) is two and more tiles then, at half
+// the pair's rate.  One request of 48 tiles 11.1 us against 10.8 on pairs, of 96 13.3 against 12.3, of 192 18.9 against 14.3; two requests of 64
+// tiles 11.8 against 13.2, of 96 13.4 against 12.7; four of 64 13.2 against 13.5.  (Three and more reach the limit of one wave before.)
 constexpr int kSingleCtaHeads = 32, kSingleCtaUnits = 148, kSingleCtaTiles = 40;     // (units: the SMs of the device this library is for)
 bool use_pair_kernel(const omni_mla_desc_t *d)
 {
@@ -85,7 +85,7 @@ bool use_pair_kernel(const omni_mla_desc_t *d)
     return d->num_heads > kSingleCtaHeads || (long)d->batch * ((tiles + 1) / 2) > kSingleCtaUnits || tiles > (long)kSingleCtaTiles * d->batch;
 }
 
-// The 8-bit kernel takes more than 64 heads (both CTAs of its pairs have some).
+// The 8-bit entry point takes more than 64 heads, as the header says: fewer would leave half of a pair's rows and more empty.
 bool q8_shape_ok(const omni_mla_desc_t *d) { return !(d->flags & OMNI_FLAG_SIMT) && d->num_heads > kTcHeads; }
 
 // Work units one split of one request occupies in the kernel that will run.
@@ -185,7 +185,7 @@ SplitPlan split_plan(const omni_mla_desc_t *d, int sm_count, int resident_merge_
     // long again, so they are cut into as many pieces as there are pairs.  Requests of one size, and of sizes up to 1 : 1.5,
     // gain 1.08 to 1.46 times (76 x 64 units 118 -> 94 us, 80 x 128 253 -> 179, 98 x 96 192 -> 173).  The host does
     // not see the sizes.  Where they differ so much that the few run beside the longest ones the kernel takes them whole after
-    // all (c2_request_by_length_rank) and the merge kernel finds nothing to do; spread over 1 : 3 to 1 : 8 that costs up to
+    // all (c2_rank_requests) and the merge kernel finds nothing to do; spread over 1 : 3 to 1 : 8 that costs up to
     // 9 % with 88 or 98 requests (98 x 64 89 -> 98 us, 98 x 128 170 -> 176) and still gains with 76 or 80 long ones
     // (80 x 128 163 -> 152).  Below 64 units the loss is the larger part.
     const int tail = d->batch - sm_count;

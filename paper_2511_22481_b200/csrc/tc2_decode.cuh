@@ -74,7 +74,8 @@ constexpr int kScatterAhead = 1;
 // 103 us, 74 x 96 181 -> 184, 32 x 128 183 -> 195, 4 x 256 on a pair each 349 -> 381).
 // Where few pairs run, HBM is not busy and the prefetch pays up to longer units (never cut -> always, one unit to a pair): 16 and 32 pairs of
 // 48 units 41.7 -> 42.6 and 44.9 -> 46.2, 32 of 64 58.5 -> 59.4, of 96 86.3 -> 85.8; 40 pairs of 48 53.9 -> 53.8, 56 of them 63.4 -> 61.3, 74 of 64
-// 98.3 -> 95.9, 8 of 96 79.7 -> 76.7.
+// 98.3 -> 95.9, 8 of 96 79.7 -> 76.7.  The instances that merge in a cluster prefetch throughout: cut as well, 32 requests of 192 units go from
+// 128 to 121 us and 32 x 128 from 86.5 to 84.3, but the code of the test alone makes 32 x 33 27.04 -> 27.41.
 constexpr int kPrefetchAllUnits = 48, kPrefetchManyPairs = 40, kPrefetchLongUnits = 96, kPrefetchFirstUnits = 8;
 constexpr int kC2GroupPanels = 3;                        // K role: refilled in three groups of three panels
 constexpr int kC2Groups = kPanels / kC2GroupPanels;

@@ -21,9 +21,10 @@ def test_head_rows_and_tiles(heads, splits):
     check_workload(w, 0, num_splits=splits, what="H=%d S=%d" % (heads, splits))
 
 
-@pytest.mark.parametrize("batch,tiles", [(1, 40), (1, 41), (2, 81), (1, 192)])
+@pytest.mark.parametrize("batch,tiles", [(1, 40), (1, 41), (2, 80), (2, 81), (1, 192)])
 def test_either_side_of_forty_tiles_a_request(batch, tiles):
-    """The longest selection that few requests of few heads take to this kernel, and the first that pairs serve."""
+    """The longest selection that few requests of few heads take to this kernel (40 tiles for each of them), and the first that
+    pairs serve."""
     rng = np.random.default_rng(tiles)
     lists = [rng.permutation(tiles * 64), np.arange(tiles * 64 - 63)][:batch]
     pages = [tiles] * batch
