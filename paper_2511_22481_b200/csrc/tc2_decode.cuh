@@ -1177,7 +1177,7 @@ __device__ __forceinline__ void tc2_decode_body(const CUtensorMap &q_map, const 
         int round = 0;
         // Several units per pair: CTA 0 asks for the next one and hands it to both CTAs, some 3 us before the pair is free; the answer takes
         // 0.3 us.  Where the unit in hand ends in a whole page it asks once the K loads of the last tile have been requested (the earlier, the less
-        // is known of who is free first: a tile earlier 75 x 32 and one of 16 units take 60.9 us, not 58.2), behind scattered rows at once, two
+        // is known of who is free first: a tile earlier 256 x 8 units take 60.9 us, not 58.2), behind scattered rows at once, two
         // tiles earlier, since the next unit's are late without a prefetch (100 x 11 after a selection 57.1 -> 55.7).
         auto deal = [&](int round) {
             if (lane == 0) {
