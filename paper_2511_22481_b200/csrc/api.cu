@@ -215,10 +215,11 @@ bool merge_in_kernel(const omni_mla_desc_t *d)
 
 // The form of the paired-CTA kernel that serves a problem (see tc2_kernel_for): two splits merged inside a cluster, several work units per
 // pair, or one.  Several where there are more units than pairs and they are taken by size (not more than 256 requests), short, and
-// neither cut at the end only nor merged by the last CTA of a request; the units are dealt out as pairs become free.  What is saved is part of the start and the end of every
-// unit but a pair's first: 128 requests x 18 units of a rolling cache 64.7 -> 62.7 us, 128 x 18 of a list 58.4 -> 57.7, 148 x 17
-// 62.2 -> 61.2.  Where the main loop is most of a unit, its inner loop, which has to look for gaps, weighs more: 128 x 64 172 ->
-// 178, 288 units of 114 674 -> 740.
+// neither cut at the end only nor merged by the last CTA of a request; the units are dealt out as pairs become free.  What is saved is
+// part of the start and the end of every unit but a pair's first; the longer a unit, the more its main loop weighs, which takes longer in this form.
+// One unit per pair -> several, us, by the longest unit: 100 alike 16 46.8 -> 44.0, 24 63.5 -> 62.9, 32 79.1 -> 80.5, 40 95.5 -> 96.8, 48 113 -> 115; 148 alike 16
+// 58.7 -> 55.5, 24 79.4 -> 80.4, 32 102 -> 100, 40 126 -> 125, 48 143 -> 148, 64 182 -> 189; 200 from 4 units up to 32 89.4 -> 83.0, to 40 103 -> 99, to 48
+// 118 -> 116, to 64 146 -> 146.
 constexpr int kMultiUnits = 32;
 int pair_form(const omni_mla_desc_t *d, int splits, int whole, bool cluster_merge, bool fused_merge, int pairs)
 {
